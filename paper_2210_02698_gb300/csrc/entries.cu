@@ -158,11 +158,27 @@ void setup_tables(hb_ctx* c) {
   compute_self(c);
 }
 
-// The cell-integrated self terms at the handle's omega (the only
-// precomputed entry data that depends on it; the tables do not), into
-// d_self (allocated on first use).
+// The precomputed entry data that depends on omega (the tables do not): the
+// cell-integrated self terms into d_self (allocated on first use) and the
+// Hankel expansions of the dense apply.
 void compute_self(hb_ctx* c) {
   if (!c->d_self) c->d_self = dev_alloc<double2>(c->Nv);
+  // the expansions of the Hankel pair up to the largest omega tau of the
+  // tables (and a tenth of tau^2 more, for cells outside the node hull; past
+  // the rows the kernels use the asymptotic series)
+  double t2max = 0.0;
+  for (double v : c->tab[0]) t2max = std::max(t2max, v);
+  const double top = std::min(HT_CAP, c->omega * std::sqrt(1.1 * t2max) + 1.0);
+  const int nrow = top > HT_LO ? (int)std::ceil((top - HT_LO) * HT_PER) + 2 : 0;
+  dev_free(c->d_hank);
+  c->d_hank = nullptr;
+  c->hank_top = 0.0f;
+  if (nrow > 0) {
+    c->d_hank = dev_alloc<double2>((size_t)nrow * HT_ROW);
+    hankel_table_kernel<<<(nrow + 127) / 128, 128>>>(c->d_hank, nrow);
+    HB_CHECK_LAUNCH();
+    c->hank_top = (float)top;
+  }
   std::vector<double> glx, glw;
   gauss_legendre(64, glx, glw);
   // the quadrature rule is scratch: freed on the way out, also when a step throws
@@ -194,44 +210,57 @@ EntryParams entry_params(const hb_ctx* c, int transposed) {
   p.LZ = c->d_LZ;
   p.H = c->d_H[transposed ? 1 : 0];
   p.self = c->d_self;
+  p.hank = HankelTable{c->d_hank, c->hank_top};
   return p;
 }
 
 // ------------------------------------------------------- dense apply ----
-// One CTA owns 64 consecutive cells of one grid line (the outputs) and sweeps
-// the source line segments of 64 cells of its share of the source lines
-// (blockIdx.y of gridDim.y contiguous shares; all lines when gridDim.y = 1).
-// Thread t: output o = t & 63, quarter t >> 6 takes every 4th source of the
-// segment.  RC right-hand sides per pass.  FP64 throughout.  With one share
-// the CTA writes u; with several it writes its unscaled partial sums to
-// part[share][r][cell] and dense_reduce_kernel adds the shares in order.
+// One CTA owns the L <= 64 cells of one segment of a grid line (the outputs; a
+// line is cut into equal segments) and sweeps the source line segments of L
+// cells of its share of the source lines (blockIdx.y of gridDim.y contiguous
+// shares; all lines when gridDim.y = 1).  Thread t: output t mod L, group
+// t / L takes every (256 / L)-th source of the segment.  RC right-hand sides
+// per pass.  FP64 throughout.  With one share the CTA writes u; with several
+// it writes its unscaled partial sums to part[share][r][cell] and
+// dense_reduce_kernel adds the shares in order.
+//
+// Bound by the FP64 unit (2 FMAs a cycle and SM).  Per entry: 3 KI for the
+// observation contraction (the basis values in registers, the source's P
+// broadcast from shared memory), 27 for the Hankel pair (hankel_table.cuh)
+// and 4 RC.  sqrt(pi)/2 and the factors of f1 are folded into P.  Measured:
+// 64^2, one right-hand side 55 -> 3.3 ms, 144 x 100 with 16 (adjoint) 435 ->
+// 62 ms against the evaluation by recurrences with the basis in shared memory
+// (stride of 128 bytes: every lane on one bank).
 constexpr int DT = 64;
+constexpr double HB_C0 = 0.88622692545275801365;   // sqrt(pi)/2
 
-template <int RC, bool ADJ>
-__global__ void __launch_bounds__(256) dense_kernel(EntryParams p, const double2* __restrict__ s,
-                                                    double2* __restrict__ u, long long Nv, int r0,
+template <int RC, bool ADJ, int KI>
+__global__ void __launch_bounds__(256, RC <= 4 ? 2 : 1) dense_kernel(EntryParams p, const double2* __restrict__ s,
+                                                    double2* __restrict__ u, long long Nv, int L, int r0,
                                                     double scale, double2* __restrict__ part) {
   extern __shared__ double smem[];
   const int nI = p.nI;
-  double* LXo = smem;                         // DT x 16
-  double* M = LXo + DT * MAX_NI;              // 3 x 16 x 16
-  double* P = M + 3 * MAX_NI * MAX_NI;        // 3 x DT x 16
-  double2* S = reinterpret_cast<double2*>(P + 3 * DT * MAX_NI);  // DT x RC
-  double2* red = S + DT * RC;                 // 3 x DT x RC (quarter partial sums)
+  double* M = smem;                           // 3 x KI x KI
+  double* P = M + 3 * KI * KI;                // 3 x DT x KI
+  double2* S = reinterpret_cast<double2*>(P + 3 * DT * KI);  // DT x RC
+  double2* red = S + DT * RC;                 // 256 x RC (partial sums of the groups)
 
   const int t = threadIdx.x;
-  const int ntx = (p.nx + DT - 1) / DT;
+  const int ntx = (p.nx + L - 1) / L;
   const int bo = blockIdx.x / ntx;
-  const int ao0 = (blockIdx.x % ntx) * DT;
-  const int olen = min(DT, p.nx - ao0);
-  const int o = t & (DT - 1);
-  const int quarter = t >> 6;
+  const int ao0 = (blockIdx.x % ntx) * L;
+  const int olen = min(L, p.nx - ao0);
+  const int ngr = 256 / L;
+  const int o = t % L;
+  const int grp = t / L;
+  const bool active = grp < ngr && o < olen;
   const long long onat = (long long)bo * p.nx + ao0 + o;
+  const double w2 = p.omega * p.omega;
+  const double c1 = 2.0 * HB_C0 / w2;
 
-  for (int idx = t; idx < DT * nI; idx += blockDim.x) {
-    int r = idx / nI, k = idx % nI;
-    LXo[r * MAX_NI + k] = (r < olen) ? p.LX[(size_t)(ao0 + r) * nI + k] : 0.0;
-  }
+  double lxo[KI];
+#pragma unroll
+  for (int k = 0; k < KI; ++k) lxo[k] = (active && k < nI) ? p.LX[(size_t)(ao0 + o) * nI + k] : 0.0;
   double2 acc[RC];
 #pragma unroll
   for (int r = 0; r < RC; ++r) acc[r] = make_double2(0.0, 0.0);
@@ -241,47 +270,59 @@ __global__ void __launch_bounds__(256) dense_kernel(EntryParams p, const double2
   const int bq1 = (int)((long long)p.ny * (blockIdx.y + 1) / gridDim.y);
   for (int bq = bq0; bq < bq1; ++bq) {
     __syncthreads();
-    // M[q][i1][j1] = sum_i2 LZ[bo][i2] H[q][bq][(i2,i1)][j1]
-    for (int idx = t; idx < 3 * nI * nI; idx += blockDim.x) {
-      int q = idx / (nI * nI), i1 = (idx / nI) % nI, j1 = idx % nI;
-      const double* Hq = p.H + (((size_t)q * p.ny + bq) * NI) * nI;
+    // M[q][i1][j1] = sum_i2 LZ[bo][i2] H[q][bq][(i2,i1)][j1], zero past nI
+    for (int idx = t; idx < 3 * KI * KI; idx += blockDim.x) {
+      const int q = idx / (KI * KI), i1 = (idx / KI) % KI, j1 = idx % KI;
       double a = 0.0;
-      for (int i2 = 0; i2 < nI; ++i2)
-        a = fma(p.LZ[(size_t)bo * nI + i2], Hq[(size_t)(i2 * nI + i1) * nI + j1], a);
-      M[(q * MAX_NI + i1) * MAX_NI + j1] = a;
+      if (i1 < nI && j1 < nI) {
+        const double* Hq = p.H + (((size_t)q * p.ny + bq) * NI) * nI;
+        for (int i2 = 0; i2 < nI; ++i2)
+          a = fma(p.LZ[(size_t)bo * nI + i2], Hq[(size_t)(i2 * nI + i1) * nI + j1], a);
+        if (q == 1) a *= HB_C0;
+        if (q == 2) a *= c1;
+      }
+      M[idx] = a;
     }
     __syncthreads();
-    for (int aq0 = 0; aq0 < p.nx; aq0 += DT) {
-      const int qlen = min(DT, p.nx - aq0);
+    for (int aq0 = 0; aq0 < p.nx; aq0 += L) {
+      const int qlen = min(L, p.nx - aq0);
       // P[q][c][i1] = sum_j1 M[q][i1][j1] LX[a_c][j1]
-      for (int idx = t; idx < 3 * DT * nI; idx += blockDim.x) {
-        int q = idx / (DT * nI), cc = (idx / nI) % DT, i1 = idx % nI;
+      for (int idx = t; idx < 3 * qlen * KI; idx += blockDim.x) {
+        const int q = idx / (qlen * KI), cc = (idx / KI) % qlen, i1 = idx % KI;
+        const double* lx = p.LX + (size_t)(aq0 + cc) * nI;
         double a = 0.0;
-        if (cc < qlen) {
-          const double* lx = p.LX + (size_t)(aq0 + cc) * nI;
-          for (int j1 = 0; j1 < nI; ++j1) a = fma(M[(q * MAX_NI + i1) * MAX_NI + j1], lx[j1], a);
-        }
-        P[(q * DT + cc) * MAX_NI + i1] = a;
+        for (int j1 = 0; j1 < nI; ++j1) a = fma(M[(q * KI + i1) * KI + j1], lx[j1], a);
+        P[(q * DT + cc) * KI + i1] = a;
       }
-      for (int idx = t; idx < DT * RC; idx += blockDim.x) {
-        int cc = idx / RC, r = idx % RC;
-        double2 v = make_double2(0.0, 0.0);
-        if (cc < qlen) v = s[(size_t)(r0 + r) * Nv + (size_t)bq * p.nx + aq0 + cc];
-        S[cc * RC + r] = v;
+      for (int idx = t; idx < qlen * RC; idx += blockDim.x) {
+        const int cc = idx % qlen, r = idx / qlen;
+        S[cc * RC + r] = s[(size_t)(r0 + r) * Nv + (size_t)bq * p.nx + aq0 + cc];
       }
       __syncthreads();
-      if (o < olen) {
-        for (int cc = quarter; cc < qlen; cc += 4) {
+      if (active) {
+        for (int cc = grp; cc < qlen; cc += ngr) {
           double f[3];
 #pragma unroll
           for (int q = 0; q < 3; ++q) {
-            const double* pq = P + (q * DT + cc) * MAX_NI;
+            const double2* pq = reinterpret_cast<const double2*>(P + (q * DT + cc) * KI);
             double a = 0.0;
-            for (int i1 = 0; i1 < nI; ++i1) a = fma(LXo[o * MAX_NI + i1], pq[i1], a);
+#pragma unroll
+            for (int k = 0; k < KI / 2; ++k) {
+              const double2 v = pq[k];
+              a = fma(lxo[2 * k], v.x, a);
+              a = fma(lxo[2 * k + 1], v.y, a);
+            }
             f[q] = a;
           }
           const long long qnat = (long long)bq * p.nx + aq0 + cc;
-          double2 g = (qnat == onat) ? p.self[onat] : hb_green(f[0], f[1], f[2], p.omega);
+          double2 g;
+          if (qnat == onat) {
+            g = p.self[onat];
+          } else {
+            // g = i v0 H0 - i v1 x H1 (the constants are in P)
+            const HankelFG h = hankel_of_t2(p.hank, w2, f[0]);
+            g = make_double2(fma(-h.F.y, f[1], h.G.y * f[2]), fma(h.F.x, f[1], -h.G.x * f[2]));
+          }
           if (ADJ) g.y = -g.y;
 #pragma unroll
           for (int r = 0; r < RC; ++r) {
@@ -294,18 +335,18 @@ __global__ void __launch_bounds__(256) dense_kernel(EntryParams p, const double2
       __syncthreads();
     }
   }
-  // reduce the four quarters
-  if (quarter > 0) {
+  // add the groups' sums in order
+  if (active && grp > 0) {
 #pragma unroll
-    for (int r = 0; r < RC; ++r) red[((quarter - 1) * DT + o) * RC + r] = acc[r];
+    for (int r = 0; r < RC; ++r) red[((grp - 1) * L + o) * RC + r] = acc[r];
   }
   __syncthreads();
-  if (quarter == 0 && o < olen) {
+  if (active && grp == 0) {
 #pragma unroll
     for (int r = 0; r < RC; ++r) {
       double2 a = acc[r];
-      for (int qq = 0; qq < 3; ++qq) {
-        double2 b = red[(qq * DT + o) * RC + r];
+      for (int qq = 0; qq < ngr - 1; ++qq) {
+        double2 b = red[(qq * L + o) * RC + r];
         a.x += b.x;
         a.y += b.y;
       }
@@ -331,15 +372,14 @@ __global__ void dense_reduce_kernel(const double2* __restrict__ part, double2* _
   }
 }
 
-template <int RC, bool ADJ>
-static void launch_dense(const EntryParams& p, const double2* s, double2* u, long long Nv, int r0,
+template <int RC, bool ADJ, int KI>
+static void launch_dense(const EntryParams& p, const double2* s, double2* u, long long Nv, int L, int r0,
                          double scale, int nsplit, double2* part, cudaStream_t st) {
-  size_t sm = sizeof(double) * (DT * MAX_NI + 3 * MAX_NI * MAX_NI + 3 * DT * MAX_NI) +
-              sizeof(double2) * (DT * RC + 3 * DT * RC);
-  auto k = dense_kernel<RC, ADJ>;
+  size_t sm = sizeof(double) * (3 * KI * KI + 3 * DT * KI) + sizeof(double2) * (DT + 256) * RC;
+  auto k = dense_kernel<RC, ADJ, KI>;
   HB_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  int ntx = (p.nx + DT - 1) / DT;
-  k<<<dim3(ntx * p.ny, nsplit), 256, sm, st>>>(p, s, u, Nv, r0, scale, nsplit > 1 ? part : nullptr);
+  const int ntx = (p.nx + L - 1) / L;
+  k<<<dim3(ntx * p.ny, nsplit), 256, sm, st>>>(p, s, u, Nv, L, r0, scale, nsplit > 1 ? part : nullptr);
   HB_CHECK_LAUNCH();
   if (nsplit > 1) {
     const long long n = Nv * RC;
@@ -359,7 +399,9 @@ void dense_apply(hb_ctx* c, const double2* s, double2* u, int nrhs, int adjoint,
   int dev = 0, nsm = 0;
   HB_CUDA(cudaGetDevice(&dev));
   HB_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  const long long cta = (long long)((p.nx + DT - 1) / DT) * p.ny;
+  // equal segments of at most DT cells: a ragged last segment would idle threads
+  const int L = (p.nx + (p.nx + DT - 1) / DT - 1) / ((p.nx + DT - 1) / DT);
+  const long long cta = (long long)((p.nx + L - 1) / L) * p.ny;
   const int nsplit = (int)std::max<long long>(1, std::min<long long>(p.ny, (8LL * nsm + cta - 1) / cta));
   if (nsplit > 1) {
     const size_t need = (size_t)nsplit * 16 * (size_t)c->Nv;
@@ -375,10 +417,16 @@ void dense_apply(hb_ctx* c, const double2* s, double2* u, int nrhs, int adjoint,
   while (r0 < nrhs) {
     int left = nrhs - r0;
     int rc = left >= 16 ? 16 : left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
-#define HB_DENSE_CASE(R)                                                              \
-  case R:                                                                             \
-    if (adjoint) launch_dense<R, true>(p, s, u, c->Nv, r0, scale, nsplit, c->d_dense_part, st); \
-    else launch_dense<R, false>(p, s, u, c->Nv, r0, scale, nsplit, c->d_dense_part, st);       \
+#define HB_DENSE_LAUNCH(R, A, K) launch_dense<R, A, K>(p, s, u, c->Nv, L, r0, scale, nsplit, c->d_dense_part, st)
+#define HB_DENSE_CASE(R)                                              \
+  case R:                                                             \
+    if (p.nI <= 8) {                                                  \
+      if (adjoint) HB_DENSE_LAUNCH(R, true, 8);                       \
+      else HB_DENSE_LAUNCH(R, false, 8);                              \
+    } else {                                                          \
+      if (adjoint) HB_DENSE_LAUNCH(R, true, 16);                      \
+      else HB_DENSE_LAUNCH(R, false, 16);                             \
+    }                                                                 \
     break;
     switch (rc) {
       HB_DENSE_CASE(16)
@@ -388,6 +436,7 @@ void dense_apply(hb_ctx* c, const double2* s, double2* u, int nrhs, int adjoint,
       HB_DENSE_CASE(1)
     }
 #undef HB_DENSE_CASE
+#undef HB_DENSE_LAUNCH
     r0 += rc;
   }
 }

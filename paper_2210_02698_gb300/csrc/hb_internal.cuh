@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "../../include/hb.h"
+#include "hankel_table.cuh"
 
 namespace hb {
 
@@ -105,6 +106,7 @@ struct EntryParams {
   const double* LZ;      // ny x nI   l_k(z_b)
   const double* H;       // 3 x ny x NI x nI  (see entries.cu)
   const double2* self;   // Nv self terms K_ii
+  HankelTable hank;      // expansions of H0, x H1 (dense apply)
 };
 
 // ------------------------------------------------------ butterfly plan ----
@@ -247,6 +249,8 @@ struct hb_ctx {
   double* d_H[2] = {nullptr, nullptr};
   double* d_ncell = nullptr;
   double2* d_self = nullptr;
+  double2* d_hank = nullptr;   // Hankel expansions (hankel_table.cuh) of x < hank_top
+  float hank_top = 0.0f;
 
   // cluster tree
   int Lv = 0;
