@@ -5,8 +5,8 @@
 //   steps of small dense products over all butterflies      (build.cu plans)
 //   u  = y scattered back to natural order
 //
-// FP64 path: complex128 factors and vectors, one CTA per task, plain FP64
-// FMAs (the baseline).  Mixed path (HB_MIXED_BF16X3): split-BF16 factors and
+// FP64 path: complex128 factors and vectors, the step tasks' products on the
+// FP16 tensor cores by integer digits, as accurate as FP64 FMAs.  Mixed path (HB_MIXED_BF16X3): split-BF16 factors and
 // vectors in the MMA-fragment layout of bf_mma.cu, up to 32 right-hand
 // sides per pass.
 #include <cuda_runtime.h>
@@ -17,105 +17,323 @@
 #include <vector>
 
 #include "hb_internal.cuh"
+#include "split_fixed.cuh"
 
 namespace hb {
 
-__global__ void f64_to_f32_kernel(const double2* __restrict__ a, float2* __restrict__ b, long long n) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    b[i] = make_float2((float)a[i].x, (float)a[i].y);
-}
-
-void convert_f64_f32(const double2* a, float2* b, long long n, cudaStream_t st) {
-  if (n <= 0) return;
-  f64_to_f32_kernel<<<1216, 256, 0, st>>>(a, b, n);
-  HB_CHECK_LAUNCH();
-}
-
-template <class C>
-struct Real;
-template <>
-struct Real<double2> {
-  using T = double;
-  static __device__ __forceinline__ double2 make(double x, double y) { return make_double2(x, y); }
-};
-template <>
-struct Real<float2> {
-  using T = float;
-  static __device__ __forceinline__ float2 make(float x, float y) { return make_float2(x, y); }
-};
-
 // x[p][r] = scale * s[r*Nv + perm[p]]   (column-major natural -> row-major tree order)
-// for tree positions p in [lo, hi); 0 elsewhere (a shard's share of the input)
-template <class C>
-__global__ void gather_kernel(const double2* __restrict__ s, const long long* __restrict__ perm, C* __restrict__ x,
-                              long long Nv, int R, double scale, long long lo, long long hi) {
-  long long total = Nv * R;
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (long long)gridDim.x * blockDim.x) {
-    long long p = idx / R;
-    int r = (int)(idx % R);
+// for tree positions p in [lo, hi); 0 elsewhere (a shard's share of the
+// input).  blockDim.x = R rounded up to a power of two: lane -> right-hand side.
+__global__ void gather_kernel(const double2* __restrict__ s, const long long* __restrict__ perm,
+                              double2* __restrict__ x, long long Nv, int R, double scale, long long lo, long long hi) {
+  const int r = threadIdx.x;
+  if (r >= R) return;
+  for (long long p = (long long)blockIdx.x * blockDim.y + threadIdx.y; p < Nv; p += (long long)gridDim.x * blockDim.y) {
     const double2 v = (p >= lo && p < hi) ? s[(size_t)r * Nv + perm[p]] : make_double2(0.0, 0.0);
-    x[idx] = Real<C>::make((typename Real<C>::T)(v.x * scale), (typename Real<C>::T)(v.y * scale));
+    x[p * R + r] = make_double2(v.x * scale, v.y * scale);
   }
 }
 
 // u[r*Nv + perm[p]] = y[p][r] for tree positions p in [lo, hi)
-template <class C>
-__global__ void scatter_kernel(const C* __restrict__ y, const long long* __restrict__ perm, double2* __restrict__ u,
-                               long long Nv, int R, long long lo, long long hi) {
-  long long total = (hi - lo) * R;
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (long long)gridDim.x * blockDim.x) {
-    long long p = lo + idx / R;
-    int r = (int)(idx % R);
-    C v = y[(size_t)p * R + r];
-    u[(size_t)r * Nv + perm[p]] = make_double2((double)v.x, (double)v.y);
-  }
+__global__ void scatter_kernel(const double2* __restrict__ y, const long long* __restrict__ perm,
+                               double2* __restrict__ u, long long Nv, int R, long long lo, long long hi) {
+  const int r = threadIdx.x;
+  if (r >= R) return;
+  for (long long p = lo + (long long)blockIdx.x * blockDim.y + threadIdx.y; p < hi;
+       p += (long long)gridDim.x * blockDim.y)
+    u[(size_t)r * Nv + perm[p]] = y[(size_t)p * R + r];
 }
 
-// One CTA per task; thread -> (output row, right-hand side), rows fastest.
-template <class C>
-__global__ void __launch_bounds__(128) step_kernel(const Task* __restrict__ tasks, const C* __restrict__ F,
-                                                   C* __restrict__ x, C* __restrict__ y, C* __restrict__ xh,
-                                                   int R) {
-  using T = typename Real<C>::T;
-  const Task tk = tasks[blockIdx.x];
-  C* bufs[3] = {x, y, xh};
-  C* out = bufs[tk.y_buf] + (size_t)tk.y_off * R;
-  const int total = tk.r_out * R;
+// ------------------------------------------------------- step tasks ----
+// Y = op(F) X of one task on the FP16 tensor cores by integer digits
+// (split_fixed.cuh), in the orientation of the mixed apply: the MMA's M is
+// right-hand sides, N outputs, K = 2 x 8 inputs with real and imaginary
+// parts interleaved; D_r takes A rows (Re X, -Im X), D_i (Im X, Re X).  Up to
+// eight right-hand sides (HALF) both go into one MMA, rows 0-7 and 8-15.
+//
+// A CTA of 8 warps takes up to 64 outputs (8 n-tiles, blockIdx.y of them) of
+// one task.  It scales X per right-hand side and F per task (tk.fe, found
+// when the plan is made), splits X into digit fragments in shared memory,
+// KC k-steps at a time, and every warp streams its n-tile's F straight from
+// global memory into registers, one k-step ahead, splitting it there (each
+// F value is used by one warp only).  With fewer than 8 n-tiles the k-steps
+// are dealt over 2, 4 or 8 warps and the integer sums added: the result does
+// not depend on the split.  The split is a function of the task alone, so a
+// shard's sums equal the whole apply's.
+//
+// Bound by instruction issue: 42 (21) MMAs and about 150 integer instructions
+// a warp per 8 outputs x 8 inputs, as much again to split the task's X where
+// its rank is near 16, and the epilogue, against 1024 x 4 FP64 FMAs for 16
+// right-hand sides (2048 cycles of an SM's FP64 unit).  Measured (192^2, 16
+// right-hand sides): 3.67 -> 1.92 ms against one FP64 FMA loop per output;
+// 120 x 88 adjoint with 5: 601 -> 251 us.
+constexpr int TASK_THREADS = 256;
+constexpr int TASK_WARPS = TASK_THREADS / 32;
+constexpr int TASK_KC = 16;              // k-steps of X held at a time
+constexpr uint32_t SPLIT_IM_SIGN = 0x80000000u;
+
+// Rows [row0, row1) of a task with plain FP64 FMAs: what a task does whose
+// inputs are not all finite (thread -> (row, right-hand side), rows fastest).
+__device__ __noinline__ void task_plain(const Task* __restrict__ task, const double2* __restrict__ F, double2* x, double2* y,
+                                        double2* xh, int R, int row0, int row1) {
+  const Task& tk = *task;
+  double2* bufs[3] = {x, y, xh};
+  double2* out = bufs[tk.y_buf] + (size_t)tk.y_off * R;
+  const int rows = row1 - row0, total = rows * R;
   for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
-    const int row = idx % tk.r_out, rr = idx / tk.r_out;
-    T ar = 0, ai = 0;
+    const int row = row0 + idx % rows, rr = idx / rows;
+    double ar = 0, ai = 0;
     for (int t = 0; t < tk.nterm; ++t) {
-      const C* f = F + tk.f_off[t];
-      const C* xin = bufs[tk.x_buf] + (size_t)tk.x_off[t] * R + rr;
+      const double2* f = F + tk.f_off[t];
+      const double2* xin = bufs[tk.x_buf] + (size_t)tk.x_off[t] * R + rr;
       const int rin = tk.r_in[t];
       if (!tk.conj_t) {
         for (int k = 0; k < rin; ++k) {
-          const C a = f[(size_t)k * tk.r_out + row];
-          const C v = xin[(size_t)k * R];
+          const double2 a = f[(size_t)k * tk.r_out + row];
+          const double2 v = xin[(size_t)k * R];
           ar = fma(a.x, v.x, fma(-a.y, v.y, ar));
           ai = fma(a.x, v.y, fma(a.y, v.x, ai));
         }
       } else {
-        const C* fr = f + (size_t)row * rin;
+        const double2* fr = f + (size_t)row * rin;
         for (int k = 0; k < rin; ++k) {
-          const C a = fr[k];
-          const C v = xin[(size_t)k * R];
+          const double2 a = fr[k];
+          const double2 v = xin[(size_t)k * R];
           ar = fma(a.x, v.x, fma(a.y, v.y, ar));     // conj(a) v
           ai = fma(a.x, v.y, fma(-a.y, v.x, ai));
         }
       }
     }
-    C* o = out + (size_t)row * R + rr;
+    double2* o = out + (size_t)row * R + rr;
     if (tk.accumulate) {
-      C prev = *o;
+      const double2 prev = *o;
       ar += prev.x;
       ai += prev.y;
     }
-    *o = Real<C>::make(ar, ai);
+    *o = make_double2(ar, ai);
   }
+}
+
+template <bool HALF>
+__global__ void __launch_bounds__(TASK_THREADS, HALF ? 3 : 2)
+    task_kernel(const Task* __restrict__ tasks, const double2* __restrict__ F, double2* x, double2* y, double2* xh,
+                int R) {
+  constexpr int NR = HALF ? 8 : 16;        // right-hand sides of the MMA rows
+  constexpr int NE = HALF ? 4 : 8;         // accumulator elements per lane and digit diagonal
+  constexpr int XW = HALF ? 2 : 4;         // X fragment words per lane
+  extern __shared__ __align__(16) uint32_t xs[];   // [k-step][digit][lane][XW]
+  __shared__ int s_ex[16];
+  __shared__ int s_bad;
+  const Task tk = tasks[blockIdx.x];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+  const int tile0 = 8 * blockIdx.y;
+  const int ntile = min(8, (tk.r_out + 7) / 8 - tile0);
+  if (ntile <= 0) return;
+  const double2* xin = tk.x_buf == 0 ? x : tk.x_buf == 1 ? y : xh;
+  const int rin0 = tk.r_in[0], rin1 = tk.nterm > 1 ? tk.r_in[1] : 0;
+  const int ks0 = (rin0 + 7) / 8, ks = ks0 + (rin1 + 7) / 8;
+
+  // the exponent of every right-hand side over the task's inputs
+  if (tid < 16) s_ex[tid] = 1;
+  if (tid == 0) s_bad = (tk.fe == SPLIT_NONFINITE) ? 1 : 0;
+  __syncthreads();
+  const int xr = tid & (NR - 1), xk = tid / NR;
+  constexpr int XK = TASK_THREADS / NR;
+  if (xr < R) {
+    int e = 1;
+    for (int k = xk; k < rin0; k += XK) e = max(e, block_exponent(xin[(tk.x_off[0] + k) * R + xr]));
+    for (int k = xk; k < rin1; k += XK) e = max(e, block_exponent(xin[(tk.x_off[1] + k) * R + xr]));
+    atomicMax(&s_ex[xr], e);
+    if (e == SPLIT_NONFINITE) s_bad = 1;
+  }
+  __syncthreads();
+  if (s_bad) {
+    task_plain(tasks + blockIdx.x, F, x, y, xh, R, 8 * tile0, min(tk.r_out, 8 * (tile0 + 8)));
+    return;
+  }
+
+  // warp -> n-tile and share of the k-steps
+  const int kw = ntile > 4 ? 1 : ntile > 2 ? 2 : ntile > 1 ? 4 : 8;
+  const int wt = warp % (TASK_WARPS / kw), kp = warp / (TASK_WARPS / kw);
+  const bool work = wt < ntile;
+  const int row = 8 * (tile0 + wt) + g;
+  const bool rok = work && row < tk.r_out;
+
+  // F values (row, k = 2t) and (row, 2t + 1) of k-step q
+  auto load_f = [&](int q, double2& f0, double2& f1) {
+    f0 = f1 = make_double2(0.0, 0.0);
+    if (!rok || q >= ks) return;
+    const int term = q >= ks0, rin = term ? rin1 : rin0;
+    const int k = 8 * (term ? q - ks0 : q) + 2 * t;
+    const double2* f = F + (term ? tk.f_off[1] : tk.f_off[0]);
+    if (!tk.conj_t) {
+      if (k < rin) f0 = __ldcs(f + (size_t)k * tk.r_out + row);
+      if (k + 1 < rin) f1 = __ldcs(f + (size_t)(k + 1) * tk.r_out + row);
+    } else {
+      const double2* fr = f + (size_t)row * rin + k;
+      if (k < rin) f0 = __ldcs(fr);
+      if (k + 1 < rin) f1 = __ldcs(fr + 1);
+      f0.y = -f0.y;
+      f1.y = -f1.y;
+    }
+  };
+
+  float acc[SPLIT_ACC][NE];
+  long long hi[NE], lo[NE];
+#pragma unroll
+  for (int e = 0; e < NE; ++e) {
+    hi[e] = lo[e] = 0;
+#pragma unroll
+    for (int d = 0; d < SPLIT_ACC; ++d) acc[d][e] = 0.f;
+  }
+  const int myex = s_ex[xr];
+  double2 f0, f1;
+  load_f(kp, f0, f1);
+  for (int c0 = 0; c0 < ks; c0 += TASK_KC) {
+    const int c1 = min(ks, c0 + TASK_KC);
+    if (c0) __syncthreads();
+    // X of k-steps [c0, c1) into digit fragments: word j of lane (g, t) is
+    // (right-hand side g + 8 (j & 1), input 2t + (j >> 1)); HALF: (g, 2t + j)
+    for (int k = 8 * c0 + xk; k < 8 * c1; k += XK) {
+      const int q = k >> 3, kk = k & 7;
+      const int term = q >= ks0, kin = term ? k - 8 * ks0 : k;
+      double2 v = make_double2(0.0, 0.0);
+      if (xr < R && kin < (term ? rin1 : rin0)) v = xin[((term ? tk.x_off[1] : tk.x_off[0]) + kin) * R + xr];
+      uint32_t w[SPLIT_DIGITS];
+      split_pair(v.x, v.y, myex, w);
+      const int j = HALF ? (kk & 1) : 2 * (kk & 1) + (xr >> 3);
+      uint32_t* dst = xs + (((q - c0) * SPLIT_DIGITS) * 32 + (xr & 7) * 4 + (kk >> 1)) * XW + j;
+#pragma unroll
+      for (int s = 0; s < SPLIT_DIGITS; ++s) dst[s * 32 * XW] = w[s];
+    }
+    __syncthreads();
+    if (work) {
+      int since = 0;
+      for (int q = c0 + (kp - c0 % kw + kw) % kw; q < c1; q += kw) {
+        const double2 a0 = f0, a1 = f1;
+        load_f(q + kw, f0, f1);
+        uint32_t b0[SPLIT_DIGITS], b1[SPLIT_DIGITS];
+        split_pair(a0.x, a0.y, tk.fe, b0);
+        split_pair(a1.x, a1.y, tk.fe, b1);
+        const uint32_t* xq = xs + ((q - c0) * SPLIT_DIGITS * 32 + lane) * XW;
+#pragma unroll
+        for (int i = 0; i < SPLIT_DIGITS; ++i) {
+          if constexpr (HALF) {
+            const uint2 w = *reinterpret_cast<const uint2*>(xq + i * 32 * XW);
+            const uint32_t a[4] = {w.x ^ SPLIT_IM_SIGN, __byte_perm(w.x, 0, 0x1032), w.y ^ SPLIT_IM_SIGN,
+                                   __byte_perm(w.y, 0, 0x1032)};
+#pragma unroll
+            for (int j = 0; i + j < SPLIT_DIGITS; ++j)
+              mma_f16(acc[i == 2 && j == 0 ? 6 : i + j], a[0], a[1], a[2], a[3], b0[j], b1[j]);
+          } else {
+            const uint4 w = *reinterpret_cast<const uint4*>(xq + i * 32 * XW);
+            const uint32_t r[4] = {w.x ^ SPLIT_IM_SIGN, w.y ^ SPLIT_IM_SIGN, w.z ^ SPLIT_IM_SIGN, w.w ^ SPLIT_IM_SIGN};
+            const uint32_t m[4] = {__byte_perm(w.x, 0, 0x1032), __byte_perm(w.y, 0, 0x1032),
+                                   __byte_perm(w.z, 0, 0x1032), __byte_perm(w.w, 0, 0x1032)};
+#pragma unroll
+            for (int j = 0; i + j < SPLIT_DIGITS; ++j) {
+              const int d = i == 2 && j == 0 ? 6 : i + j;
+              mma_f16(acc[d], r[0], r[1], r[2], r[3], b0[j], b1[j]);
+              mma_f16(acc[d] + 4, m[0], m[1], m[2], m[3], b0[j], b1[j]);
+            }
+          }
+        }
+        if (++since == 2 || q + kw >= c1) {
+          since = 0;
+#pragma unroll
+          for (int e = 0; e < NE; ++e)
+            split_flush(acc[0][e], acc[1][e], acc[2][e], acc[3][e], acc[4][e], acc[5][e], acc[6][e], hi[e], lo[e]);
+        }
+      }
+    }
+  }
+  // add the shares of the k-steps
+  if (kw > 1) {
+    longlong2* red = reinterpret_cast<longlong2*>(xs);   // [kp - 1][n-tile][element][lane]
+    __syncthreads();
+    if (work && kp > 0)
+#pragma unroll
+      for (int e = 0; e < NE; ++e) red[(((kp - 1) * ntile + wt) * NE + e) * 32 + lane] = make_longlong2(hi[e], lo[e]);
+    __syncthreads();
+    if (!work || kp > 0) return;
+    for (int p = 0; p < kw - 1; ++p)
+#pragma unroll
+      for (int e = 0; e < NE; ++e) {
+        const longlong2 v = red[((p * ntile + wt) * NE + e) * 32 + lane];
+        hi[e] += v.x;
+        lo[e] += v.y;
+      }
+  }
+  if (!work) return;
+  double2* out = (tk.y_buf == 0 ? x : tk.y_buf == 1 ? y : xh) + (size_t)tk.y_off * R;
+  // element e of D: right-hand side g + 8 (e >> 1), output 2t + (e & 1); HALF:
+  // elements 0, 1 are D_r and 2, 3 D_i of right-hand side g
+#pragma unroll
+  for (int e = 0; e < NE / 2; ++e) {
+    const int rr = HALF ? g : g + 8 * (e >> 1);
+    const int ro = 8 * (tile0 + wt) + 2 * t + (e & 1);
+    if (rr >= R || ro >= tk.r_out) continue;
+    const int ex = tk.fe + s_ex[rr] - 2 * SPLIT_EXP_BIAS;
+    const int ei = HALF ? e + 2 : e + 4;
+    double2 v = make_double2(fixed_to_double(hi[e], lo[e], ex), fixed_to_double(hi[ei], lo[ei], ex));
+    double2* o = out + (size_t)ro * R + rr;
+    if (tk.accumulate) {
+      const double2 prev = *o;
+      v.x += prev.x;
+      v.y += prev.y;
+    }
+    *o = v;
+  }
+}
+
+// tasks[i].fe = the largest exponent of task i's factor blocks, one warp each
+__global__ void __launch_bounds__(256) task_exponent_kernel(Task* __restrict__ tasks, int n,
+                                                            const double2* __restrict__ F) {
+  const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (i >= n) return;
+  int e = 1;
+  for (int t = 0; t < tasks[i].nterm; ++t) {
+    const long long cnt = (long long)tasks[i].r_out * tasks[i].r_in[t];
+    const double2* f = F + tasks[i].f_off[t];
+    for (long long k = lane; k < cnt; k += 32) e = max(e, block_exponent(f[k]));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+  if (lane == 0) tasks[i].fe = (unsigned short)e;
+}
+
+void task_exponents(Task* d_tasks, int n, const double2* F, cudaStream_t st) {
+  if (n <= 0) return;
+  task_exponent_kernel<<<(n + 7) / 8, 256, 0, st>>>(d_tasks, n, F);
+  HB_CHECK_LAUNCH();
+}
+
+StepShape step_shape(const Task* tasks, int n) {
+  StepShape s{0, 0};
+  for (int i = 0; i < n; ++i) {
+    const Task& t = tasks[i];
+    s.max_out = std::max(s.max_out, t.r_out);
+    s.max_ks = std::max(s.max_ks, (t.r_in[0] + 7) / 8 + (t.nterm > 1 ? (t.r_in[1] + 7) / 8 : 0));
+  }
+  return s;
+}
+
+// One launch of FP64 step tasks, R <= 16 right-hand sides.
+void run_tasks_fp64(const Task* d_tasks, int n, const StepShape& sh, const double2* F, double2* x, double2* y,
+                    double2* xh, int R, cudaStream_t st) {
+  if (n <= 0) return;
+  const dim3 grid((unsigned)n, (unsigned)std::max(1, (sh.max_out + 63) / 64));
+  const size_t frag = (size_t)std::min(TASK_KC, std::max(1, sh.max_ks)) * SPLIT_DIGITS * 32 * 4;
+  const size_t red = (size_t)7 * 32 * sizeof(longlong2);   // the k-step shares of one CTA: at most 7 n-tile shares
+  if (R <= 8) {
+    const size_t smem = std::max(frag * 2, red * 4);
+    task_kernel<true><<<grid, TASK_THREADS, smem, st>>>(d_tasks, F, x, y, xh, R);
+  } else {
+    const size_t smem = std::max(frag * 4, red * 8);
+    HB_CUDA(cudaFuncSetAttribute(task_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 56 << 10));
+    task_kernel<false><<<grid, TASK_THREADS, smem, st>>>(d_tasks, F, x, y, xh, R);
+  }
+  HB_CHECK_LAUNCH();
 }
 
 namespace {
@@ -210,29 +428,30 @@ void ensure_scratch(hb_ctx* c, int nrhs, bool fp64) {
 
 }  // namespace
 
-// One launch of FP64 step tasks (one CTA each), for other operators'
-// butterflies (curve_bf.cu).
-void run_tasks_fp64(const Task* d_tasks, int n, const double2* F, double2* x, double2* y, double2* xh, int R,
-                    cudaStream_t st) {
-  if (n <= 0) return;
-  step_kernel<double2><<<n, 128, 0, st>>>(d_tasks, F, x, y, xh, R);
-  HB_CHECK_LAUNCH();
-}
-
 namespace {
 
-template <class C>
-void run_steps(hb_ctx* c, const C* F, int nrhs, int dir, cudaStream_t st, TimerScope& ts) {
+void run_steps(hb_ctx* c, const double2* F, int nrhs, int dir, cudaStream_t st, TimerScope& ts) {
   const std::vector<int>& sb = c->step_begin[dir];
   for (size_t s = 0; s + 1 < sb.size(); ++s) {
-    int n = sb[s + 1] - sb[s];
+    const int n = sb[s + 1] - sb[s];
     if (n == 0) continue;
     ts.begin(dir ? "bf_step_adjoint" : "bf_step");
-    step_kernel<C><<<n, 128, 0, st>>>(c->d_tasks[dir] + sb[s], F, (C*)c->d_x, (C*)c->d_y, (C*)c->d_xh, nrhs);
-    HB_CHECK_LAUNCH();
+    run_tasks_fp64(c->d_tasks[dir] + sb[s], n, c->step_shapes[dir][s], F, (double2*)c->d_x, (double2*)c->d_y,
+                   (double2*)c->d_xh, nrhs, st);
     ts.end();
   }
 }
+
+// launch shape of the gather / scatter kernels: lanes over the right-hand sides
+struct VecGrid {
+  dim3 grid, block;
+  VecGrid(long long rows, int R) {
+    int rp = 1;
+    while (rp < R) rp *= 2;
+    block = dim3((unsigned)rp, (unsigned)(256 / rp));
+    grid = dim3((unsigned)std::max<long long>(1, std::min<long long>((rows + block.y - 1) / block.y, 152LL * 16)));
+  }
+};
 
 }  // namespace
 
@@ -252,16 +471,15 @@ void apply_bf(hb_ctx* c, const double2* s, double2* u, int nrhs, int adjoint, in
     const int R = std::min(chunk, nrhs - r0);
     const double2* sc = s + (size_t)r0 * c->Nv;
     double2* uc = u + (size_t)r0 * c->Nv;
-    const long long total = c->Nv * R;
-    const int grid = (int)std::min<long long>((total + 255) / 256, 152LL * 16);
+    const VecGrid vg(c->Nv, R);
     if (precision == HB_FP64) {
       ts.begin("gather");
-      gather_kernel<double2><<<grid, 256, 0, st>>>(sc, c->d_perm, (double2*)c->d_x, c->Nv, R, scale, 0, c->Nv);
+      gather_kernel<<<vg.grid, vg.block, 0, st>>>(sc, c->d_perm, (double2*)c->d_x, c->Nv, R, scale, 0, c->Nv);
       HB_CHECK_LAUNCH();
       ts.end();
-      run_steps<double2>(c, c->d_f64, R, adjoint, st, ts);
+      run_steps(c, c->d_f64, R, adjoint, st, ts);
       ts.begin("scatter");
-      scatter_kernel<double2><<<grid, 256, 0, st>>>((double2*)c->d_y, c->d_perm, uc, c->Nv, R, 0, c->Nv);
+      scatter_kernel<<<vg.grid, vg.block, 0, st>>>((double2*)c->d_y, c->d_perm, uc, c->Nv, R, 0, c->Nv);
       HB_CHECK_LAUNCH();
       ts.end();
     } else {
@@ -297,6 +515,7 @@ void shard_rows(const hb_ctx* c, int nranks, int rank, long long* lo, long long*
 namespace {
 struct ShardSteps {
   std::vector<int> begin;
+  std::vector<StepShape> shapes;
   Task* d_tasks = nullptr;
 };
 }  // namespace
@@ -318,6 +537,8 @@ static ShardSteps& shard_steps(hb_ctx* c, int dir, long long lo, long long hi) {
     }
   }
   S->begin.push_back((int)keep.size());
+  for (size_t q = 0; q + 1 < S->begin.size(); ++q)
+    S->shapes.push_back(step_shape(keep.data() + S->begin[q], S->begin[q + 1] - S->begin[q]));
   try {
     S->d_tasks = upload(keep);
   } catch (...) {
@@ -371,10 +592,9 @@ void apply_bf_shard(hb_ctx* c, const double2* s, double2* u, int nrhs, int adjoi
     const int R = std::min(chunk, nrhs - r0);
     const double2* sc = s + (size_t)r0 * c->Nv;
     double2* uc = u + (size_t)r0 * c->Nv;
-    const long long total = c->Nv * R;
-    const int grid = (int)std::min<long long>((total + 255) / 256, 152LL * 16);
+    const VecGrid vg(c->Nv, R);
     if (precision == HB_FP64) {
-      gather_kernel<double2><<<grid, 256, 0, st>>>(sc, c->d_perm, (double2*)c->d_x, c->Nv, R, scale, glo, ghi);
+      gather_kernel<<<vg.grid, vg.block, 0, st>>>(sc, c->d_perm, (double2*)c->d_x, c->Nv, R, scale, glo, ghi);
       HB_CHECK_LAUNCH();
       if (adjoint) {
         HB_CUDA(cudaMemsetAsync(c->d_y, 0, sizeof(double2) * (size_t)c->Nv * R, st));
@@ -384,12 +604,11 @@ void apply_bf_shard(hb_ctx* c, const double2* s, double2* u, int nrhs, int adjoi
       for (size_t q = 0; q + 1 < S.begin.size(); ++q) {
         const int n = S.begin[q + 1] - S.begin[q];
         if (n == 0) continue;
-        step_kernel<double2><<<n, 128, 0, st>>>(S.d_tasks + S.begin[q], c->d_f64, (double2*)c->d_x,
-                                               (double2*)c->d_y, (double2*)c->d_xh, R);
-        HB_CHECK_LAUNCH();
+        run_tasks_fp64(S.d_tasks + S.begin[q], n, S.shapes[q], c->d_f64, (double2*)c->d_x, (double2*)c->d_y,
+                       (double2*)c->d_xh, R, st);
       }
-      const int g2 = (int)std::max<long long>(1, std::min<long long>(((shi - slo) * R + 255) / 256, 152LL * 16));
-      scatter_kernel<double2><<<g2, 256, 0, st>>>((double2*)c->d_y, c->d_perm, uc, c->Nv, R, slo, shi);
+      const VecGrid vs(shi - slo, R);
+      scatter_kernel<<<vs.grid, vs.block, 0, st>>>((double2*)c->d_y, c->d_perm, uc, c->Nv, R, slo, shi);
       HB_CHECK_LAUNCH();
     } else {
       flow_launch_shard(c->flow_plan[adjoint], c->d_nat[adjoint], sc, scale, c->d_mx, c->d_mxh, c->xh_tiles, uc,

@@ -539,7 +539,15 @@ static void make_plans(hb_ctx* c, std::vector<Butterfly>& bfs, const std::vector
     }
     begins.push_back((int)c->tasks_h[dir].size());
     c->step_begin[dir] = begins;
+    c->step_shapes[dir].clear();
+    for (size_t q = 0; q + 1 < begins.size(); ++q)
+      c->step_shapes[dir].push_back(step_shape(c->tasks_h[dir].data() + begins[q], begins[q + 1] - begins[q]));
+    // the factor exponents are found on the device and kept on both sides (a
+    // shard uploads a part of the host list)
     c->d_tasks[dir] = upload(c->tasks_h[dir]);
+    task_exponents(c->d_tasks[dir], (int)c->tasks_h[dir].size(), c->d_f64, 0);
+    HB_CUDA(cudaMemcpy(c->tasks_h[dir].data(), c->d_tasks[dir], sizeof(Task) * c->tasks_h[dir].size(),
+                       cudaMemcpyDeviceToHost));
   }
 
   // native arenas and plans of the mixed apply

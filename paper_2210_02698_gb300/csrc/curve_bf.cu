@@ -45,6 +45,7 @@ struct CurveBfly {
   int L = 0;
   long long nrows = 0, ncols = 0, xh_rows = 0, entries = 0;
   std::vector<int> step_begin;
+  std::vector<StepShape> shapes;   // per step
   std::vector<int> max_rank;    // per butterfly level
   Task* d_tasks = nullptr;
   double2* d_F = nullptr;
@@ -387,7 +388,9 @@ CurveBfly* build_bfly(const hb_ctx* c, const BfSide& R, const BfSide& C, int L) 
     B->entries = fbase;
     B->xh_rows = xh;
     B->step_begin = sb;
+    for (size_t q = 0; q + 1 < sb.size(); ++q) B->shapes.push_back(step_shape(tasks.data() + sb[q], sb[q + 1] - sb[q]));
     B->d_tasks = upload(tasks);
+    task_exponents(B->d_tasks, (int)tasks.size(), B->d_F, 0);
     B->d_rperm = upload(R.perm);
     B->d_cperm = upload(C.perm);
     HB_CUDA(cudaDeviceSynchronize());
@@ -462,24 +465,30 @@ void curve_bf_apply(hb_ctx* c, int which, const double2* x_nat, long long ldx, d
                     long long ldy, int accumulate, int nrhs, cudaStream_t st) {
   CurveBfly* B = static_cast<CurveBfly*>(c->curve_bf[which]);
   if (!B) throw Error{HB_ERR_STATE, "no compressed curve operator"};
-  if (B->cap < nrhs) {
+  // passes of 16 right-hand sides (what one step task takes)
+  const int chunk = std::min(nrhs, 16);
+  if (B->cap < chunk) {
     for (void* p : {(void*)B->d_x, (void*)B->d_y, (void*)B->d_xh}) dev_free(p);
     B->d_x = B->d_y = B->d_xh = nullptr;
     B->cap = 0;
-    B->d_x = dev_alloc<double2>((size_t)B->ncols * nrhs);
-    B->d_y = dev_alloc<double2>((size_t)B->nrows * nrhs);
-    B->d_xh = dev_alloc<double2>((size_t)std::max<long long>(B->xh_rows, 1) * nrhs);
-    B->cap = nrhs;
+    B->d_x = dev_alloc<double2>((size_t)B->ncols * chunk);
+    B->d_y = dev_alloc<double2>((size_t)B->nrows * chunk);
+    B->d_xh = dev_alloc<double2>((size_t)std::max<long long>(B->xh_rows, 1) * chunk);
+    B->cap = chunk;
     HB_CUDA(cudaDeviceSynchronize());
   }
-  gather_tree_kernel<<<grid_for(B->ncols * nrhs), 256, 0, st>>>(x_nat, ldx, B->d_cperm, B->ncols, nrhs, scale, B->d_x);
-  HB_CHECK_LAUNCH();
-  for (size_t s = 0; s + 1 < B->step_begin.size(); ++s)
-    run_tasks_fp64(B->d_tasks + B->step_begin[s], B->step_begin[s + 1] - B->step_begin[s], B->d_F, B->d_x, B->d_y,
-                   B->d_xh, nrhs, st);
-  scatter_tree_kernel<<<grid_for(B->nrows * nrhs), 256, 0, st>>>(B->d_y, B->d_rperm, B->nrows, nrhs, y_nat, ldy,
-                                                                 accumulate);
-  HB_CHECK_LAUNCH();
+  for (int r0 = 0; r0 < nrhs; r0 += chunk) {
+    const int R = std::min(chunk, nrhs - r0);
+    gather_tree_kernel<<<grid_for(B->ncols * R), 256, 0, st>>>(x_nat + (size_t)r0 * ldx, ldx, B->d_cperm, B->ncols, R,
+                                                               scale, B->d_x);
+    HB_CHECK_LAUNCH();
+    for (size_t s = 0; s + 1 < B->step_begin.size(); ++s)
+      run_tasks_fp64(B->d_tasks + B->step_begin[s], B->step_begin[s + 1] - B->step_begin[s], B->shapes[s], B->d_F,
+                     B->d_x, B->d_y, B->d_xh, R, st);
+    scatter_tree_kernel<<<grid_for(B->nrows * R), 256, 0, st>>>(B->d_y, B->d_rperm, B->nrows, R,
+                                                               y_nat + (size_t)r0 * ldy, ldy, accumulate);
+    HB_CHECK_LAUNCH();
+  }
 }
 
 void curve_bf_info(const hb_ctx* c, int which, int* levels, int* max_rank, long long* entries) {

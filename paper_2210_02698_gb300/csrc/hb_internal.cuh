@@ -123,7 +123,13 @@ struct Task {
   int r_out;
   int r_in[2];
   unsigned char nterm, x_buf, y_buf, accumulate;
-  unsigned char conj_t, kind, pad0, pad1;
+  unsigned char conj_t, kind;
+  unsigned short fe;        // largest biased exponent of its factor blocks (task_exponents)
+};
+// The largest task of a step: outputs, and k-steps of 8 inputs (each term's
+// inputs rounded up).
+struct StepShape {
+  int max_out, max_ks;
 };
 
 // Native (MMA-fragment) layout of the mixed apply (bf_mma.cu).  A factor
@@ -279,6 +285,7 @@ struct hb_ctx {
   long long* d_pperm = nullptr;       // padded row -> natural index (-1: padding)
   // apply plans: steps[0] forward, steps[1] adjoint; each step = task range
   std::vector<int> step_begin[2];
+  std::vector<hb::StepShape> step_shapes[2];
   std::vector<hb::Task> tasks_h[2];
   std::vector<std::pair<long long, long long>> task_rows[2];   // tree-position rows each task serves
   hb::Task* d_tasks[2] = {nullptr, nullptr};
@@ -415,8 +422,12 @@ void curve_bf_free(hb_ctx* c);
 void curve_bf_info(const hb_ctx* c, int which, int* levels, int* max_rank, long long* entries);
 void curve_bf_apply(hb_ctx* c, int which, const double2* x_nat, long long ldx, double scale, double2* y_nat,
                     long long ldy, int accumulate, int nrhs, cudaStream_t st);
-void run_tasks_fp64(const Task* d_tasks, int n, const double2* F, double2* x, double2* y, double2* xh, int R,
-                    cudaStream_t st);   // apply.cu
+// FP64 step tasks (apply.cu): the factor exponents of n tasks, the largest
+// task of a step, and one step
+void task_exponents(Task* d_tasks, int n, const double2* F, cudaStream_t st);
+StepShape step_shape(const Task* tasks, int n);
+void run_tasks_fp64(const Task* d_tasks, int n, const StepShape& shape, const double2* F, double2* x, double2* y,
+                    double2* xh, int R, cudaStream_t st);
 void curve_free(hb_ctx* c);
 void curve_operators(hb_ctx* c, double2* k_s2s, double2* k_v2s, double2* k_s2v, cudaStream_t st);
 void apply_inclusion(hb_ctx* c, const double2* s, double2* u, int nrhs, int v2v_dense, cudaStream_t st);
