@@ -135,6 +135,7 @@ struct StepArgs {
   int selftest;               // the first warp also waits on a barrier nothing completes
   const unsigned* need = nullptr;   // fused pairs: producer chains of each component slot, PAIR_SLOTS per CTA
   unsigned* gsync = nullptr;        // grid barriers: [0] arrivals, [1] CTAs finished (both 0 between launches)
+  int more = 0;                     // another step launch of this apply follows (it is let start early)
 };
 
 // Accumulate ks k-steps of an item into acc: NTL n-tiles whose tiles are
@@ -387,6 +388,13 @@ __global__ void __launch_bounds__(NWARP * 32, 1) bf_step_kernel(StepArgs a) {
   };
   load_win(0);
   load_win(1);
+  // The next depth's launch may begin: its CTAs take an SM as this launch's
+  // leave it and fetch their records and factor runs there while other SMs
+  // still compute; they read vectors only past griddepcontrol.wait, i.e. once
+  // this launch is complete (and with it, as every warp here waits too, all
+  // before it).  Triggering at the end instead put the launch and those
+  // fetches after the slowest CTA: 188 -> 169 us at 256^2, 59 -> 54 at 64^2.
+  if (a.more && lane == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   auto f_bytes = [](const WItem& w) { return (uint32_t)w.ntl * (uint32_t)w.ks * 512u; };
   auto x_bytes = [](const WItem& w) { return (uint32_t)w.ks * (uint32_t)(MT * 1024); };
   // PAIRS: a consumer item (flags & 16) reads the outputs of its component's
@@ -611,7 +619,6 @@ __global__ void __launch_bounds__(NWARP * 32, 1) bf_step_kernel(StepArgs a) {
       }
     }
   }
-  if (lane == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // ------------------------------------------------ persistent dataflow ----
@@ -1781,9 +1788,9 @@ static void launch_shape(FlowPlan* P, const LaunchShape& L, const LaunchCtx& c,
   if (L.mode == 0) {
     gather_native(c.s, c.pperm, c.x, L.tc ? c.x_tc : nullptr, c.nv_tiles, c.Nv, c.R, MT, c.scale, c.st);
     bool first = true;   // the timer brackets all depth launches (PDL stays intact)
-    auto launch = [&](const DepthStreams& ds, bool cone_kernel) {
+    auto launch = [&](const DepthStreams& ds, bool cone_kernel, bool more) {
       StepArgs args{ds.d_items, ds.d_off, c.F, c.x, c.xh, c.u, c.pperm, c.Nv, c.R, L.stages, L.stage, c.budget,
-                    c.err, c.selftest ? 1 : 0};
+                    c.err, c.selftest ? 1 : 0, nullptr, nullptr, more ? 1 : 0};
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(ds.grid);
       cfg.blockDim = dim3(NWARP * 32);
@@ -1825,7 +1832,7 @@ static void launch_shape(FlowPlan* P, const LaunchShape& L, const LaunchCtx& c,
       if (cs.pair_grid != L.grid) build_pair_streams(cs, L.grid, ntransfer);
       for (const DepthStreams& ds : cs.pair_streams) {
         StepArgs args{ds.d_items, ds.d_off, c.F, c.x, c.xh, c.u, c.pperm, c.Nv, c.R, L.stages, L.stage, c.budget,
-                      c.err, c.selftest ? 1 : 0, ds.d_need};
+                      c.err, c.selftest ? 1 : 0, ds.d_need, nullptr, 1};
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(ds.grid);
         cfg.blockDim = dim3(NWARP * 32);
@@ -1844,7 +1851,7 @@ static void launch_shape(FlowPlan* P, const LaunchShape& L, const LaunchCtx& c,
         tc_leaf_launch(c.tc_plan, MT, c.F_tc, c.x_tc, c.xh, c.u, c.pperm, c.Nv, c.R, c.err, c.budget, c.st);
       } else {
         if (cs.depth_grid != L.grid) build_depth_streams(cs, L.grid);
-        launch(cs.depth_streams.back(), false);   // the leaf outputs
+        launch(cs.depth_streams.back(), false, false);   // the leaf outputs
       }
       timer(0, false);
       return;
@@ -1852,9 +1859,9 @@ static void launch_shape(FlowPlan* P, const LaunchShape& L, const LaunchCtx& c,
     if (L.cones) {
       if (cs.cone_grid != L.grid) build_cone_streams(cs, L.grid);
       if (cs.depth_grid_c != L.grid) build_depth_streams(cs, L.grid, true);
-      launch(cs.cone_streams, true);
+      launch(cs.cone_streams, true, true);
       for (const DepthStreams& ds : cs.depth_streams_c)
-        if (ds.grid) launch(ds, false);
+        if (ds.grid) launch(ds, false, L.tc || &ds != &cs.depth_streams_c.back());
       if (L.tc) {
         tc_leaf_launch(c.tc_plan, MT, c.F_tc, c.x_tc, c.xh, c.u, c.pperm, c.Nv, c.R, c.err, c.budget, c.st);
       }
@@ -1862,24 +1869,8 @@ static void launch_shape(FlowPlan* P, const LaunchShape& L, const LaunchCtx& c,
       return;
     }
     if (cs.depth_grid != L.grid) build_depth_streams(cs, L.grid);
-    for (const DepthStreams& ds : cs.depth_streams) {
-      if (ds.grid == 0) continue;
-      StepArgs args{ds.d_items, ds.d_off, c.F, c.x, c.xh, c.u, c.pperm, c.Nv, c.R, L.stages, L.stage, c.budget,
-                    c.err, c.selftest ? 1 : 0};
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(ds.grid);
-      cfg.blockDim = dim3(NWARP * 32);
-      cfg.dynamicSmemBytes = L.smem;
-      cfg.stream = c.st;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      attr[0].val.programmaticStreamSerializationAllowed = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      if (first) timer(0, true);
-      first = false;
-      HB_CUDA(cudaLaunchKernelEx(&cfg, bf_step_kernel<MT, 0>, args));
-    }
+    for (const DepthStreams& ds : cs.depth_streams)
+      if (ds.grid) launch(ds, false, L.tc || &ds != &cs.depth_streams.back());
     if (L.tc) {   // the leaf outputs (the last depth) on the tensor cores
       if (first) timer(0, true);
       first = false;
@@ -2054,7 +2045,7 @@ static void launch_shard_mt(FlowPlan* P, const LaunchCtx& c, long long lo, long 
   for (const DepthStreams& ds : cs.depth_streams) {
     if (ds.grid == 0) continue;
     StepArgs args{ds.d_items, ds.d_off, c.F, c.x, c.xh, c.u, c.pperm, c.Nv, c.R, L.stages, L.stage, c.budget,
-                  c.err, 0};
+                  c.err, 0, nullptr, nullptr, &ds != &cs.depth_streams.back() ? 1 : 0};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ds.grid);
     cfg.blockDim = dim3(NWARP * 32);
