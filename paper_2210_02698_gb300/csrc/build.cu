@@ -44,6 +44,14 @@ namespace hb {
 #endif
 constexpr int LEAF_NG = HB_LEAF_NG;   // n-tiles per group of the leaf-output tasks (mixed apply)
 constexpr int BLOCK_NG = HB_NG;       // n-tiles per group of the other tasks
+// A depth with fewer chains than this has its groups halved (down to single
+// tiles): a chain is a serial unit of one warp (64^2: 64 leaf chains of 30
+// k-steps x 8 tiles, 11 us of the 59), and the tiles' sums are the same in any
+// group.  Half the GPU's warps, measured (us, one right-hand side, 64^2 / 96^2 /
+// 128^2 / 256^2): never halved 54 / 59 / 75 / 169, below 608 chains 32 / 52 / 59
+// / 169, below 1216 32 / 54 / 63 / 171, below 2432 32 / 57 / 67 / 185 (every
+// chain reads its inputs again).
+constexpr long long CHAINS_WANTED = 608;
 // Cones: levels 0 .. min(L, CONE_M) of every butterfly (forward; adjoint: its
 // first CONE_M + 1 steps) split into groups closed under their dependencies.
 // Forward: level k block (i, j) reads level k - 1 blocks (i/2, 2j), (i/2, 2j+1),
@@ -579,6 +587,15 @@ static void make_plans(hb_ctx* c, std::vector<Butterfly>& bfs, const std::vector
       // n-tiles per group: 4, and LEAF_NG for the many-term leaf outputs,
       // whose accumulation chains are long (smaller groups balance better)
       int ng = BLOCK_NG;
+      auto pick_ng = [&](int most, const std::vector<int>& tiles) {
+        int n = most;
+        for (; n > 1; n /= 2) {
+          long long chains = 0;
+          for (int v : tiles) chains += (v + n - 1) / n;
+          if (chains >= CHAINS_WANTED) break;
+        }
+        return n;
+      };
       // a native block of op(F) with outputs (r1 | r2) and inputs (k1 | k2)
       auto nat = [&](long long src, int ld, int r1, int r2, int k1, int k2) {
         NatBlock B{};
@@ -603,6 +620,8 @@ static void make_plans(hb_ctx* c, std::vector<Butterfly>& bfs, const std::vector
         tm.x_buf = x_buf;
         return tm;
       };
+      std::vector<int> leaf_tiles;
+      for (long long t = 0; t < nleaf; ++t) leaf_tiles.push_back((int)tiles8(leaf_size(t)));
       std::vector<NatTask> nt;
       // first cone id of every butterfly: 2^(L - min(L, CONE_M)) cones each
       std::vector<long long> cone_base(bfs.size() + 1, 0);
@@ -619,7 +638,12 @@ static void make_plans(hb_ctx* c, std::vector<Butterfly>& bfs, const std::vector
       };
       if (dir == 0) {
         // depth k: V^0 (k = 0) and W^k of every butterfly with L >= k
-        for (int k = 0; k <= Lmax; ++k)
+        for (int k = 0; k <= Lmax; ++k) {
+          std::vector<int> tiles;
+          for (const Butterfly& b : bfs)
+            if (b.L >= k)
+              for (const BlockRec& br : b.lev[(size_t)k]) tiles.push_back((int)tiles8(br.rank));
+          ng = pick_ng(BLOCK_NG, tiles);
           for (size_t bi = 0; bi < bfs.size(); ++bi) {
             const Butterfly& b = bfs[bi];
             if (b.L < k) continue;
@@ -653,8 +677,9 @@ static void make_plans(hb_ctx* c, std::vector<Butterfly>& bfs, const std::vector
                 nt.push_back(std::move(t));
               }
           }
+        }
         // last depth: y(leaf t) = D_t x(t) + sum over levels of K^L x_hat
-        ng = LEAF_NG;
+        ng = pick_ng(LEAF_NG, leaf_tiles);
         for (long long t = 0; t < nleaf; ++t) {
           const int sz = leaf_size(t);
           NatTask o = task(c->leaf_tile[(size_t)t], tiles8(sz), Lmax + 1, 1);
@@ -675,6 +700,12 @@ static void make_plans(hb_ctx* c, std::vector<Butterfly>& bfs, const std::vector
         }
       } else {
         // depth 0: K^L^H
+        {
+          std::vector<int> tiles;
+          for (const Butterfly& b : bfs)
+            for (const BlockRec& br : b.lev[(size_t)b.L]) tiles.push_back((int)tiles8(br.rank));
+          ng = pick_ng(BLOCK_NG, tiles);
+        }
         for (size_t bi = 0; bi < bfs.size(); ++bi) {
           const Butterfly& b = bfs[bi];
           for (int i = 0; i < (1 << b.L); ++i) {
@@ -693,7 +724,15 @@ static void make_plans(hb_ctx* c, std::vector<Butterfly>& bfs, const std::vector
           }
         }
         // depth d: W^{L-d+1}^H, writing the pair of level L-d blocks
-        for (int d = 1; d <= Lmax; ++d)
+        for (int d = 1; d <= Lmax; ++d) {
+          std::vector<int> tiles;
+          for (const Butterfly& b : bfs)
+            if (b.L >= d) {
+              const auto& lev = b.lev[(size_t)(b.L - d)];   // written in pairs (2j, 2j + 1)
+              for (size_t q = 0; q + 1 < lev.size(); q += 2)
+                tiles.push_back((int)(tiles8(lev[q].rank) + tiles8(lev[q + 1].rank)));
+            }
+          ng = pick_ng(BLOCK_NG, tiles);
           for (size_t bi = 0; bi < bfs.size(); ++bi) {
             const Butterfly& b = bfs[bi];
             if (b.L < d) continue;
@@ -723,8 +762,9 @@ static void make_plans(hb_ctx* c, std::vector<Butterfly>& bfs, const std::vector
                 nt.push_back(std::move(t));
               }
           }
+        }
         // last depth: y(leaf t) = D_t^H x(t) + sum over levels of V^0^H x_hat
-        ng = LEAF_NG;
+        ng = pick_ng(LEAF_NG, leaf_tiles);
         for (long long t = 0; t < nleaf; ++t) {
           const int sz = leaf_size(t);
           NatTask o = task(c->leaf_tile[(size_t)t], tiles8(sz), Lmax + 1, 1);
