@@ -51,7 +51,7 @@ __global__ void scatter_kernel(const double2* __restrict__ y, const long long* _
 // parts interleaved; D_r takes A rows (Re X, -Im X), D_i (Im X, Re X).  Up to
 // eight right-hand sides (HALF) both go into one MMA, rows 0-7 and 8-15.
 //
-// A CTA of 8 warps takes up to 64 outputs (8 n-tiles, blockIdx.y of them) of
+// A CTA of 8 warps takes up to 64 outputs (8 n-tiles; row_blocks CTAs per task) of
 // one task.  It scales X per right-hand side and F per task (tk.fe, found
 // when the plan is made), splits X into digit fragments in shared memory,
 // KC k-steps at a time, and every warp streams its n-tile's F straight from
@@ -117,16 +117,17 @@ __device__ __noinline__ void task_plain(const Task* __restrict__ task, const dou
 template <bool HALF>
 __global__ void __launch_bounds__(TASK_THREADS, HALF ? 3 : 2)
     task_kernel(const Task* __restrict__ tasks, const double2* __restrict__ F, double2* x, double2* y, double2* xh,
-                int R) {
+                int R, int row_blocks) {
   constexpr int NR = HALF ? 8 : 16;        // right-hand sides of the MMA rows
   constexpr int NE = HALF ? 4 : 8;         // accumulator elements per lane and digit diagonal
   constexpr int XW = HALF ? 2 : 4;         // X fragment words per lane
   extern __shared__ __align__(16) uint32_t xs[];   // [k-step][digit][lane][XW]
   __shared__ int s_ex[16];
   __shared__ int s_bad;
-  const Task tk = tasks[blockIdx.x];
+  const Task* task = tasks + blockIdx.x / row_blocks;
+  const Task tk = *task;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
-  const int tile0 = 8 * blockIdx.y;
+  const int tile0 = 8 * (blockIdx.x % row_blocks);
   const int ntile = min(8, (tk.r_out + 7) / 8 - tile0);
   if (ntile <= 0) return;
   const double2* xin = tk.x_buf == 0 ? x : tk.x_buf == 1 ? y : xh;
@@ -148,7 +149,7 @@ __global__ void __launch_bounds__(TASK_THREADS, HALF ? 3 : 2)
   }
   __syncthreads();
   if (s_bad) {
-    task_plain(tasks + blockIdx.x, F, x, y, xh, R, 8 * tile0, min(tk.r_out, 8 * (tile0 + 8)));
+    task_plain(task, F, x, y, xh, R, 8 * tile0, min(tk.r_out, 8 * (tile0 + 8)));
     return;
   }
 
@@ -286,25 +287,25 @@ __global__ void __launch_bounds__(TASK_THREADS, HALF ? 3 : 2)
   }
 }
 
-// tasks[i].fe = the largest exponent of task i's factor blocks, one warp each
-__global__ void __launch_bounds__(256) task_exponent_kernel(Task* __restrict__ tasks, int n,
-                                                            const double2* __restrict__ F) {
-  const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (i >= n) return;
+// tasks[i].fe = the largest exponent of task i's factor blocks (1 before),
+// blockIdx.y of gridDim.y shares of them
+__global__ void __launch_bounds__(256) task_exponent_kernel(Task* __restrict__ tasks, const double2* __restrict__ F) {
+  Task& tk = tasks[blockIdx.x];
   int e = 1;
-  for (int t = 0; t < tasks[i].nterm; ++t) {
-    const long long cnt = (long long)tasks[i].r_out * tasks[i].r_in[t];
-    const double2* f = F + tasks[i].f_off[t];
-    for (long long k = lane; k < cnt; k += 32) e = max(e, block_exponent(f[k]));
+  for (int t = 0; t < tk.nterm; ++t) {
+    const long long cnt = (long long)tk.r_out * tk.r_in[t];
+    const double2* f = F + tk.f_off[t];
+#pragma unroll 4
+    for (long long k = blockIdx.y * 256 + threadIdx.x; k < cnt; k += 256 * gridDim.y) e = max(e, block_exponent(f[k]));
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-  if (lane == 0) tasks[i].fe = (unsigned short)e;
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((threadIdx.x & 31) == 0) atomicMax(&tk.fe, e);
 }
 
 void task_exponents(Task* d_tasks, int n, const double2* F, cudaStream_t st) {
   if (n <= 0) return;
-  task_exponent_kernel<<<(n + 7) / 8, 256, 0, st>>>(d_tasks, n, F);
+  const unsigned share = (unsigned)std::max(1, std::min(128, 608 / n));
+  task_exponent_kernel<<<dim3((unsigned)n, share), 256, 0, st>>>(d_tasks, F);
   HB_CHECK_LAUNCH();
 }
 
@@ -322,16 +323,17 @@ StepShape step_shape(const Task* tasks, int n) {
 void run_tasks_fp64(const Task* d_tasks, int n, const StepShape& sh, const double2* F, double2* x, double2* y,
                     double2* xh, int R, cudaStream_t st) {
   if (n <= 0) return;
-  const dim3 grid((unsigned)n, (unsigned)std::max(1, (sh.max_out + 63) / 64));
+  const int rb = std::max(1, (sh.max_out + 63) / 64);
+  const unsigned grid = (unsigned)n * (unsigned)rb;
   const size_t frag = (size_t)std::min(TASK_KC, std::max(1, sh.max_ks)) * SPLIT_DIGITS * 32 * 4;
   const size_t red = (size_t)7 * 32 * sizeof(longlong2);   // the k-step shares of one CTA: at most 7 n-tile shares
   if (R <= 8) {
     const size_t smem = std::max(frag * 2, red * 4);
-    task_kernel<true><<<grid, TASK_THREADS, smem, st>>>(d_tasks, F, x, y, xh, R);
+    task_kernel<true><<<grid, TASK_THREADS, smem, st>>>(d_tasks, F, x, y, xh, R, rb);
   } else {
     const size_t smem = std::max(frag * 4, red * 8);
     HB_CUDA(cudaFuncSetAttribute(task_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 56 << 10));
-    task_kernel<false><<<grid, TASK_THREADS, smem, st>>>(d_tasks, F, x, y, xh, R);
+    task_kernel<false><<<grid, TASK_THREADS, smem, st>>>(d_tasks, F, x, y, xh, R, rb);
   }
   HB_CHECK_LAUNCH();
 }
@@ -428,6 +430,98 @@ void ensure_scratch(hb_ctx* c, int nrhs, bool fp64) {
 
 }  // namespace
 
+// ------------------------------------------------- dense product ----
+// Y = alpha A X (or +=) for a stored column-major A (m x k): step tasks over
+// ranges of the inputs (enough CTAs for the chip when m is small; the ranges'
+// sums are added in order), X and Y converted between columns and the tasks'
+// rows of R values.
+__global__ void pack_rows_kernel(const double2* __restrict__ X, long long ldx, long long k, int R, double scale,
+                                 double2* __restrict__ x) {
+  const int r = threadIdx.x;
+  if (r >= R) return;
+  for (long long p = (long long)blockIdx.x * blockDim.y + threadIdx.y; p < k; p += (long long)gridDim.x * blockDim.y) {
+    const double2 v = X[(size_t)r * ldx + p];
+    x[p * R + r] = make_double2(scale * v.x, scale * v.y);
+  }
+}
+
+__global__ void sum_rows_kernel(const double2* __restrict__ y, long long m, int parts, int R, double2* __restrict__ Y,
+                                long long ldy, int accumulate) {
+  const int r = threadIdx.x;
+  if (r >= R) return;
+  for (long long i = (long long)blockIdx.x * blockDim.y + threadIdx.y; i < m; i += (long long)gridDim.x * blockDim.y) {
+    double2 a = accumulate ? Y[(size_t)r * ldy + i] : make_double2(0.0, 0.0);
+    for (int c = 0; c < parts; ++c) {
+      const double2 v = y[((size_t)c * m + i) * R + r];
+      a.x += v.x;
+      a.y += v.y;
+    }
+    Y[(size_t)r * ldy + i] = a;
+  }
+}
+
+DenseOp dense_op(const double2* A, long long m, long long k, cudaStream_t st) {
+  if (m > INT32_MAX || k > INT32_MAX) throw Error{HB_ERR_UNSUPPORTED, "stored operator too large"};
+  DenseOp D;
+  D.A = A;
+  D.m = m;
+  D.k = k;
+  // inputs per task: at least 128 (the exponent scan and the epilogue are per
+  // task), and 304 CTAs of 64 outputs in all where that leaves as many
+  const long long rb = (m + 63) / 64;
+  const long long parts = std::max<long long>(1, std::min<long long>((304 + rb - 1) / rb, (k + 127) / 128));
+  const long long kc = ((k + parts - 1) / parts + 7) / 8 * 8;
+  std::vector<Task> tasks;
+  for (long long k0 = 0; k0 < k; k0 += kc) {
+    Task t{};
+    t.y_off = (long long)tasks.size() * m;
+    t.f_off[0] = k0 * m;
+    t.x_off[0] = k0;
+    t.r_out = (int)m;
+    t.r_in[0] = (int)std::min(kc, k - k0);
+    t.nterm = 1;
+    t.x_buf = 0;
+    t.y_buf = 1;
+    tasks.push_back(t);
+  }
+  D.ntask = (int)tasks.size();
+  D.shape = step_shape(tasks.data(), D.ntask);
+  D.d_tasks = upload(tasks, st);
+  task_exponents(D.d_tasks, D.ntask, A, st);
+  HB_CUDA(cudaStreamSynchronize(st));
+  return D;
+}
+
+void dense_op_free(DenseOp& D) {
+  dev_free(D.d_tasks);
+  D = DenseOp{};
+}
+
+namespace {
+
+// launch shape of the vector kernels: lanes over the right-hand sides
+struct VecGrid {
+  dim3 grid, block;
+  VecGrid(long long rows, int R) {
+    int rp = 1;
+    while (rp < R) rp *= 2;
+    block = dim3((unsigned)rp, (unsigned)(256 / rp));
+    grid = dim3((unsigned)std::max<long long>(1, std::min<long long>((rows + block.y - 1) / block.y, 152LL * 16)));
+  }
+};
+
+}  // namespace
+
+void dense_product(const DenseOp& D, const double2* X, long long ldx, double2* Y, long long ldy, int R, double alpha,
+                   int accumulate, double2* x, double2* y, cudaStream_t st) {
+  const VecGrid in(D.k, R), out(D.m, R);
+  pack_rows_kernel<<<in.grid, in.block, 0, st>>>(X, ldx, D.k, R, alpha, x);
+  HB_CHECK_LAUNCH();
+  run_tasks_fp64(D.d_tasks, D.ntask, D.shape, D.A, x, y, nullptr, R, st);
+  sum_rows_kernel<<<out.grid, out.block, 0, st>>>(y, D.m, D.ntask, R, Y, ldy, accumulate);
+  HB_CHECK_LAUNCH();
+}
+
 namespace {
 
 void run_steps(hb_ctx* c, const double2* F, int nrhs, int dir, cudaStream_t st, TimerScope& ts) {
@@ -441,17 +535,6 @@ void run_steps(hb_ctx* c, const double2* F, int nrhs, int dir, cudaStream_t st, 
     ts.end();
   }
 }
-
-// launch shape of the gather / scatter kernels: lanes over the right-hand sides
-struct VecGrid {
-  dim3 grid, block;
-  VecGrid(long long rows, int R) {
-    int rp = 1;
-    while (rp < R) rp *= 2;
-    block = dim3((unsigned)rp, (unsigned)(256 / rp));
-    grid = dim3((unsigned)std::max<long long>(1, std::min<long long>((rows + block.y - 1) / block.y, 152LL * 16)));
-  }
-};
 
 }  // namespace
 

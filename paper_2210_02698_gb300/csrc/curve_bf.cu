@@ -456,6 +456,8 @@ void curve_compress(hb_ctx* c, int leaf_s) {
   c->curve_bf[0] = v2s;
   c->curve_bf[1] = s2v;
   // the dense forms are not needed any more
+  dense_op_free(c->op_v2s);
+  dense_op_free(c->op_s2v);
   dev_free(c->d_kv2s);
   dev_free(c->d_ks2v);
   c->d_kv2s = c->d_ks2v = nullptr;

@@ -124,12 +124,21 @@ struct Task {
   int r_in[2];
   unsigned char nterm, x_buf, y_buf, accumulate;
   unsigned char conj_t, kind;
-  unsigned short fe;        // largest biased exponent of its factor blocks (task_exponents)
+  int fe;                   // largest biased exponent of its factor blocks (task_exponents)
 };
 // The largest task of a step: outputs, and k-steps of 8 inputs (each term's
 // inputs rounded up).
 struct StepShape {
   int max_out, max_ks;
+};
+// A stored dense operator (m x k, column-major) as step tasks over ranges of
+// its inputs (apply.cu).
+struct DenseOp {
+  const double2* A = nullptr;
+  long long m = 0, k = 0;
+  int ntask = 0;
+  StepShape shape{0, 0};
+  Task* d_tasks = nullptr;
 };
 
 // Native (MMA-fragment) layout of the mixed apply (bf_mma.cu).  A factor
@@ -315,17 +324,21 @@ struct hb_ctx {
 
   // curve inclusion (inclusion.cu): segments and the dense surface operators
   long long ns = 0;                // segments; 0: no curve set
+  long long ns_set = 0;            // segments of the arrays below (set before ns, while they are assembled)
   double2* d_seg = nullptr;        // ns centres (x, z)
   double* d_segw = nullptr;        // ns lengths
   double* d_segn = nullptr;        // ns values of n at the centres
-  double2* d_cellpts = nullptr;    // N_v cell centres (x, z)
   double2* d_lu = nullptr;         // K^{s2s} LU-factored in place (ns x ns, column-major)
   int* d_piv = nullptr;            // its row interchanges
   double2* d_inv = nullptr;        // (K^{s2s})^{-1} from the LU factors, ns x ns column-major
   double2* d_kv2s = nullptr;       // K^{v2s}, ns x N_v column-major
   double2* d_ks2v = nullptr;       // K^{s2v}, N_v x ns column-major
+  hb::DenseOp op_v2s, op_inv, op_s2v;   // the three as step tasks
+  double* d_seglag = nullptr;      // Lagrange basis at the segment centres (inclusion.cu)
+  double* d_segG = nullptr;        // table contractions at the segment centres (inclusion.cu)
   double2* d_cy = nullptr;         // surface vectors of an apply, 2 ns x cy_cap (Y, then P)
   int cy_cap = 0;
+  double2* d_pack = nullptr;       // operands of the dense products (rows of up to 16 right-hand sides)
   void* curve_bf[2] = {nullptr, nullptr};   // hb_curve_compress: K^{v2s} (0), K^{s2v} (1) as butterflies
 
   // hb_record_id_blocks: blocks per butterfly level to keep, and the kept ones
@@ -426,6 +439,12 @@ void curve_bf_apply(hb_ctx* c, int which, const double2* x_nat, long long ldx, d
 // task of a step, and one step
 void task_exponents(Task* d_tasks, int n, const double2* F, cudaStream_t st);
 StepShape step_shape(const Task* tasks, int n);
+// a stored dense operator as step tasks; Y = alpha A X (or +=) for R <= 16
+// columns, x / y: row-major operands (k x R and ntask m x R)
+DenseOp dense_op(const double2* A, long long m, long long k, cudaStream_t st);
+void dense_op_free(DenseOp& D);
+void dense_product(const DenseOp& D, const double2* X, long long ldx, double2* Y, long long ldy, int R, double alpha,
+                   int accumulate, double2* x, double2* y, cudaStream_t st);
 void run_tasks_fp64(const Task* d_tasks, int n, const StepShape& shape, const double2* F, double2* x, double2* y,
                     double2* xh, int R, cudaStream_t st);
 void curve_free(hb_ctx* c);

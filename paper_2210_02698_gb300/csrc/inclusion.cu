@@ -62,77 +62,148 @@ __device__ __forceinline__ void basis_at(const double* nodes, const double* bw, 
   for (int k = 0; k < nI; ++k) L[k] /= den;
 }
 
-// out[a + b*ldo] = sgn * w_b * g(obs_a, src_b) for a < m (w_b = wsrc[b], or 1
-// when wsrc is null).  With diag (the observation points are the source
-// points, m = n) the entry a == b is the K^{s2s} diagonal of segment a
-// (lengths wsrc, index nseg).  One CTA per source point b: first
-// G[q][i] = sum_j F_q[i][j] T_j(src_b) (T_j = l_{j1}(x) l_{j2}(z),
-// j = j2 n_I + j1) in shared memory, then the threads take the observation
-// points, f_q = sum_i T_i(obs_a) G[q][i].
-__global__ void __launch_bounds__(256) green_columns_kernel(PointTables P, const double2* __restrict__ obs, long long m,
-                                                            const double2* __restrict__ src,
-                                                            const double* __restrict__ wsrc,
-                                                            const double* __restrict__ nseg, double sgn, int diag,
-                                                            double2* __restrict__ out, long long ldo) {
-  __shared__ double G[3 * CMAX_NI * CMAX_NI];
-  __shared__ double bw[2][CMAX_NI];
-  __shared__ double Ls[2][CMAX_NI];
-  const int nI = P.nI, NI = P.NI, t = threadIdx.x;
-  const long long b = blockIdx.x;
-  if (t < 2 * nI) {
-    const int d = t / nI, k = t % nI;
-    const double* nd = P.nodes + d * nI;
-    double p = 1.0;
-    for (int q = 0; q < nI; ++q)
-      if (q != k) p *= (nd[k] - nd[q]);
-    bw[d][k] = 1.0 / p;
+// ---- the dense curve operators ----
+// Every entry is g(seg, cell), g(cell, seg) or g(seg, seg'), so the tables are
+// contracted with a segment's basis once, and the cells' tensor structure
+// does the rest line by line: 48 FMAs and a tabulated Hankel pair (27) an
+// entry.  (Contracting per source cell and evaluating the full basis and the
+// recurrences per entry took 28.8 ms of FP64 at 96^2 with 300 segments.)
+
+// lag[p][0..nI) = l_k(x_p), lag[p][16..16 + nI) = l_k(z_p) of segment centre p
+__global__ void seg_basis_kernel(PointTables P, const double2* __restrict__ seg, long long ns, double* __restrict__ lag) {
+  const long long p = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 1;
+  const int d = threadIdx.x & 1;
+  if (p >= ns) return;
+  const double* nd = P.nodes + d * P.nI;
+  double bw[CMAX_NI], L[CMAX_NI];
+  for (int k = 0; k < P.nI; ++k) {
+    double v = 1.0;
+    for (int q = 0; q < P.nI; ++q)
+      if (q != k) v *= (nd[k] - nd[q]);
+    bw[k] = 1.0 / v;
   }
+  basis_at(nd, bw, P.nI, d == 0 ? seg[p].x : seg[p].y, L);
+  for (int k = 0; k < CMAX_NI; ++k) lag[(size_t)p * 32 + 16 * d + k] = k < P.nI ? L[k] : 0.0;
+}
+
+// G[((t 3 + q) N_I + i) ns + p] = sum_j tab_t[q][i][j] T_j(seg_p), T_j =
+// l_{j1}(x) l_{j2}(z); t = 0: the tables (p a source), 1: transposed (p an
+// observation point).  blockIdx.y = (t, q, i), lanes over segments.
+__global__ void __launch_bounds__(128) seg_contract_kernel(PointTables P, const double* __restrict__ lag, long long ns,
+                                                           double* __restrict__ G) {
+  __shared__ double row[CMAX_NI * CMAX_NI];
+  const int nI = P.nI, NI = P.NI;
+  const double* f = P.tab + (size_t)blockIdx.y * NI;
+  for (int j = threadIdx.x; j < NI; j += blockDim.x) row[j] = f[j];
   __syncthreads();
-  if (t < 2) {
-    const double2 s = src[b];
-    basis_at(P.nodes + t * nI, bw[t], nI, t == 0 ? s.x : s.y, Ls[t]);
+  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= ns) return;
+  const double* l = lag + (size_t)p * 32;
+  double lx[CMAX_NI];
+#pragma unroll
+  for (int k = 0; k < CMAX_NI; ++k) lx[k] = l[k];
+  double acc = 0.0;
+  for (int j2 = 0; j2 < nI; ++j2) {
+    double a = 0.0;
+#pragma unroll
+    for (int j1 = 0; j1 < CMAX_NI; ++j1)
+      if (j1 < nI) a = fma(row[j2 * nI + j1], lx[j1], a);
+    acc = fma(l[16 + j2], a, acc);
   }
-  __syncthreads();
-  for (int idx = t; idx < 3 * NI; idx += blockDim.x) {
-    const int q = idx / NI, i = idx % NI;
-    const double* Fr = P.tab + ((size_t)q * NI + i) * NI;
-    double acc = 0.0;
-    for (int j2 = 0; j2 < nI; ++j2) {
-      double a2 = 0.0;
-      for (int j1 = 0; j1 < nI; ++j1) a2 = fma(Fr[j2 * nI + j1], Ls[0][j1], a2);
-      acc = fma(Ls[1][j2], a2, acc);
+  G[(size_t)blockIdx.y * ns + p] = acc;
+}
+
+// g from interpolated tau^2, v0, v1 with the tabulated Hankel pair (as the
+// dense apply): i c (v0 H0 - (2 / w^2) v1 x H1)
+__device__ __forceinline__ double2 green_tab(const HankelTable& T, double omega, double t2, double v0, double v1) {
+  const double c = 0.88622692545275801365;   // sqrt(pi)/2
+  const double w2 = omega * omega;
+  const HankelFG h = hankel_of_t2(T, w2, t2);
+  const double a = c * v0, b = (2.0 * c / w2) * v1;
+  return make_double2(fma(-h.F.y, a, h.G.y * b), fma(h.F.x, a, -h.G.x * b));
+}
+
+// Segment p (one thread) against the cells [a0, a1) of grid line line0 + blockIdx.y.
+// V2S: out[cell ns + p] = g(seg_p, cell) (G: the transposed contractions); else
+// out[p Nv + cell] = w_p g(cell, seg_p), two cells at a time (one 32-byte sector).
+template <bool V2S>
+__global__ void __launch_bounds__(64) seg_line_kernel(EntryParams E, const double* __restrict__ G, long long ns,
+                                                      const double* __restrict__ w, int line0, double2* __restrict__ out) {
+  const int nI = E.nI;
+  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= ns) return;
+  const int b = line0 + blockIdx.y;
+  const double* lz = E.LZ + (size_t)b * nI;
+  double P[3][CMAX_NI];
+#pragma unroll
+  for (int q = 0; q < 3; ++q)
+#pragma unroll
+    for (int k1 = 0; k1 < CMAX_NI; ++k1) {
+      double a = 0.0;
+      if (k1 < nI)
+        for (int k2 = 0; k2 < nI; ++k2) a = fma(lz[k2], G[(size_t)(q * E.NI + k2 * nI + k1) * ns + p], a);
+      P[q][k1] = a;
     }
-    G[idx] = acc;
-  }
-  __syncthreads();
-  const double wb = wsrc ? wsrc[b] : 1.0;
-  for (long long a = t; a < m; a += blockDim.x) {
-    double2 val;
-    if (diag && a == b) {
-      const double w = wsrc[b];
-      const double c = (2.0 / HB_PI) * (log(GAMMA_EXP * P.omega * nseg[b] * w / 4.0) - 1.0);
-      val = make_double2(0.25 * w * c, -0.25 * w);   // -(i w/4)(1 + i c)
-    } else {
-      const double2 o = obs[a];
-      double Lx[CMAX_NI], Lz[CMAX_NI];
-      basis_at(P.nodes, bw[0], nI, o.x, Lx);
-      basis_at(P.nodes + nI, bw[1], nI, o.y, Lz);
-      double f[3];
-      for (int q = 0; q < 3; ++q) {
-        const double* Gq = G + q * NI;
-        double acc = 0.0;
-        for (int i2 = 0; i2 < nI; ++i2) {
-          double a2 = 0.0;
-          for (int i1 = 0; i1 < nI; ++i1) a2 = fma(Lx[i1], Gq[i2 * nI + i1], a2);
-          acc = fma(Lz[i2], a2, acc);
-        }
-        f[q] = acc;
+  const int a0 = (int)((long long)E.nx * blockIdx.z / gridDim.z), a1 = (int)((long long)E.nx * (blockIdx.z + 1) / gridDim.z);
+  const double wp = V2S ? 1.0 : w[p];
+  const long long Nv = (long long)E.nx * E.ny;
+  for (int a = a0; a < a1; ++a) {
+    const double* lx = E.LX + (size_t)a * nI;
+    double f[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int k = 0; k < CMAX_NI; ++k) {
+      if (k < nI) {
+        const double l = lx[k];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) f[q] = fma(l, P[q][k], f[q]);
       }
-      const double2 g = hb_green(f[0], f[1], f[2], P.omega);
-      val = make_double2(sgn * wb * g.x, sgn * wb * g.y);
     }
-    out[(size_t)b * ldo + a] = val;
+    const double2 g = green_tab(E.hank, E.omega, f[0], f[1], f[2]);
+    const long long cell = (long long)b * E.nx + a;
+    if (V2S) out[cell * ns + p] = g;
+    else out[p * Nv + cell] = make_double2(wp * g.x, wp * g.y);
   }
+}
+
+// K^{s2s}: entry (i, j) = -w_j g(seg_i, seg_j), the diagonal the segment's own
+// term.  One thread per i, blockIdx.y = j (G: the forward contractions).
+__global__ void __launch_bounds__(128) seg_seg_kernel(EntryParams E, const double* __restrict__ lag,
+                                                      const double* __restrict__ G, long long ns,
+                                                      const double* __restrict__ w, const double* __restrict__ nseg,
+                                                      double2* __restrict__ out) {
+  __shared__ double g[3 * CMAX_NI * CMAX_NI];
+  const int nI = E.nI, NI = E.NI;
+  const long long j = blockIdx.y;
+  for (int k = threadIdx.x; k < 3 * NI; k += blockDim.x) g[k] = G[(size_t)k * ns + j];
+  __syncthreads();
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= ns) return;
+  const double wj = w[j];
+  double2 v;
+  if (i == j) {
+    const double c = (2.0 / HB_PI) * (log(GAMMA_EXP * E.omega * nseg[j] * wj / 4.0) - 1.0);
+    v = make_double2(0.25 * wj * c, -0.25 * wj);   // -(i w/4)(1 + i c)
+  } else {
+    const double* l = lag + (size_t)i * 32;
+    double lx[CMAX_NI];
+#pragma unroll
+    for (int k = 0; k < CMAX_NI; ++k) lx[k] = l[k];
+    double f[3];
+    for (int q = 0; q < 3; ++q) {
+      double acc = 0.0;
+      for (int i2 = 0; i2 < nI; ++i2) {
+        double a = 0.0;
+#pragma unroll
+        for (int i1 = 0; i1 < CMAX_NI; ++i1)
+          if (i1 < nI) a = fma(lx[i1], g[q * NI + i2 * nI + i1], a);
+        acc = fma(l[16 + i2], a, acc);
+      }
+      f[q] = acc;
+    }
+    const double2 gr = green_tab(E.hank, E.omega, f[0], f[1], f[2]);
+    v = make_double2(-wj * gr.x, -wj * gr.y);
+  }
+  out[(size_t)j * ns + i] = v;
 }
 
 // Batched columns of curve-operator blocks: job q (one CTA) writes
@@ -191,97 +262,209 @@ __global__ void __launch_bounds__(256) green_jobs_kernel(PointTables P, const do
   }
 }
 
-__global__ void cell_points_kernel(int nx, long long Nv, double x0, double y0, double h, double2* __restrict__ pts) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < Nv; i += (long long)gridDim.x * blockDim.x) {
-    const long long a = i % nx, b = i / nx;
-    pts[i] = make_double2(x0 + (a + 0.5) * h, y0 + (b + 0.5) * h);
-  }
+// ---- LU with partial pivoting, panels of LU_NB columns ----
+// Per panel two launches: one CTA factors the panel (pivot p of column j =
+// the row of the largest |A_ij|^2 over i >= j, lowest index on ties; rows
+// interchanged, multipliers A_ij /= A_jj), then a CTA per strip of LU_CS other
+// columns interchanges their rows and, right of the panel, solves with the
+// panel's unit lower triangle and subtracts the products.  Panels are narrow
+// because one SM's FP64 unit factors them (2 FMAs a cycle: 16 columns of 300
+// rows took 188 us); strips are of 2 columns until they fill the chip.
+constexpr int LU_NB = 4;
+constexpr int LU_PT = 512;    // threads of the panel kernel
+constexpr int LU_SB = 16;     // rows per block of the substitutions
+inline int lu_strip(int columns) { return columns < 2 * 608 ? 2 : 8; }
+
+__device__ __forceinline__ double2 csub_mul(double2 a, double2 l, double2 u) {   // a - l u
+  a.x = fma(-l.x, u.x, fma(l.y, u.y, a.x));
+  a.y = fma(-l.x, u.y, fma(-l.y, u.x, a.y));
+  return a;
+}
+__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
+  return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-// Step k of the LU factorisation with partial pivoting of the column-major
-// n x n matrix A: pivot p = the row of the largest |A_ik|^2 over i >= k
-// (lowest index on ties), rows k and p interchanged across all columns,
-// multipliers A_ik /= A_kk for i > k.  One CTA of 256 threads.
-__global__ void __launch_bounds__(256) lu_pivot_kernel(double2* __restrict__ A, int n, int k, int* __restrict__ piv,
-                                                       int* __restrict__ singular) {
-  __shared__ double bv[256];
-  __shared__ int bi[256];
-  const int t = threadIdx.x;
-  double2* colk = A + (size_t)k * n;
+__global__ void __launch_bounds__(LU_PT) lu_panel_kernel(double2* __restrict__ A, int n, int k0, int* __restrict__ piv,
+                                                         int* __restrict__ singular) {
+  __shared__ double wv[LU_PT / 32];
+  __shared__ int wi[LU_PT / 32];
+  __shared__ int s_p;
+  __shared__ double2 urow[LU_NB];
+  __shared__ double2 s_inv;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int nb = min(LU_NB, n - k0);
+  auto at = [&](int i, int c) -> double2& { return A[(size_t)(k0 + c) * n + i]; };
   double best = -1.0;
-  int at = n;
-  for (int i = k + t; i < n; i += blockDim.x) {
-    const double2 v = colk[i];
+  int bi = n;
+  for (int i = k0 + t; i < n; i += LU_PT) {
+    const double2 v = at(i, 0);
     const double m2 = v.x * v.x + v.y * v.y;
     if (m2 > best) {
       best = m2;
-      at = i;
+      bi = i;
     }
   }
-  bv[t] = best;
-  bi[t] = at;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (t < s) {
-      const double o = bv[t + s];
-      const int oi = bi[t + s];
-      if (o > bv[t] || (o == bv[t] && oi < bi[t])) {
-        bv[t] = o;
-        bi[t] = oi;
+  for (int j = 0; j < nb; ++j) {
+    const int k = k0 + j;
+    auto take = [&](double ov, int oi) {
+      if (ov > best || (ov == best && oi < bi)) {
+        best = ov;
+        bi = oi;
+      }
+    };
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) take(__shfl_xor_sync(0xffffffffu, best, o), __shfl_xor_sync(0xffffffffu, bi, o));
+    if (lane == 0) {
+      wv[warp] = best;
+      wi[warp] = bi;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      best = lane < LU_PT / 32 ? wv[lane] : -1.0;
+      bi = lane < LU_PT / 32 ? wi[lane] : n;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) take(__shfl_xor_sync(0xffffffffu, best, o), __shfl_xor_sync(0xffffffffu, bi, o));
+      const bool zero = !(best > 0.0) || bi >= n;   // an all-zero (or NaN) column
+      const int p = bi >= n ? k : bi;
+      if (lane == 0) {
+        s_p = p;
+        piv[k] = p;
+        if (zero) *singular = 1;
+      }
+      // the panel's rows k and p interchanged; row k from the pivot column on is U
+      if (lane < nb) {
+        const double2 a = at(k, lane), b = at(p, lane);
+        if (p != k) {
+          at(k, lane) = b;
+          at(p, lane) = a;
+        }
+        urow[lane] = b;
+        if (lane == j) {   // one warp divides: 16 of them would hold the FP64 unit for microseconds
+          const double dd = b.x * b.x + b.y * b.y;
+          s_inv = dd > 0.0 ? make_double2(b.x / dd, -b.y / dd) : make_double2(1.0, 0.0);
+        }
       }
     }
     __syncthreads();
-  }
-  int p = bi[0];
-  const bool zero = !(bv[0] > 0.0) || p >= n;   // an all-zero (or NaN) column
-  if (p >= n) p = k;
-  if (t == 0) {
-    piv[k] = p;
-    if (zero) *singular = 1;
-  }
-  if (p != k)
-    for (int j = t; j < n; j += blockDim.x) {
-      double2* cj = A + (size_t)j * n;
-      const double2 a = cj[k];
-      cj[k] = cj[p];
-      cj[p] = a;
+    best = -1.0;
+    bi = n;
+    const double2 inv = s_inv;
+    for (int i = k + 1 + t; i < n; i += LU_PT) {
+      const double2 l = cmul(at(i, j), inv);
+      at(i, j) = l;
+      for (int c = j + 1; c < nb; ++c) {
+        const double2 v = csub_mul(at(i, c), l, urow[c]);
+        at(i, c) = v;
+        if (c == j + 1) {
+          const double m2 = v.x * v.x + v.y * v.y;
+          if (m2 > best) {
+            best = m2;
+            bi = i;
+          }
+        }
+      }
     }
+    __syncthreads();   // row k + 1 .. of the panel complete before the next interchange
+  }
+}
+
+// Strip blockIdx.x of CS columns outside the panel [k0, k0 + nb).
+template <int CS>
+__global__ void __launch_bounds__(256) lu_strip_kernel(double2* __restrict__ A, int n, int k0, const int* __restrict__ piv) {
+  __shared__ double2 U[LU_NB][CS];
+  const int t = threadIdx.x, nb = min(LU_NB, n - k0);
+  const int c0 = blockIdx.x * CS, nc = min(CS, n - nb - c0);
+  auto col = [&](int c) { return A + (size_t)(c0 + c < k0 ? c0 + c : c0 + c + nb) * n; };   // skips the panel
+  if (t < nc) {
+    double2* a = col(t);
+    for (int j = 0; j < nb; ++j) {
+      const int p = piv[k0 + j];
+      if (p != k0 + j) {
+        const double2 v = a[k0 + j];
+        a[k0 + j] = a[p];
+        a[p] = v;
+      }
+    }
+    if (c0 + t >= k0) {
+      double2 u[LU_NB];
+#pragma unroll
+      for (int i = 0; i < LU_NB; ++i) {
+        u[i] = make_double2(0.0, 0.0);
+        if (i < nb) {
+          u[i] = a[k0 + i];
+#pragma unroll
+          for (int j = 0; j < LU_NB; ++j)
+            if (j < i) u[i] = csub_mul(u[i], A[(size_t)(k0 + j) * n + k0 + i], u[j]);
+          a[k0 + i] = u[i];
+        }
+        U[i][t] = u[i];
+      }
+    }
+  }
+  if (c0 + nc <= k0) return;   // wholly left of the panel: interchanges only
   __syncthreads();
-  const double2 d = colk[k];
-  const double dd = d.x * d.x + d.y * d.y;
-  if (dd > 0.0) {
-    const double ir = d.x / dd, ii = -d.y / dd;   // 1 / d
-    for (int i = k + 1 + t; i < n; i += blockDim.x) {
-      const double2 a = colk[i];
-      colk[i] = make_double2(a.x * ir - a.y * ii, a.x * ii + a.y * ir);
+  for (int i = k0 + nb + t; i < n; i += 256) {
+    double2 l[LU_NB];
+#pragma unroll
+    for (int j = 0; j < LU_NB; ++j) l[j] = j < nb ? A[(size_t)(k0 + j) * n + i] : make_double2(0.0, 0.0);
+    for (int c = max(0, k0 - c0); c < nc; ++c) {
+      double2* a = col(c) + i;
+      double2 v = *a;
+#pragma unroll
+      for (int j = 0; j < LU_NB; ++j)
+        if (j < nb) v = csub_mul(v, l[j], U[j][c]);
+      *a = v;
     }
   }
 }
 
-// Trailing update of step k: A_ij -= A_ik A_kj for i, j > k (column
-// j = k + 1 + blockIdx.y).
-__global__ void lu_update_kernel(double2* __restrict__ A, int n, int k) {
-  const int j = k + 1 + blockIdx.y;
-  const double2* colk = A + (size_t)k * n;
-  double2* colj = A + (size_t)j * n;
-  const double2 akj = colj[k];
-  for (int i = k + 1 + blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const double2 l = colk[i];
-    double2 a = colj[i];
-    a.x = fma(-l.x, akj.x, fma(l.y, akj.y, a.x));
-    a.y = fma(-l.x, akj.y, fma(-l.y, akj.x, a.y));
-    colj[i] = a;
+// D[(2 b + up) SB^2 + c SB + r] = entry (r, c) of the inverse of diagonal
+// block b's unit lower (up = 0) or upper triangle.  One warp per (b, up), lane = column.
+__global__ void __launch_bounds__(32) lu_diag_kernel(const double2* __restrict__ A, int n, double2* __restrict__ D) {
+  __shared__ double2 T[LU_SB][LU_SB];
+  const int b0 = (blockIdx.x >> 1) * LU_SB, up = blockIdx.x & 1, nb = min(LU_SB, n - b0), c = threadIdx.x;
+  for (int e = c; e < nb * nb; e += 32) T[e % nb][e / nb] = A[(size_t)(b0 + e / nb) * n + b0 + e % nb];
+  __syncwarp();
+  if (c >= LU_SB) return;
+  double2* d = D + (size_t)blockIdx.x * LU_SB * LU_SB + c * LU_SB;
+  double2 x[LU_SB];
+#pragma unroll
+  for (int k = 0; k < LU_SB; ++k) x[k] = make_double2(k == c && c < nb ? 1.0 : 0.0, 0.0);
+  if (!up) {
+#pragma unroll
+    for (int i = 0; i < LU_SB; ++i)
+#pragma unroll
+      for (int j = 0; j < LU_SB; ++j)
+        if (j < i && i < nb) x[i] = csub_mul(x[i], T[i][j], x[j]);
+  } else {
+#pragma unroll
+    for (int i = LU_SB - 1; i >= 0; --i) {
+      if (i < nb) {
+#pragma unroll
+        for (int j = 0; j < LU_SB; ++j)
+          if (j > i && j < nb) x[i] = csub_mul(x[i], T[i][j], x[j]);
+        const double2 q = T[i][i], v = x[i];
+        const double dd = q.x * q.x + q.y * q.y;
+        x[i] = make_double2((v.x * q.x + v.y * q.y) / dd, (v.y * q.x - v.x * q.y) / dd);
+      }
+    }
   }
+#pragma unroll
+  for (int k = 0; k < LU_SB; ++k) d[k] = x[k];
 }
 
-// y <- A^{-1} y with the factors of lu_pivot_kernel / lu_update_kernel: the
-// row interchanges in order, then the unit lower and the upper triangular
-// substitutions.  One CTA per column of Y (leading dimension ldy).
-__global__ void __launch_bounds__(256) lu_solve_kernel(const double2* __restrict__ A, const int* __restrict__ piv,
-                                                       int n, double2* __restrict__ Y, long long ldy) {
-  double2* y = Y + (size_t)blockIdx.x * ldy;
+// Y <- A^{-1} Y with those factors and diagonal inverses, a CTA per strip of
+// CS columns of Y (leading dimension n): the interchanges, then the unit
+// lower and the upper triangular substitutions by blocks of LU_SB rows.
+template <int CS>
+__global__ void __launch_bounds__(256) lu_solve_kernel(const double2* __restrict__ A, const double2* __restrict__ D,
+                                                       const int* __restrict__ piv, int n, double2* __restrict__ Y) {
+  __shared__ double2 B[LU_SB][CS];
+  __shared__ double2 X[LU_SB][CS];
   const int t = threadIdx.x;
-  if (t == 0)
+  const int c0 = blockIdx.x * CS, nc = min(CS, n - c0);
+  if (t < nc) {
+    double2* y = Y + (size_t)(c0 + t) * n;
     for (int k = 0; k < n; ++k) {
       const int p = piv[k];
       if (p != k) {
@@ -290,34 +473,36 @@ __global__ void __launch_bounds__(256) lu_solve_kernel(const double2* __restrict
         y[p] = a;
       }
     }
-  __syncthreads();
-  for (int k = 0; k < n; ++k) {
-    const double2 yk = y[k];
-    const double2* colk = A + (size_t)k * n;
-    for (int i = k + 1 + t; i < n; i += blockDim.x) {
-      const double2 l = colk[i];
-      double2 v = y[i];
-      v.x = fma(-l.x, yk.x, fma(l.y, yk.y, v.x));
-      v.y = fma(-l.x, yk.y, fma(-l.y, yk.x, v.y));
-      y[i] = v;
-    }
-    __syncthreads();
   }
-  for (int k = n - 1; k >= 0; --k) {
-    const double2* colk = A + (size_t)k * n;
-    if (t == 0) {
-      const double2 d = colk[k], v = y[k];
-      const double dd = d.x * d.x + d.y * d.y;
-      y[k] = make_double2((v.x * d.x + v.y * d.y) / dd, (v.y * d.x - v.x * d.y) / dd);
+  __syncthreads();
+  const int blocks = (n + LU_SB - 1) / LU_SB;
+  for (int s = 0; s < 2 * blocks; ++s) {
+    const bool upper = s >= blocks;
+    const int bk = upper ? 2 * blocks - 1 - s : s, b0 = LU_SB * bk, nb = min(LU_SB, n - b0);
+    const int r = t % LU_SB, c = t / LU_SB;   // entry of the block's solution
+    if (c < CS) B[r][c] = (c < nc && r < nb) ? Y[(size_t)(c0 + c) * n + b0 + r] : make_double2(0.0, 0.0);
+    __syncthreads();
+    if (c < CS) {
+      const double2* d = D + (size_t)(2 * bk + (upper ? 1 : 0)) * LU_SB * LU_SB + r;
+      double2 v = make_double2(0.0, 0.0);
+#pragma unroll
+      for (int j = 0; j < LU_SB; ++j) v = csub_mul(v, d[j * LU_SB], make_double2(-B[j][c].x, -B[j][c].y));
+      X[r][c] = v;
+      if (c < nc && r < nb) Y[(size_t)(c0 + c) * n + b0 + r] = v;
     }
     __syncthreads();
-    const double2 yk = y[k];
-    for (int i = t; i < k; i += blockDim.x) {
-      const double2 u = colk[i];
-      double2 v = y[i];
-      v.x = fma(-u.x, yk.x, fma(u.y, yk.y, v.x));
-      v.y = fma(-u.x, yk.y, fma(-u.y, yk.x, v.y));
-      y[i] = v;
+    const int i0 = upper ? 0 : b0 + nb, i1 = upper ? b0 : n;
+    for (int i = i0 + t; i < i1; i += 256) {
+      double2 l[LU_SB];
+#pragma unroll
+      for (int j = 0; j < LU_SB; ++j) l[j] = j < nb ? A[(size_t)(b0 + j) * n + i] : make_double2(0.0, 0.0);
+      for (int q = 0; q < nc; ++q) {
+        double2* y = Y + (size_t)(c0 + q) * n + i;
+        double2 v = *y;
+#pragma unroll
+        for (int j = 0; j < LU_SB; ++j) v = csub_mul(v, l[j], X[j][q]);
+        *y = v;
+      }
     }
     __syncthreads();
   }
@@ -328,35 +513,6 @@ __global__ void identity_kernel(double2* __restrict__ A, long long n) {
   for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < n * n;
        idx += (long long)gridDim.x * blockDim.x)
     A[idx] = make_double2(idx % n == idx / n ? 1.0 : 0.0, 0.0);
-}
-
-// Y[:, r] (= or +=) alpha A X[:, r] for r < R; A column-major m x k, X with
-// leading dimension ldx, Y with ldy.  One thread per output (row fastest).
-__global__ void cgemm_kernel(const double2* __restrict__ A, long long m, long long k, const double2* __restrict__ X,
-                             long long ldx, double2* __restrict__ Y, long long ldy, int R, double alpha,
-                             int accumulate) {
-  const long long total = m * R;
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const long long i = idx % m;
-    const int r = (int)(idx / m);
-    const double2* x = X + (size_t)r * ldx;
-    double re = 0.0, im = 0.0;
-    for (long long j = 0; j < k; ++j) {
-      const double2 a = A[(size_t)j * m + i];
-      const double2 v = x[j];
-      re = fma(a.x, v.x, fma(-a.y, v.y, re));
-      im = fma(a.x, v.y, fma(a.y, v.x, im));
-    }
-    double2* y = Y + (size_t)r * ldy + i;
-    re *= alpha;
-    im *= alpha;
-    if (accumulate) {
-      re += y->x;
-      im += y->y;
-    }
-    *y = make_double2(re, im);
-  }
 }
 
 PointTables point_tables(const hb_ctx* c) {
@@ -370,20 +526,31 @@ PointTables point_tables(const hb_ctx* c) {
 }
 
 // The three surface operators into column-major outputs (any may be null).
-void assemble(const hb_ctx* c, const double2* seg, const double* w, const double* nseg, long long ns,
-              const double2* cells, double2* k_s2s, double2* k_v2s, double2* k_s2v, cudaStream_t st) {
-  const PointTables P = point_tables(c);
+void assemble(const hb_ctx* c, double2* k_s2s, double2* k_v2s, double2* k_s2v, cudaStream_t st) {
+  const EntryParams E = entry_params(c, 0);
+  const long long ns = c->ns_set;
+  const double* G0 = c->d_segG;
+  const double* G1 = c->d_segG + (size_t)3 * c->NI * ns;
+  // lines cut so that a small curve still fills the chip (about 8 warps an SM)
+  const long long warps = (ns + 31) / 32 * c->ny;
+  const unsigned cut = (unsigned)std::max<long long>(1, std::min<long long>((1216 + warps - 1) / warps, (c->nx + 15) / 16));
+  auto lines = [&](int b0) { return dim3((unsigned)((ns + 63) / 64), (unsigned)std::min(65535, c->ny - b0), cut); };
   if (k_s2s) {
-    green_columns_kernel<<<(unsigned)ns, 256, 0, st>>>(P, seg, ns, seg, w, nseg, -1.0, 1, k_s2s, ns);
+    seg_seg_kernel<<<dim3((unsigned)((ns + 127) / 128), (unsigned)ns), 128, 0, st>>>(E, c->d_seglag, G0, ns, c->d_segw,
+                                                                                    c->d_segn, k_s2s);
     HB_CHECK_LAUNCH();
   }
   if (k_v2s) {
-    green_columns_kernel<<<(unsigned)c->Nv, 256, 0, st>>>(P, seg, ns, cells, nullptr, nullptr, 1.0, 0, k_v2s, ns);
-    HB_CHECK_LAUNCH();
+    for (int b0 = 0; b0 < c->ny; b0 += 65535) {
+      seg_line_kernel<true><<<lines(b0), 64, 0, st>>>(E, G1, ns, c->d_segw, b0, k_v2s);
+      HB_CHECK_LAUNCH();
+    }
   }
   if (k_s2v) {
-    green_columns_kernel<<<(unsigned)ns, 256, 0, st>>>(P, cells, c->Nv, seg, w, nullptr, 1.0, 0, k_s2v, c->Nv);
-    HB_CHECK_LAUNCH();
+    for (int b0 = 0; b0 < c->ny; b0 += 65535) {
+      seg_line_kernel<false><<<lines(b0), 64, 0, st>>>(E, G0, ns, c->d_segw, b0, k_s2v);
+      HB_CHECK_LAUNCH();
+    }
   }
 }
 
@@ -400,13 +567,20 @@ void green_jobs(const hb_ctx* c, const double2* d_obs, const GreenCol* d_jobs, l
 }
 
 void curve_free(hb_ctx* c) {
-  for (void* p : {(void*)c->d_seg, (void*)c->d_segw, (void*)c->d_segn, (void*)c->d_cellpts, (void*)c->d_lu,
-                  (void*)c->d_piv, (void*)c->d_kv2s, (void*)c->d_ks2v, (void*)c->d_cy, (void*)c->d_inv})
+  for (void* p : {(void*)c->d_seg, (void*)c->d_segw, (void*)c->d_segn, (void*)c->d_lu, (void*)c->d_piv,
+                  (void*)c->d_kv2s, (void*)c->d_ks2v, (void*)c->d_cy, (void*)c->d_inv, (void*)c->d_seglag,
+                  (void*)c->d_segG, (void*)c->d_pack})
     dev_free(p);
+  dense_op_free(c->op_v2s);
+  dense_op_free(c->op_inv);
+  dense_op_free(c->op_s2v);
+  c->d_seglag = c->d_segG = nullptr;
+  c->d_pack = nullptr;
+  c->ns_set = 0;
   c->d_inv = nullptr;
   c->d_seg = nullptr;
   c->d_segw = c->d_segn = nullptr;
-  c->d_cellpts = c->d_lu = c->d_kv2s = c->d_ks2v = c->d_cy = nullptr;
+  c->d_lu = c->d_kv2s = c->d_ks2v = c->d_cy = nullptr;
   c->d_piv = nullptr;
   c->ns = 0;
   c->cy_cap = 0;
@@ -429,9 +603,13 @@ void curve_set(hb_ctx* c, const double* centers, const double* lengths, const do
     c->d_seg = upload(cen);
     c->d_segw = upload(std::vector<double>(lengths, lengths + ns));
     c->d_segn = upload(std::vector<double>(n_seg, n_seg + ns));
-    c->d_cellpts = dev_alloc<double2>((size_t)c->Nv);
-    cell_points_kernel<<<(unsigned)std::min<long long>((c->Nv + 255) / 256, 152LL * 8), 256>>>(
-        c->nx, c->Nv, c->x0, c->y0, c->h, c->d_cellpts);
+    c->ns_set = ns;
+    c->d_seglag = dev_alloc<double>((size_t)ns * 32);
+    c->d_segG = dev_alloc<double>((size_t)6 * c->NI * ns);
+    const PointTables P = point_tables(c);
+    seg_basis_kernel<<<(unsigned)((2 * ns + 127) / 128), 128>>>(P, c->d_seg, ns, c->d_seglag);
+    HB_CHECK_LAUNCH();
+    seg_contract_kernel<<<dim3((unsigned)((ns + 127) / 128), (unsigned)(6 * c->NI)), 128>>>(P, c->d_seglag, ns, c->d_segG);
     HB_CHECK_LAUNCH();
     c->d_lu = dev_alloc<double2>((size_t)ns * ns);
     c->d_piv = dev_alloc<int>((size_t)ns);
@@ -440,14 +618,15 @@ void curve_set(hb_ctx* c, const double* centers, const double* lengths, const do
     std::vector<int> zero(1, 0);
     int* d_sing = upload(zero);
     try {
-      assemble(c, c->d_seg, c->d_segw, c->d_segn, ns, c->d_cellpts, c->d_lu, c->d_kv2s, c->d_ks2v, 0);
+      assemble(c, c->d_lu, c->d_kv2s, c->d_ks2v, 0);
       const int n = (int)ns;
-      for (int k = 0; k < n; ++k) {
-        lu_pivot_kernel<<<1, 256>>>(c->d_lu, n, k, c->d_piv, d_sing);
+      for (int k = 0; k < n; k += LU_NB) {
+        lu_panel_kernel<<<1, LU_PT>>>(c->d_lu, n, k, c->d_piv, d_sing);
         HB_CHECK_LAUNCH();
-        if (k + 1 < n) {
-          dim3 grid((unsigned)std::min((n - k - 1 + 255) / 256, 4), (unsigned)(n - k - 1));
-          lu_update_kernel<<<grid, 256>>>(c->d_lu, n, k);
+        const int others = n - std::min(LU_NB, n - k);
+        if (others > 0) {
+          if (lu_strip(n) == 2) lu_strip_kernel<2><<<(unsigned)((others + 1) / 2), 256>>>(c->d_lu, n, k, c->d_piv);
+          else lu_strip_kernel<8><<<(unsigned)((others + 7) / 8), 256>>>(c->d_lu, n, k, c->d_piv);
           HB_CHECK_LAUNCH();
         }
       }
@@ -460,9 +639,22 @@ void curve_set(hb_ctx* c, const double* centers, const double* lengths, const do
       c->d_inv = dev_alloc<double2>((size_t)ns * ns);
       identity_kernel<<<(unsigned)std::min<long long>((ns * ns + 255) / 256, 152LL * 8), 256>>>(c->d_inv, ns);
       HB_CHECK_LAUNCH();
-      lu_solve_kernel<<<(unsigned)ns, 256>>>(c->d_lu, c->d_piv, n, c->d_inv, ns);
-      HB_CHECK_LAUNCH();
-      HB_CUDA(cudaDeviceSynchronize());
+      const int diag = 2 * ((n + LU_SB - 1) / LU_SB);
+      double2* d_diag = dev_alloc<double2>((size_t)diag * LU_SB * LU_SB);
+      lu_diag_kernel<<<(unsigned)diag, 32>>>(c->d_lu, n, d_diag);
+      if (lu_strip(n) == 2) lu_solve_kernel<2><<<(unsigned)((n + 1) / 2), 256>>>(c->d_lu, d_diag, c->d_piv, n, c->d_inv);
+      else lu_solve_kernel<8><<<(unsigned)((n + 7) / 8), 256>>>(c->d_lu, d_diag, c->d_piv, n, c->d_inv);
+      const cudaError_t le = cudaGetLastError(), se = cudaDeviceSynchronize();
+      dev_free(d_diag);
+      HB_CUDA(le);
+      HB_CUDA(se);
+      c->op_v2s = dense_op(c->d_kv2s, ns, c->Nv, 0);
+      c->op_inv = dense_op(c->d_inv, ns, ns, 0);
+      c->op_s2v = dense_op(c->d_ks2v, c->Nv, ns, 0);
+      size_t rows = 0;
+      for (const DenseOp* D : {&c->op_v2s, &c->op_inv, &c->op_s2v})
+        rows = std::max<size_t>(rows, (size_t)D->k + (size_t)D->ntask * (size_t)D->m);
+      c->d_pack = dev_alloc<double2>(rows * 16);
     } catch (...) {
       cudaDeviceSynchronize();
       dev_free(d_sing);
@@ -478,7 +670,7 @@ void curve_set(hb_ctx* c, const double* centers, const double* lengths, const do
 
 void curve_operators(hb_ctx* c, double2* k_s2s, double2* k_v2s, double2* k_s2v, cudaStream_t st) {
   if (c->ns == 0) throw Error{HB_ERR_STATE, "no curve set (hb_curve_set)"};
-  assemble(c, c->d_seg, c->d_segw, c->d_segn, c->ns, c->d_cellpts, k_s2s, k_v2s, k_s2v, st);
+  assemble(c, k_s2s, k_v2s, k_s2v, st);
 }
 
 void apply_inclusion(hb_ctx* c, const double2* s, double2* u, int nrhs, int v2v_dense, cudaStream_t st) {
@@ -497,26 +689,22 @@ void apply_inclusion(hb_ctx* c, const double2* s, double2* u, int nrhs, int v2v_
   if (v2v_dense) dense_apply(c, s, u, nrhs, 0, st);
   else apply_bf(c, s, u, nrhs, 0, c->opt.precision, st);
   const long long ns = c->ns;
-  auto grid = [](long long total) { return (unsigned)std::max<long long>(1, std::min<long long>((total + 255) / 256, 152LL * 8)); };
+  auto product = [&](const DenseOp& D, const double2* X, long long ldx, double2* Y, long long ldy, double alpha,
+                     int accumulate) {   // 16 columns at a time
+    for (int r0 = 0; r0 < nrhs; r0 += 16)
+      dense_product(D, X + (size_t)r0 * ldx, ldx, Y + (size_t)r0 * ldy, ldy, std::min(16, nrhs - r0), alpha, accumulate,
+                    c->d_pack, c->d_pack + (size_t)D.k * 16, st);
+  };
   const bool compressed = c->curve_bf[0] && c->curve_bf[1];
   // Y = K^{v2s} I = h^2 K^{v2s} s
-  if (compressed) {
-    curve_bf_apply(c, 0, s, c->Nv, c->h * c->h, c->d_cy, ns, 0, nrhs, st);
-  } else {
-    cgemm_kernel<<<grid(ns * nrhs), 256, 0, st>>>(c->d_kv2s, ns, c->Nv, s, c->Nv, c->d_cy, ns, nrhs, c->h * c->h, 0);
-    HB_CHECK_LAUNCH();
-  }
+  if (compressed) curve_bf_apply(c, 0, s, c->Nv, c->h * c->h, c->d_cy, ns, 0, nrhs, st);
+  else product(c->op_v2s, s, c->Nv, c->d_cy, ns, c->h * c->h, 0);
   // P = (K^{s2s})^{-1} Y
   double2* P = c->d_cy + (size_t)ns * nrhs;
-  cgemm_kernel<<<grid(ns * nrhs), 256, 0, st>>>(c->d_inv, ns, ns, c->d_cy, ns, P, ns, nrhs, 1.0, 0);
-  HB_CHECK_LAUNCH();
+  product(c->op_inv, c->d_cy, ns, P, ns, 1.0, 0);
   // U += K^{s2v} P
-  if (compressed) {
-    curve_bf_apply(c, 1, P, ns, 1.0, u, c->Nv, 1, nrhs, st);
-  } else {
-    cgemm_kernel<<<grid(c->Nv * nrhs), 256, 0, st>>>(c->d_ks2v, c->Nv, ns, P, ns, u, c->Nv, nrhs, 1.0, 1);
-    HB_CHECK_LAUNCH();
-  }
+  if (compressed) curve_bf_apply(c, 1, P, ns, 1.0, u, c->Nv, 1, nrhs, st);
+  else product(c->op_s2v, P, ns, u, c->Nv, 1.0, 1);
 }
 
 }  // namespace hb
