@@ -453,30 +453,32 @@ __global__ void __launch_bounds__(32) lu_diag_kernel(const double2* __restrict__
   for (int k = 0; k < LU_SB; ++k) d[k] = x[k];
 }
 
-// Y <- A^{-1} Y with those factors and diagonal inverses, a CTA per strip of
-// CS columns of Y (leading dimension n): the interchanges, then the unit
-// lower and the upper triangular substitutions by blocks of LU_SB rows.
+// Y = A^{-1} (Y zero before) with those factors and diagonal inverses, a CTA
+// per strip of CS columns of Y (leading dimension n): the unit columns through
+// the interchanges, then the unit lower (from the first non-zero block on) and
+// the upper triangular substitutions by blocks of LU_SB rows.
 template <int CS>
-__global__ void __launch_bounds__(256) lu_solve_kernel(const double2* __restrict__ A, const double2* __restrict__ D,
+__global__ void __launch_bounds__(256) lu_inverse_kernel(const double2* __restrict__ A, const double2* __restrict__ D,
                                                        const int* __restrict__ piv, int n, double2* __restrict__ Y) {
   __shared__ double2 B[LU_SB][CS];
   __shared__ double2 X[LU_SB][CS];
   const int t = threadIdx.x;
+  __shared__ int first;
   const int c0 = blockIdx.x * CS, nc = min(CS, n - c0);
+  if (t == 0) first = n;
+  __syncthreads();
   if (t < nc) {
-    double2* y = Y + (size_t)(c0 + t) * n;
+    int r = c0 + t;
     for (int k = 0; k < n; ++k) {
       const int p = piv[k];
-      if (p != k) {
-        const double2 a = y[k];
-        y[k] = y[p];
-        y[p] = a;
-      }
+      r = r == k ? p : r == p ? k : r;
     }
+    Y[(size_t)(c0 + t) * n + r] = make_double2(1.0, 0.0);
+    atomicMin(&first, r);
   }
   __syncthreads();
   const int blocks = (n + LU_SB - 1) / LU_SB;
-  for (int s = 0; s < 2 * blocks; ++s) {
+  for (int s = first / LU_SB; s < 2 * blocks; ++s) {
     const bool upper = s >= blocks;
     const int bk = upper ? 2 * blocks - 1 - s : s, b0 = LU_SB * bk, nb = min(LU_SB, n - b0);
     const int r = t % LU_SB, c = t / LU_SB;   // entry of the block's solution
@@ -506,13 +508,6 @@ __global__ void __launch_bounds__(256) lu_solve_kernel(const double2* __restrict
     }
     __syncthreads();
   }
-}
-
-// A = the n x n identity (column-major)
-__global__ void identity_kernel(double2* __restrict__ A, long long n) {
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < n * n;
-       idx += (long long)gridDim.x * blockDim.x)
-    A[idx] = make_double2(idx % n == idx / n ? 1.0 : 0.0, 0.0);
 }
 
 PointTables point_tables(const hb_ctx* c) {
@@ -637,13 +632,12 @@ void curve_set(hb_ctx* c, const double* centers, const double* lengths, const do
       // the inverse, column by column from the factors (an apply is then one
       // product instead of two sequential triangular solves per column)
       c->d_inv = dev_alloc<double2>((size_t)ns * ns);
-      identity_kernel<<<(unsigned)std::min<long long>((ns * ns + 255) / 256, 152LL * 8), 256>>>(c->d_inv, ns);
-      HB_CHECK_LAUNCH();
+      HB_CUDA(cudaMemsetAsync(c->d_inv, 0, sizeof(double2) * (size_t)ns * ns));
       const int diag = 2 * ((n + LU_SB - 1) / LU_SB);
       double2* d_diag = dev_alloc<double2>((size_t)diag * LU_SB * LU_SB);
       lu_diag_kernel<<<(unsigned)diag, 32>>>(c->d_lu, n, d_diag);
-      if (lu_strip(n) == 2) lu_solve_kernel<2><<<(unsigned)((n + 1) / 2), 256>>>(c->d_lu, d_diag, c->d_piv, n, c->d_inv);
-      else lu_solve_kernel<8><<<(unsigned)((n + 7) / 8), 256>>>(c->d_lu, d_diag, c->d_piv, n, c->d_inv);
+      if (lu_strip(n) == 2) lu_inverse_kernel<2><<<(unsigned)((n + 1) / 2), 256>>>(c->d_lu, d_diag, c->d_piv, n, c->d_inv);
+      else lu_inverse_kernel<8><<<(unsigned)((n + 7) / 8), 256>>>(c->d_lu, d_diag, c->d_piv, n, c->d_inv);
       const cudaError_t le = cudaGetLastError(), se = cudaDeviceSynchronize();
       dev_free(d_diag);
       HB_CUDA(le);
