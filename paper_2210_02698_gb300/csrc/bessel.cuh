@@ -51,8 +51,106 @@ HB_HD void hb_sincos(double x, double* s, double* c) {
 #endif
 }
 
+#ifdef __CUDACC__
+// ---- division by a known number ----
+// t / k from y = 1 / k (rounded to nearest): q = t y, q + (t - k q) y is the
+// correctly rounded quotient (Markstein, IBM J. Res. Dev. 34 (1990)), bit for
+// bit what the division gives, in 3 FP64 instructions instead of about 12
+// (t within 2^-900 .. 2^1000).  The unit does 2 FMAs a cycle and SM.
+__device__ __forceinline__ double div_by(double t, double k, double y) {
+  const double q = __dmul_rn(t, y);
+  return __fma_rn(__fma_rn(-k, q, t), y, q);
+}
+
+// k, 1 / k, (2k - 1) / (k (k - 1)), -(2k - 1)^2 and 4 - (2k - 1)^2, k <= 66
+// (an int to double conversion is an instruction of the FP64 unit too)
+constexpr int BESSEL_K = 67;
+struct BesselConsts {
+  double dk[BESSEL_K], rk[BESSEL_K], ck[BESSEL_K], a0[BESSEL_K], a1[BESSEL_K];
+};
+constexpr BesselConsts bessel_consts() {
+  BesselConsts c{};
+  for (int k = 1; k < BESSEL_K; ++k) {
+    c.dk[k] = (double)k;
+    c.a0[k] = -(double)((2 * k - 1) * (2 * k - 1));
+    c.a1[k] = 4.0 - (double)((2 * k - 1) * (2 * k - 1));
+    c.rk[k] = 1.0 / (double)k;
+    c.ck[k] = k > 1 ? (double)(2 * k - 1) / ((double)k * (double)(k - 1)) : 0.0;
+  }
+  return c;
+}
+static __constant__ BesselConsts g_bessel = bessel_consts();
+
+// The device forms of the two branches below: the same operations on the same
+// values (their results are the same bits), with the order index uniform over
+// the warp (constants, no conversions), divisions by small integers as
+// above and no FP64 comparisons.
+
+// Lanes start at their own M: before it their sums stay zero.
+__device__ __forceinline__ Bessel01 bessel01_miller_dev(double x) {
+  const int M = 2 * (int)(0.8 * x + 13.0);
+  const int top = __reduce_max_sync(__activemask(), M);
+  const double two_over_x = 2.0 / x;
+  double tp1 = 0.0, t = 0.0, norm = 0.0, sy0 = 0.0, sy1 = 0.0, t1 = 0.0;
+  const long long big = __double_as_longlong(1e250);
+  auto step = [&](int n) {
+    const double tm1 = __fma_rn(__dmul_rn(g_bessel.dk[n], two_over_x), t, -tp1);
+    tp1 = t;
+    t = tm1;
+    if ((__double_as_longlong(t) & 0x7fffffffffffffffLL) > big) {
+      t *= 1e-250; tp1 *= 1e-250; norm *= 1e-250; sy0 *= 1e-250; sy1 *= 1e-250; t1 *= 1e-250;
+    }
+  };
+#pragma unroll 1
+  for (int k = top >> 1; k >= 1; --k) {
+    // order 2k
+    if (2 * k == M) t = 1e-30;
+    norm = __fma_rn(2.0, t, norm);
+    const double q = div_by(t, g_bessel.dk[k], g_bessel.rk[k]);
+    sy0 = __dadd_rn(sy0, (k & 1) ? -q : q);
+    step(2 * k);
+    // order 2k - 1
+    if (k >= 2) sy1 = __fma_rn((k & 1) ? -g_bessel.ck[k] : g_bessel.ck[k], t, sy1);
+    else t1 = t;
+    step(2 * k - 1);
+  }
+  norm += t;
+  const double sc = 1.0 / norm;
+  Bessel01 r;
+  r.j0 = t * sc;
+  r.j1 = t1 * sc;
+  const double lg = log(0.5 * x) + HB_EULER_GAMMA;
+  r.y0 = (2.0 / HB_PI) * (lg * r.j0 - 2.0 * sy0 * sc);
+  r.y1 = (2.0 / HB_PI) * ((lg - 1.0) * r.j1 - r.j0 / x + sy1 * sc);
+  return r;
+}
+
+__device__ __forceinline__ void bessel01_asym_sums(double x, double& P0, double& Q0, double& P1, double& Q1) {
+  const double inv8x = 0.125 / x;
+  double b0 = 1.0, b1 = 1.0;
+  P0 = P1 = 1.0;
+  Q0 = Q1 = 0.0;
+  const long long tiny = __double_as_longlong(1e-17);
+#pragma unroll 1
+  for (int k = 1; k < 60; ++k) {
+    const double f = div_by(inv8x, g_bessel.dk[k], g_bessel.rk[k]);
+    b0 = __dmul_rn(b0, __dmul_rn(g_bessel.a0[k], f));
+    b1 = __dmul_rn(b1, __dmul_rn(g_bessel.a1[k], f));
+    const bool neg = (k >> 1) & 1;
+    const double s0 = neg ? -b0 : b0, s1 = neg ? -b1 : b1;
+    if (k & 1) { Q0 = __dadd_rn(Q0, s0); Q1 = __dadd_rn(Q1, s1); }
+    else       { P0 = __dadd_rn(P0, s0); P1 = __dadd_rn(P1, s1); }
+    if ((__double_as_longlong(b0) & 0x7fffffffffffffffLL) < tiny &&
+        (__double_as_longlong(b1) & 0x7fffffffffffffffLL) < tiny) break;
+  }
+}
+#endif
+
 // Miller + Neumann branch, 0 < x < HB_BESSEL_SWITCH.
 HB_HD Bessel01 bessel01_miller(double x) {
+#ifdef __CUDA_ARCH__
+  return bessel01_miller_dev(x);
+#else
   const int M = 2 * (int)(0.8 * x + 13.0);          // even start order >= 26
   const double two_over_x = 2.0 / x;
   double tp1 = 0.0, t = 1e-30;                       // t_{n+1}, t_n at n = M
@@ -87,13 +185,17 @@ HB_HD Bessel01 bessel01_miller(double x) {
   r.y0 = (2.0 / HB_PI) * (lg * r.j0 - 2.0 * sy0 * sc);
   r.y1 = (2.0 / HB_PI) * ((lg - 1.0) * r.j1 - r.j0 / x + sy1 * sc);
   return r;
+#endif
 }
 
 // Hankel asymptotic branch, x >= HB_BESSEL_SWITCH.
 HB_HD Bessel01 bessel01_asym(double x) {
+  double P0 = 1.0, Q0 = 0.0, P1 = 1.0, Q1 = 0.0;
+#ifdef __CUDA_ARCH__
+  bessel01_asym_sums(x, P0, Q0, P1, Q1);
+#else
   const double inv8x = 0.125 / x;
   double b0 = 1.0, b1 = 1.0;                          // running a_k(nu) / x^k
-  double P0 = 1.0, Q0 = 0.0, P1 = 1.0, Q1 = 0.0;
   for (int k = 1; k < 60; ++k) {
     const double odd = (double)(2 * k - 1);
     const double f = inv8x / (double)k;
@@ -105,6 +207,7 @@ HB_HD Bessel01 bessel01_asym(double x) {
     else       { P0 += sg * b0; P1 += sg * b1; }
     if (fabs(b0) < 1e-17 && fabs(b1) < 1e-17) break;
   }
+#endif
   double s, c;
   hb_sincos(x, &s, &c);
   const double amp = sqrt(2.0 / (HB_PI * x));
@@ -124,14 +227,21 @@ HB_HD Bessel01 bessel01(double x) {
 
 #ifdef __CUDACC__
 // g = v0 f0 + v1 f1 from interpolated tau^2, v0, v1 (Eq. babich, Eq. termf).
-__device__ __forceinline__ double2 hb_green(double t2, double v0, double v1, double omega) {
-  const double tau = sqrt(fmax(t2, 0.0));
+__device__ __forceinline__ double2 hb_green(double t2, double v0, double v1, double omega);
+// whether hb_green takes the asymptotic branch (for grouping its calls by branch)
+__device__ __forceinline__ bool hb_green_far(double tau, double omega) {
+  return !(fmax(omega * tau, 1e-12) < HB_BESSEL_SWITCH);
+}
+__device__ __forceinline__ double2 hb_green_tau(double tau, double v0, double v1, double omega) {
   const double x = fmax(omega * tau, 1e-12);
   const Bessel01 b = bessel01(x);
   const double c = 0.88622692545275801365;         // sqrt(pi)/2
   const double k1 = c * 2.0 * tau / omega;
   // f0 = c(-Y0 + i J0),  f1 = k1 (Y1 - i J1)
   return make_double2(-c * b.y0 * v0 + k1 * b.y1 * v1, c * b.j0 * v0 - k1 * b.j1 * v1);
+}
+__device__ __forceinline__ double2 hb_green(double t2, double v0, double v1, double omega) {
+  return hb_green_tau(sqrt(fmax(t2, 0.0)), v0, v1, omega);
 }
 #endif
 

@@ -73,20 +73,31 @@ __global__ void htable_kernel(const double* __restrict__ F, const double* __rest
 
 // Self term K_ii = (i/4) I / h^2, I = (n0 w)^-2 [8 int_0^{pi/4} R H1(R) dth + 4i],
 // R = h n0 w / (2 cos th)  (Appendix A); theta quadrature: Gauss-Legendre.
-__global__ void self_kernel(const double* __restrict__ ncell, long long Nv, double h, double omega,
-                            const double* __restrict__ glx, const double* __restrict__ glw, int ngl,
-                            double2* __restrict__ out) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= Nv) return;
-  double n0 = ncell[i];
-  double k = 0.5 * h * n0 * omega;
+// A CTA takes SELF_CELLS cells: its threads evaluate the points of the rule, then
+// one thread per cell adds them in order (one thread per cell throughout left
+// most SMs without work on small grids).
+constexpr int SELF_NGL = 64, SELF_CELLS = 4;
+__global__ void __launch_bounds__(SELF_NGL * SELF_CELLS) self_kernel(const double* __restrict__ ncell, long long Nv, double h,
+                                                                     double omega, const double* __restrict__ glx,
+                                                                     const double* __restrict__ glw,
+                                                                     double2* __restrict__ out) {
+  __shared__ double2 val[SELF_CELLS][SELF_NGL];   // R J1(R), R Y1(R)
+  const int cell = threadIdx.x / SELF_NGL, g = threadIdx.x % SELF_NGL;
+  const long long i = (long long)blockIdx.x * SELF_CELLS + cell;
+  const double n0 = ncell[i < Nv ? i : Nv - 1];
+  {
+    const double k = 0.5 * h * n0 * omega;
+    const double th = (HB_PI / 8.0) * (glx[g] + 1.0);   // map [-1,1] -> [0, pi/4]
+    const double R = k / cos(th);
+    const Bessel01 b = bessel01(R);
+    val[cell][g] = make_double2(R * b.j1, R * b.y1);
+  }
+  __syncthreads();
+  if (g != 0 || i >= Nv) return;
   double re = 0.0, im = 0.0;
-  for (int g = 0; g < ngl; ++g) {
-    double th = (HB_PI / 8.0) * (glx[g] + 1.0);   // map [-1,1] -> [0, pi/4]
-    double R = k / cos(th);
-    Bessel01 b = bessel01(R);
-    re = fma(glw[g], R * b.j1, re);
-    im = fma(glw[g], R * b.y1, im);
+  for (int q = 0; q < SELF_NGL; ++q) {
+    re = fma(glw[q], val[cell][q].x, re);
+    im = fma(glw[q], val[cell][q].y, im);
   }
   re *= HB_PI / 8.0;
   im *= HB_PI / 8.0;
@@ -180,14 +191,14 @@ void compute_self(hb_ctx* c) {
     c->hank_top = (float)top;
   }
   std::vector<double> glx, glw;
-  gauss_legendre(64, glx, glw);
+  gauss_legendre(SELF_NGL, glx, glw);
   // the quadrature rule is scratch: freed on the way out, also when a step throws
   double* d_gl = upload(glx);
   double* d_gw = nullptr;
   try {
     d_gw = upload(glw);
-    self_kernel<<<(unsigned)((c->Nv + 127) / 128), 128>>>(c->d_ncell, c->Nv, c->h, c->omega, d_gl, d_gw,
-                                                          64, c->d_self);
+    self_kernel<<<(unsigned)((c->Nv + SELF_CELLS - 1) / SELF_CELLS), SELF_NGL * SELF_CELLS>>>(
+        c->d_ncell, c->Nv, c->h, c->omega, d_gl, d_gw, c->d_self);
     HB_CHECK_LAUNCH();
     HB_CUDA(cudaDeviceSynchronize());
   } catch (...) {
@@ -448,14 +459,26 @@ void dense_apply(hb_ctx* c, const double2* s, double2* u, int nrhs, int adjoint,
 // contiguous; seg array (int64 x 3 per segment): b, first row, count.
 // Output: column-major m x n at out_off; row a of the sorted list goes to
 // out row rdst[row_off + a] (identity for the build).
-constexpr int SEGC = 8;   // row lines per pass
+// FP64-bound: a warp's FP64 instruction costs the same with few lanes live or on
+// the other branch, so a pass takes enough lines that its rows fill the
+// threads (with 8 lines it held 40 to 60 rows), and the Hankel pairs are
+// evaluated from lists of the near arguments (recurrence) and the far ones
+// (asymptotic series), a warp all on one branch.  The lists' order does not
+// matter to the values.
+constexpr int SEGC = 32;     // row lines per pass
+constexpr int ECHUNK = 512;  // rows per round of the lists
+constexpr int ETHREADS = 128;
 
-__global__ void __launch_bounds__(128) block_entries_kernel(
+__global__ void __launch_bounds__(ETHREADS) block_entries_kernel(
     EntryParams p, const BlockMeta* __restrict__ meta, const long long* __restrict__ items,
     const long long* __restrict__ rows, const int* __restrict__ rdst, const long long* __restrict__ cols,
     const long long* __restrict__ segs, double2* __restrict__ out) {
   __shared__ double G[3][256];
   __shared__ double P[3][SEGC][MAX_NI];
+  __shared__ int s_line[SEGC], s_first[SEGC];
+  __shared__ double lt[ECHUNK], l0[ECHUNK], l1[ECHUNK];   // near from the front, far from the back
+  __shared__ int lrow[ECHUNK];
+  __shared__ int s_near, s_far;
   const int nI = p.nI, NI = p.NI;
   const long long it = items[blockIdx.x];
   const int b = (int)(it >> 20);
@@ -463,7 +486,7 @@ __global__ void __launch_bounds__(128) block_entries_kernel(
   const BlockMeta bm = meta[b];
   const long long qnat = cols[bm.col_off + jj];
   const int aq = (int)(qnat % p.nx), bq = (int)(qnat / p.nx);
-  const int t = threadIdx.x;
+  const int t = threadIdx.x, lane = t & 31;
   // G[q][i] = sum_j1 H[q][bq][i][j1] LX[aq][j1]
   for (int idx = t; idx < 3 * NI; idx += blockDim.x) {
     int q = idx / NI, i = idx % NI;
@@ -476,33 +499,75 @@ __global__ void __launch_bounds__(128) block_entries_kernel(
   for (int s0 = 0; s0 < bm.nseg; s0 += SEGC) {
     const int ns = (int)min((long long)SEGC, bm.nseg - s0);
     __syncthreads();
+    if (t < ns) {
+      s_line[t] = (int)segs[(bm.seg_off + s0 + t) * 3];
+      s_first[t] = (int)segs[(bm.seg_off + s0 + t) * 3 + 1];
+    }
+    __syncthreads();
     for (int idx = t; idx < 3 * ns * nI; idx += blockDim.x) {
       int q = idx / (ns * nI), sl = (idx / nI) % ns, i1 = idx % nI;
-      int bo = (int)segs[(bm.seg_off + s0 + sl) * 3];
+      int bo = s_line[sl];
       const double* lz = p.LZ + (size_t)bo * nI;
       double a = 0.0;
       for (int i2 = 0; i2 < nI; ++i2) a = fma(lz[i2], G[q][i2 * nI + i1], a);
       P[q][sl][i1] = a;
     }
-    __syncthreads();
     const long long rfirst = segs[(bm.seg_off + s0) * 3 + 1];
     const long long rlast = segs[(bm.seg_off + s0 + ns - 1) * 3 + 1] + segs[(bm.seg_off + s0 + ns - 1) * 3 + 2];
-    for (long long r = rfirst + t; r < rlast; r += blockDim.x) {
-      // locate the segment of row r (ns <= 8, linear scan)
-      int sl = 0;
-      while (sl + 1 < ns && segs[(bm.seg_off + s0 + sl + 1) * 3 + 1] <= r) ++sl;
-      const long long onat = rows[bm.row_off + r];
-      const int ao = (int)(onat % p.nx);
-      const double* lx = p.LX + (size_t)ao * nI;
-      double f[3];
+    for (long long rc = rfirst; rc < rlast; rc += ECHUNK) {
+      __syncthreads();   // P complete, and the lists of the last round read
+      if (t == 0) s_near = s_far = 0;
+      __syncthreads();
+      const int cnt = (int)min((long long)ECHUNK, rlast - rc);
+      for (int r0 = 0; r0 < cnt; r0 += ETHREADS) {
+        const bool live = r0 + t < cnt;
+        const long long r = rc + (live ? r0 + t : 0);
+        // the line of row r: the last one starting at or before it
+        int sl = 0;
 #pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        double a = 0.0;
-        for (int i1 = 0; i1 < nI; ++i1) a = fma(lx[i1], P[q][sl][i1], a);
-        f[q] = a;
+        for (int w = SEGC / 2; w > 0; w >>= 1)
+          if (sl + w < ns && s_first[sl + w] <= r) sl += w;
+        const long long onat = rows[bm.row_off + r];
+        const int ao = (int)(onat % p.nx);
+        const double* lx = p.LX + (size_t)ao * nI;
+        double f[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          double a = 0.0;
+          for (int i1 = 0; i1 < nI; ++i1) a = fma(lx[i1], P[q][sl][i1], a);
+          f[q] = a;
+        }
+        const double tau = sqrt(fmax(f[0], 0.0));
+        const bool self = onat == qnat;
+        if (live && self) out[bm.out_off + (long long)jj * bm.m + rdst[bm.row_off + r]] = p.self[onat];
+        const bool far = hb_green_far(tau, p.omega);
+        const unsigned mn = __ballot_sync(0xffffffffu, live && !self && !far);
+        const unsigned mf = __ballot_sync(0xffffffffu, live && !self && far);
+        int bn = 0, bf = 0;
+        if (lane == 0) {
+          bn = atomicAdd(&s_near, __popc(mn));
+          bf = atomicAdd(&s_far, __popc(mf));
+        }
+        bn = __shfl_sync(0xffffffffu, bn, 0);
+        bf = __shfl_sync(0xffffffffu, bf, 0);
+        if (live && !self) {
+          const unsigned below = (1u << lane) - 1;
+          const int at = far ? ECHUNK - 1 - (bf + __popc(mf & below)) : bn + __popc(mn & below);
+          lt[at] = tau;
+          l0[at] = f[1];
+          l1[at] = f[2];
+          lrow[at] = (int)(r - rc);
+        }
       }
-      double2 g = (onat == qnat) ? p.self[onat] : hb_green(f[0], f[1], f[2], p.omega);
-      out[bm.out_off + (long long)jj * bm.m + rdst[bm.row_off + r]] = g;
+      __syncthreads();
+      // whole warps on one branch: near entries from slot 0, far ones from the next multiple of 32
+      const int nn = s_near, nf = s_far, f0 = (nn + 31) / 32 * 32;
+      for (int e = t; e < f0 + nf; e += ETHREADS) {
+        const int at = e < f0 ? e : ECHUNK - 1 - (e - f0);
+        if (e < f0 && e >= nn) continue;
+        const double2 g = hb_green_tau(lt[at], l0[at], l1[at], p.omega);
+        out[bm.out_off + (long long)jj * bm.m + rdst[bm.row_off + rc + lrow[at]]] = g;
+      }
     }
   }
 }
@@ -572,7 +637,7 @@ void run_blocks(hb_ctx* c, BlockBatchHost& B, double2* d_out, cudaStream_t st) {
   size_t nitems = B.items.size();
   for (size_t i0 = 0; i0 < nitems; i0 += 1u << 30) {
     unsigned cnt = (unsigned)std::min<size_t>(nitems - i0, 1u << 30);
-    block_entries_kernel<<<cnt, 128, 0, st>>>(p, d_meta, d_items + i0, d_rows, d_rdst, d_cols, d_segs, d_out);
+    block_entries_kernel<<<cnt, ETHREADS, 0, st>>>(p, d_meta, d_items + i0, d_rows, d_rdst, d_cols, d_segs, d_out);
     HB_CHECK_LAUNCH();
   }
   HB_CUDA(cudaStreamSynchronize(st));
