@@ -168,7 +168,9 @@ void id_level(const hb_ctx* c, double2* d_A, const std::vector<int>& m, const st
   std::vector<long long> soff((size_t)cnt);
   long long sacc = 0;
   int max_n = 0;
+  long long max_mn = 0;
   for (int b = 0; b < cnt; ++b) {
+    max_mn = std::max(max_mn, (long long)m[(size_t)b] * n[(size_t)b]);
     soff[(size_t)b] = sacc;
     sacc += n[(size_t)b];
     max_n = std::max(max_n, n[(size_t)b]);
@@ -186,7 +188,7 @@ void id_level(const hb_ctx* c, double2* d_A, const std::vector<int>& m, const st
   to_dev(d_s, soff);
   d_rank.p = dev_alloc<int>((size_t)cnt);
   d_perm.p = dev_alloc<int>((size_t)sacc);
-  id_batch(cnt, d_m.p, d_n.p, d_a.p, d_A, c->opt.eps, d_rank.p, d_perm.p, d_s.p, max_n, 0);
+  id_batch(cnt, d_m.p, d_n.p, d_a.p, d_A, c->opt.eps, d_rank.p, d_perm.p, d_s.p, max_n, max_mn, 0);
   HB_CUDA(cudaDeviceSynchronize());
   rank.assign((size_t)cnt, 0);
   std::vector<int> perm((size_t)sacc);

@@ -371,7 +371,8 @@ void add_block(BlockBatchHost& B, const hb_ctx* c, const long long* rows, long l
                const long long* cols, long long n, long long out_off);
 void run_blocks(hb_ctx* c, BlockBatchHost& B, double2* d_out, cudaStream_t st);
 void id_batch(int count, const int* d_m, const int* d_n, const long long* d_aoff, double2* d_A,
-              double eps, int* d_rank, int* d_perm, const long long* d_soff, int max_n, cudaStream_t st);
+              double eps, int* d_rank, int* d_perm, const long long* d_soff, int max_n, long long max_mn,
+              cudaStream_t st);   // max_n, max_mn: the largest n and m n of the matrices
 void emit_v(int count, const int* d_m, const int* d_n, const long long* d_aoff, const double2* d_A,
             const int* d_rank, const int* d_perm, const long long* d_soff, const long long* d_voff,
             int ld_is_rank, double2* V64, float2* V32, cudaStream_t st);
