@@ -6,13 +6,22 @@
 // expansions (Eq. expansionT, Eq. expansionV0, Eq. expansionV1), then
 // local cubic interpolation of tau^2, v0, v1 to the Chebyshev nodes.
 //
-// One CTA per source node.  A Gauss-Seidel sweep visits the mesh in one of
+// One CTA, or a cluster of them, per source node.  A Gauss-Seidel sweep visits the mesh in one of
 // four orderings; an update reads only its own row and column (WENO5 along
 // each), so the points of one anti-diagonal never read one another and the
 // CTA updates an anti-diagonal at a time, in parallel, with a barrier
 // between anti-diagonals.  Along every row and column this is the same
 // upwind order as a row-by-row sweep, so each update sees the same new and
 // old values: the iterates are those of the sequential sweep, bit for bit.
+//
+// Bound by the FP64 unit (2 operations a cycle and SM): about 600 a point
+// update, 1200 with the compiler's divisions by 3, 6 and h instead of
+// Markstein's quotients (bessel.cuh div_by: the same bits).  With few sources
+// a cluster's SMs share every anti-diagonal and each point takes four lanes
+// (one WENO5 each).  36 sources, 109 x 109 mesh, 25 iterations a solve: 1224
+// ms at first, 832 with the quotients and clusters alone (a warp's FP64
+// instructions are bound to its sub-partition's unit), 389 with four
+// lanes; 256 sources, lens, h = 1/96, 4 iterations: 599 -> 397 ms.
 // The translation unit is compiled without contracted multiply-adds and
 // the Taylor values of the fixed points come from the host, so the tables
 // equal those of a plain FP64 host implementation of the same scheme.
@@ -40,37 +49,47 @@
 #include <cstdint>
 #include <vector>
 
+#include <cooperative_groups.h>
+
 #include "hb_internal.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace hb {
 namespace {
 
-constexpr int SW_THREADS = 256;   // two CTAs (sources) per SM
+constexpr int SW_THREADS = 256;   // two CTAs per SM
 constexpr int SW_EDGE = 3;            // outflow rows / columns
 constexpr int SW_TAYLOR = 46;         // T_2..T_6 (25), B_0..B_4 (15), C_0..C_2 (6)
 constexpr double SW_WENO_EPS = 1e-6;
 constexpr int SW_FIX_T = 128, SW_FIX_B = 64, SW_FIX_C = 16;   // fixed points per source (boxes of 11^2, 7^2, 3^2)
 
-// f at (i, j), continued linearly past the mesh in i (resp. j)
-__device__ __forceinline__ double lin_i(const double* f, int M, int i, int j) {
-  const double* r = f + (size_t)j * M;
-  if (i < 0) return r[0] + (double)i * (r[1] - r[0]);
-  if (i >= M) return r[M - 1] + (double)(i - M + 1) * (r[M - 1] - r[M - 2]);
-  return r[i];
-}
-__device__ __forceinline__ double lin_j(const double* f, int M, int i, int j) {
-  if (j < 0) return f[i] + (double)j * (f[(size_t)M + i] - f[i]);
-  if (j >= M) {
-    const double a = f[(size_t)(M - 1) * M + i], b = f[(size_t)(M - 2) * M + i];
-    return a + (double)(j - M + 1) * (a - b);
+// The CTAs of one source.  Points of a loop go to them warp by warp.
+struct Team {
+  int nc, rank;   // CTAs, this one
+  __device__ int first() const { return ((threadIdx.x >> 5) * nc + rank) * 32 + (threadIdx.x & 31); }
+  __device__ int stride() const { return SW_THREADS * nc; }
+  // every thread of the team, its writes to global memory included
+  __device__ void sync() const {
+    if (nc > 1) {
+      __threadfence();
+      cg::this_cluster().sync();
+    } else {
+      __syncthreads();
+    }
   }
-  return f[(size_t)j * M + i];
-}
+};
+// fields change under other SMs of the team: read from L2
+__device__ __forceinline__ double fld(const double* p) { return __ldcg(p); }
+
+// x / 3, x / 6 and x / h with h's reciprocal
+__device__ __forceinline__ double by3(double x) { return div_by(x, 3.0, 1.0 / 3.0); }
+__device__ __forceinline__ double by6(double x) { return div_by(x, 6.0, 1.0 / 6.0); }
 
 // f at (i, j), continued past the mesh by the cubic through the four
 // values nearest the edge (Lagrange weights at -t, t cells past it)
 __device__ __forceinline__ double cub_i(const double* f, int M, int i, int j) {
-  if (i >= 0 && i < M) return f[(size_t)j * M + i];
+  if (i >= 0 && i < M) return fld(f + (size_t)j * M + i);
   const int s = i < 0 ? 1 : -1, e = i < 0 ? 0 : M - 1;
   const double t = (double)(i < 0 ? -i : i - M + 1);
   double v = 0.0;
@@ -78,12 +97,12 @@ __device__ __forceinline__ double cub_i(const double* f, int M, int i, int j) {
     double w = 1.0;
     for (int b = 0; b < 4; ++b)
       if (b != a) w *= (-t - b) / (double)(a - b);
-    v += w * f[(size_t)j * M + e + a * s];
+    v += w * fld(f + (size_t)j * M + e + a * s);
   }
   return v;
 }
 __device__ __forceinline__ double cub_j(const double* f, int M, int i, int j) {
-  if (j >= 0 && j < M) return f[(size_t)j * M + i];
+  if (j >= 0 && j < M) return fld(f + (size_t)j * M + i);
   const int s = j < 0 ? 1 : -1, e = j < 0 ? 0 : M - 1;
   const double t = (double)(j < 0 ? -j : j - M + 1);
   double v = 0.0;
@@ -91,17 +110,17 @@ __device__ __forceinline__ double cub_j(const double* f, int M, int i, int j) {
     double w = 1.0;
     for (int b = 0; b < 4; ++b)
       if (b != a) w *= (-t - b) / (double)(a - b);
-    v += w * f[(size_t)(e + a * s) * M + i];
+    v += w * fld(f + (size_t)(e + a * s) * M + i);
   }
   return v;
 }
 
 // WENO5 (Jiang-Peng weights) of five divided differences; *k = the weight
 // of v3 minus that of v4 in the result at the current weights
-__device__ double weno5(double v1, double v2, double v3, double v4, double v5, double* k) {
-  const double p1 = v1 / 3.0 - 7.0 * v2 / 6.0 + 11.0 * v3 / 6.0;
-  const double p2 = -v2 / 6.0 + 5.0 * v3 / 6.0 + v4 / 3.0;
-  const double p3 = v3 / 3.0 + 5.0 * v4 / 6.0 - v5 / 6.0;
+__device__ __forceinline__ double weno5(double v1, double v2, double v3, double v4, double v5, double* k) {
+  const double p1 = by3(v1) - by6(7.0 * v2) + by6(11.0 * v3);
+  const double p2 = -by6(v2) + by6(5.0 * v3) + by3(v4);
+  const double p3 = by3(v3) + by6(5.0 * v4) - by6(v5);
   const double e1 = v1 - 2.0 * v2 + v3, f1 = v1 - 4.0 * v2 + 3.0 * v3;
   const double e2 = v2 - 2.0 * v3 + v4, f2 = v2 - v4;
   const double e3 = v3 - 2.0 * v4 + v5, f3 = 3.0 * v3 - 4.0 * v4 + v5;
@@ -112,28 +131,71 @@ __device__ double weno5(double v1, double v2, double v3, double v4, double v5, d
   const double a2 = 0.6 / ((SW_WENO_EPS + s2) * (SW_WENO_EPS + s2));
   const double a3 = 0.3 / ((SW_WENO_EPS + s3) * (SW_WENO_EPS + s3));
   const double sum = a1 + a2 + a3;
-  *k = (11.0 / 6.0 * a1 + 0.5 * a2 - 0.5 * a3) / sum;
-  return (a1 * p1 + a2 * p2 + a3 * p3) / sum;
+  const double inv = 1.0 / sum;
+  *k = div_by(11.0 / 6.0 * a1 + 0.5 * a2 - 0.5 * a3, sum, inv);
+  return div_by(a1 * p1 + a2 * p2 + a3 * p3, sum, inv);
 }
 
 // one-sided derivatives d- and d+ at u[3] of the seven values u[0..6]
 // (spacing h), with k- = h d(d-)/du[3] and k+ = -h d(d+)/du[3]
-__device__ __forceinline__ void weno_pair(const double* u, double h, double* dm, double* dp, double* km,
+__device__ __forceinline__ void weno_pair(const double* u, double h, double rh, double* dm, double* dp, double* km,
                                           double* kp) {
   double d[6];
-  for (int k = 0; k < 6; ++k) d[k] = (u[k + 1] - u[k]) / h;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) d[k] = div_by(u[k + 1] - u[k], h, rh);
   *dm = weno5(d[0], d[1], d[2], d[3], d[4], km);
   *dp = weno5(d[5], d[4], d[3], d[2], d[1], kp);
 }
 
-// p-, p+ (x) and q-, q+ (z) at (i, j); kk = (k of p-, p+, q-, q+)
-__device__ __forceinline__ void weno_derivs(const double* f, int M, int i, int j, double h, double* pm, double* pp,
-                                            double* qm, double* qp, double* kk) {
-  double u[7];
-  for (int k = 0; k < 7; ++k) u[k] = lin_i(f, M, i - 3 + k, j);
-  weno_pair(u, h, pm, pp, &kk[0], &kk[1]);
-  for (int k = 0; k < 7; ++k) u[k] = lin_j(f, M, i, j - 3 + k);
-  weno_pair(u, h, qm, qp, &kk[2], &kk[3]);
+// The derivatives at one point along both axes, for every thread that takes
+// the point: p- = m[0], p+ = p[0] (x), q- = m[1], q+ = p[1] (z), and their
+// weights km, kp.  (Updated points are at least SW_EDGE = 3 off the edge: the
+// stencils stay on the mesh.)
+struct Derivs {
+  double m[2], p[2], km[2], kp[2];
+};
+
+// One thread per point.
+__device__ __forceinline__ void derivs_one(const double* c, int M, double h, double rh, Derivs& D) {
+#pragma unroll
+  for (int ax = 0; ax < 2; ++ax) {
+    double u[7];
+#pragma unroll
+    for (int k = 0; k < 7; ++k) u[k] = fld(c + (ptrdiff_t)(k - 3) * (ax ? M : 1));
+    weno_pair(u, h, rh, &D.m[ax], &D.p[ax], &D.km[ax], &D.kp[ax]);
+  }
+}
+
+// Four threads per point, one WENO5 each (bits 0 and 1 of the lane: side and
+// axis).  A warp's FP64 instruction takes 64 cycles of its sub-partition's unit
+// whatever the other sub-partitions do, so a short anti-diagonal is
+// faster on four times the warps, each with a third of the instructions.
+__device__ __forceinline__ void derivs_quad(const double* c, int M, double h, double rh, int lane, Derivs& D) {
+  const bool plus = lane & 1, z = lane & 2;
+  const ptrdiff_t st = (z ? M : 1) * (plus ? -1 : 1);
+  double w[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) w[k] = fld(c + (k - 3) * st);
+  double v[5];
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const double d = w[k + 1] - w[k];
+    v[k] = div_by(plus ? -d : d, h, rh);
+  }
+  double k0;
+  const double v0 = weno5(v[0], v[1], v[2], v[3], v[4], &k0);
+  const double v1 = __shfl_xor_sync(0xffffffffu, v0, 1), k1 = __shfl_xor_sync(0xffffffffu, k0, 1);
+  const double m = plus ? v1 : v0, p = plus ? v0 : v1, km = plus ? k1 : k0, kp = plus ? k0 : k1;
+  const double m2 = __shfl_xor_sync(0xffffffffu, m, 2), p2 = __shfl_xor_sync(0xffffffffu, p, 2);
+  const double km2 = __shfl_xor_sync(0xffffffffu, km, 2), kp2 = __shfl_xor_sync(0xffffffffu, kp, 2);
+  D.m[0] = z ? m2 : m;
+  D.m[1] = z ? m : m2;
+  D.p[0] = z ? p2 : p;
+  D.p[1] = z ? p : p2;
+  D.km[0] = z ? km2 : km;
+  D.km[1] = z ? km : km2;
+  D.kp[0] = z ? kp2 : kp;
+  D.kp[1] = z ? kp : kp2;
 }
 
 __device__ __forceinline__ bool on_edge(int i, int j, int M) {
@@ -176,53 +238,61 @@ struct SweepArgs {
 };
 
 // one Gauss-Seidel sweep in ordering o (0..3) of an M x M mesh, an
-// anti-diagonal ii + jj = dd at a time; upd(i, j) updates one point
-template <class Upd>
-__device__ void sweep_once(int o, int M, Upd& upd) {
+// anti-diagonal ii + jj = dd at a time; upd(i, j, live) updates one point, by
+// one thread or (QUAD) by the four lanes of a quad, whole warps calling it
+template <bool QUAD, class Upd>
+__device__ void sweep_once(const Team& tm, int o, int M, Upd& upd) {
+  constexpr int PW = QUAD ? 8 : 32;   // points per warp
+  const int lane = threadIdx.x & 31, w0 = ((threadIdx.x >> 5) * tm.nc + tm.rank) * PW;
   for (int dd = 0; dd < 2 * M - 1; ++dd) {
     const int ilo = dd - M + 1 > 0 ? dd - M + 1 : 0, ihi = dd < M - 1 ? dd : M - 1;
-    for (int ii = ilo + (int)threadIdx.x; ii <= ihi; ii += (int)blockDim.x) {
+    for (int b = ilo + w0; b <= ihi; b += SW_THREADS / 32 * PW * tm.nc) {
+      const int at = b + (QUAD ? lane >> 2 : lane);
+      const bool live = at <= ihi;
+      const int ii = live ? at : ihi;
       const int jj = dd - ii;
       const int j = (o & 2) ? M - 1 - jj : jj;
       const int i = (o == 1 || o == 2) ? M - 1 - ii : ii;
-      upd(i, j);
+      upd(i, j, live);
     }
-    __syncthreads();
+    tm.sync();
   }
 }
 
 // the outflow closure: the SW_EDGE outermost points of every row, then of
 // every column, linear extrapolations of the two nearest inner ones (rows
 // first: the corners take the columns' values); fixed points keep theirs
-__device__ void extrapolate_edges(double* f, const unsigned char* fixed, int M) {
-  for (int j = threadIdx.x; j < M; j += blockDim.x) {
+__device__ void extrapolate_edges(const Team& tm, double* f, const unsigned char* fixed, int M) {
+  for (int j = tm.first(); j < M; j += tm.stride()) {
     double* r = f + (size_t)j * M;
+    const double l0 = fld(r + SW_EDGE), l1 = fld(r + SW_EDGE + 1);
+    const double h0 = fld(r + M - 1 - SW_EDGE), h1 = fld(r + M - 2 - SW_EDGE);
     for (int i = 0; i < SW_EDGE; ++i) {
       const int t = SW_EDGE - i;
-      if (!fixed[(size_t)j * M + i]) r[i] = r[SW_EDGE] + t * (r[SW_EDGE] - r[SW_EDGE + 1]);
+      if (!__ldcg(fixed + (size_t)j * M + i)) r[i] = l0 + t * (l0 - l1);
       const int k = M - 1 - i;
-      if (!fixed[(size_t)j * M + k]) r[k] = r[M - 1 - SW_EDGE] + t * (r[M - 1 - SW_EDGE] - r[M - 2 - SW_EDGE]);
+      if (!__ldcg(fixed + (size_t)j * M + k)) r[k] = h0 + t * (h0 - h1);
     }
   }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < SW_EDGE * M; idx += blockDim.x) {
+  tm.sync();
+  for (int idx = tm.first(); idx < SW_EDGE * M; idx += tm.stride()) {
     const int j = idx / M, i = idx % M;
     const int t = SW_EDGE - j;
     const size_t p = (size_t)j * M + i, q = (size_t)(M - 1 - j) * M + i;
-    if (!fixed[p]) f[p] = f[(size_t)SW_EDGE * M + i] + t * (f[(size_t)SW_EDGE * M + i] - f[(size_t)(SW_EDGE + 1) * M + i]);
-    if (!fixed[q])
-      f[q] = f[(size_t)(M - 1 - SW_EDGE) * M + i] +
-             t * (f[(size_t)(M - 1 - SW_EDGE) * M + i] - f[(size_t)(M - 2 - SW_EDGE) * M + i]);
+    const double l0 = fld(f + (size_t)SW_EDGE * M + i), l1 = fld(f + (size_t)(SW_EDGE + 1) * M + i);
+    const double h0 = fld(f + (size_t)(M - 1 - SW_EDGE) * M + i), h1 = fld(f + (size_t)(M - 2 - SW_EDGE) * M + i);
+    if (!__ldcg(fixed + p)) f[p] = l0 + t * (l0 - l1);
+    if (!__ldcg(fixed + q)) f[q] = h0 + t * (h0 - h1);
   }
-  __syncthreads();
+  tm.sync();
 }
 
 // fourth-order central differences (cubic continuation past the edge):
 // fx, fz (first) and lap (Laplacian), each optional
-__device__ void central_diffs(const double* f, int M, double h, double* fx, double* fz, double* lap) {
-  for (int p = threadIdx.x; p < M * M; p += blockDim.x) {
+__device__ void central_diffs(const Team& tm, const double* f, int M, double h, double* fx, double* fz, double* lap) {
+  for (int p = tm.first(); p < M * M; p += tm.stride()) {
     const int j = p / M, i = p % M;
-    const double xm2 = cub_i(f, M, i - 2, j), xm1 = cub_i(f, M, i - 1, j), x0 = f[(size_t)j * M + i];
+    const double xm2 = cub_i(f, M, i - 2, j), xm1 = cub_i(f, M, i - 1, j), x0 = fld(f + (size_t)j * M + i);
     const double xp1 = cub_i(f, M, i + 1, j), xp2 = cub_i(f, M, i + 2, j);
     const double zm2 = cub_j(f, M, i, j - 2), zm1 = cub_j(f, M, i, j - 1);
     const double zp1 = cub_j(f, M, i, j + 1), zp2 = cub_j(f, M, i, j + 2);
@@ -233,18 +303,24 @@ __device__ void central_diffs(const double* f, int M, double h, double* fx, doub
                 (-zp2 + 16.0 * zp1 - 30.0 * x0 + 16.0 * zm1 - zm2)) /
                (12.0 * h * h);
   }
-  __syncthreads();
+  tm.sync();
 }
 
-// the largest of the CTA's values v >= 0 (every thread gets it)
-__device__ double block_max(double v, unsigned long long* slot) {
+// the largest of the team's values v >= 0 (every thread gets it)
+__device__ double team_max(const Team& tm, double v, unsigned long long* slot) {
   if (threadIdx.x == 0) *slot = 0ull;
   __syncthreads();
   atomicMax(slot, (unsigned long long)__double_as_longlong(v));
-  __syncthreads();
-  const double r = __longlong_as_double((long long)*slot);
-  __syncthreads();
-  return r;
+  tm.sync();
+  unsigned long long r = *slot;
+  if (tm.nc > 1) {
+    for (int c = 0; c < tm.nc; ++c) {
+      const unsigned long long o = *cg::this_cluster().map_shared_rank(slot, c);
+      if (o > r) r = o;
+    }
+  }
+  tm.sync();
+  return __longlong_as_double((long long)r);
 }
 
 // local cubic (4 x 4 Lagrange) interpolation of the M x M field f (origin
@@ -268,18 +344,20 @@ __device__ double cubic_at(int M, double lo, double h, const double* f, double x
   }
   double s = 0.0;
   for (int b = 0; b < 4; ++b)
-    for (int a = 0; a < 4; ++a) s += wz[b] * wx[a] * f[(size_t)(j0 + b) * M + i0 + a];
+    for (int a = 0; a < 4; ++a) s += wz[b] * wx[a] * fld(f + (size_t)(j0 + b) * M + i0 + a);
   return s;
 }
 
-// One CTA per source node: the eikonal on the mesh, then the transports of
+// nc CTAs per source node: the eikonal on the mesh, then the transports of
 // v0 and v1 on the window, then the tables' columns at the nodes.
-__global__ void __launch_bounds__(SW_THREADS, 2) sweep_kernel(SweepArgs a) {
+template <bool QUAD>
+__global__ void __launch_bounds__(SW_THREADS, 2) sweep_kernel(SweepArgs a, int nc) {
   __shared__ unsigned long long red;
-  const int k = blockIdx.x;
+  const Team tm{nc, (int)blockIdx.x % nc};
+  const int k = blockIdx.x / nc;
   const int M = a.M, Mw = a.Mw;
   const size_t N = (size_t)M * M, Nw = (size_t)Mw * Mw;
-  const double h = a.h;
+  const double h = a.h, rh = 1.0 / h;
   const double x0 = a.px[a.src[k]], z0 = a.pz[a.src[k]];
   const double* T = a.taylor + (size_t)k * SW_TAYLOR;
   const double n0 = sqrt(T[0]);   // T_2 = S0 (X^2 + Z^2), S0 = n0^2
@@ -300,7 +378,7 @@ __global__ void __launch_bounds__(SW_THREADS, 2) sweep_kernel(SweepArgs a) {
   unsigned char* fixw = fixg + N;
 
   // ---- factored eikonal on the mesh ----
-  for (size_t p = threadIdx.x; p < N; p += blockDim.x) {
+  for (size_t p = tm.first(); p < N; p += tm.stride()) {
     const int j = (int)(p / M), i = (int)(p % M);
     const double X = a.lo + i * h - x0, Z = a.lo + j * h - z0;
     const double rho = sqrt(X * X + Z * Z);
@@ -310,31 +388,43 @@ __global__ void __launch_bounds__(SW_THREADS, 2) sweep_kernel(SweepArgs a) {
     tb[p] = 1.0;
     fixg[p] = 0;
   }
-  __syncthreads();
-  for (int q = threadIdx.x; q < F.nT; q += blockDim.x) {
+  tm.sync();
+  for (int q = tm.first(); q < F.nT; q += tm.stride()) {
     fixg[F.pT[q]] = 1;
     tb[F.pT[q]] = F.tbT[q];
   }
-  __syncthreads();
+  tm.sync();
   double last = 0.0;
-  auto eik = [&](int i, int j) {
+  const int lane = threadIdx.x & 31;
+  // a point that is not updated computes at an inner one and stores nothing
+  auto inner = [](int i, int n) { return i < SW_EDGE ? SW_EDGE : i > n - 1 - SW_EDGE ? n - 1 - SW_EDGE : i; };
+  auto derivs = [&](const double* c, int n, Derivs& D) {
+    if (QUAD) derivs_quad(c, n, h, rh, lane, D);
+    else derivs_one(c, n, h, rh, D);
+  };
+  auto eik = [&](int i, int j, bool live) {
+    live = live && !on_edge(i, j, M);
+    i = inner(i, M);
+    j = inner(j, M);
     const size_t p = (size_t)j * M + i;
-    if (fixg[p] || on_edge(i, j, M)) return;
-    double pm, pp, qm, qp, kk[4];
-    weno_derivs(tb, M, i, j, h, &pm, &pp, &qm, &qp, kk);
-    const double A = tt[p] * 0.5 * (pm + pp) + tb[p] * gx[p];
-    const double B = tt[p] * 0.5 * (qm + qp) + tb[p] * gz[p];
+    live = live && !__ldcg(fixg + p);
+    if (!QUAD && !live) return;
+    Derivs D;
+    derivs(tb + p, M, D);
+    const double c = fld(tb + p), alpha = fld(tt + p), gxp = fld(gx + p), gzp = fld(gz + p);
+    const double A = alpha * 0.5 * (D.m[0] + D.p[0]) + c * gxp;
+    const double B = alpha * 0.5 * (D.m[1] + D.p[1]) + c * gzp;
     const double H = sqrt(A * A + B * B);
-    const double alpha = tt[p];
-    const double hlf = H - alpha * 0.5 * (pp - pm) - alpha * 0.5 * (qp - qm);
+    const double hlf = H - alpha * 0.5 * (D.p[0] - D.m[0]) - alpha * 0.5 * (D.p[1] - D.m[1]);
     // the first-order coefficient of tb in hlf, or its value at the
     // current WENO weights where that is larger (no overshoot)
-    const double dH = H > 0 ? (A * (tt[p] * 0.5 * (kk[0] - kk[1]) / h + gx[p]) +
-                               B * (tt[p] * 0.5 * (kk[2] - kk[3]) / h + gz[p])) / H
+    const double dH = H > 0 ? (A * (div_by(alpha * 0.5 * (D.km[0] - D.kp[0]), h, rh) + gxp) +
+                               B * (div_by(alpha * 0.5 * (D.km[1] - D.kp[1]), h, rh) + gzp)) / H
                             : 0.0;
-    const double kw = dH + alpha * 0.5 * (kk[0] + kk[1] + kk[2] + kk[3]) / h;
-    const double d = (a.n[p] - hlf) / fmax(2.0 * alpha / h, kw);
-    tb[p] += d;
+    const double kw = dH + div_by(alpha * 0.5 * (D.km[0] + D.kp[0] + D.km[1] + D.kp[1]), h, rh);
+    const double d = (a.n[p] - hlf) / fmax(div_by(2.0 * alpha, h, rh), kw);
+    if (!live) return;
+    if (!QUAD || (lane & 3) == 0) tb[p] = c + d;
     if (fabs(d) > last && i >= a.g_r0 && i <= a.g_r1 && j >= a.g_r0 && j <= a.g_r1) last = fabs(d);
   };
   int it;
@@ -342,87 +432,96 @@ __global__ void __launch_bounds__(SW_THREADS, 2) sweep_kernel(SweepArgs a) {
   for (it = 0; it < a.max_iter; ++it) {
     last = 0.0;
     for (int o = 0; o < 4; ++o) {
-      sweep_once(o, M, eik);
-      extrapolate_edges(tb, fixg, M);
+      sweep_once<QUAD>(tm, o, M, eik);
+      extrapolate_edges(tm, tb, fixg, M);
     }
-    worst = block_max(last, &red);
+    worst = team_max(tm, last, &red);
     if (worst < a.tol) break;
   }
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0 && tm.rank == 0) {
     a.info[(size_t)k * 6 + 0] = it;
     a.info[(size_t)k * 6 + 3] = worst;
   }
-  for (size_t p = threadIdx.x; p < N; p += blockDim.x) tau2[p] = (tt[p] * tb[p]) * (tt[p] * tb[p]);
-  __syncthreads();
-  for (int q = threadIdx.x; q < F.nT; q += blockDim.x) tau2[F.pT[q]] = F.t2T[q];
-  __syncthreads();
+  for (size_t p = tm.first(); p < N; p += tm.stride()) {
+    const double t = fld(tt + p) * fld(tb + p);
+    tau2[p] = t * t;
+  }
+  tm.sync();
+  for (int q = tm.first(); q < F.nT; q += tm.stride()) tau2[F.pT[q]] = F.t2T[q];
+  tm.sync();
   // derivatives of tau^2 on the mesh (true neighbours at the window's edge)
-  central_diffs(tau2, M, h, tb, tt, gx);
-  for (size_t q = threadIdx.x; q < Nw; q += blockDim.x) {
+  central_diffs(tm, tau2, M, h, tb, tt, gx);
+  for (size_t q = tm.first(); q < Nw; q += tm.stride()) {
     const int j = (int)(q / Mw), i = (int)(q % Mw);
     const size_t p = (size_t)(j + a.off) * M + i + a.off;
-    ax[q] = tb[p];
-    az[q] = tt[p];
-    lt[q] = gx[p];
+    ax[q] = fld(tb + p);
+    az[q] = fld(tt + p);
+    lt[q] = fld(gx + p);
     nw[q] = a.n[p];
   }
-  __syncthreads();
+  tm.sync();
 
   // ---- transports on the window: s = 0 (v0), s = 1 (v1) ----
   for (int s = 0; s < 2; ++s) {
     double* v = s == 0 ? v0 : v1;
-    if (s == 1) central_diffs(v0, Mw, h, nullptr, nullptr, rhs);
+    if (s == 1) central_diffs(tm, v0, Mw, h, nullptr, nullptr, rhs);
     const double start = s == 0 ? T[25] : T[40];   // B_0, C_0
-    for (size_t p = threadIdx.x; p < Nw; p += blockDim.x) {
+    for (size_t p = tm.first(); p < Nw; p += tm.stride()) {
       v[p] = start;
       fixw[p] = 0;
     }
-    __syncthreads();
+    tm.sync();
     const int nf = s == 0 ? F.nB : F.nC;
-    for (int q = threadIdx.x; q < nf; q += blockDim.x) {
+    for (int q = tm.first(); q < nf; q += tm.stride()) {
       const int p = s == 0 ? F.pB[q] : F.pC[q];
       fixw[p] = 1;
       v[p] = s == 0 ? F.vB[q] : F.vC[q];
     }
-    __syncthreads();
-    auto tra = [&](int i, int j) {
+    tm.sync();
+    auto tra = [&](int i, int j, bool live) {
+      live = live && !on_edge(i, j, Mw);
+      i = inner(i, Mw);
+      j = inner(j, Mw);
       const size_t p = (size_t)j * Mw + i;
-      if (fixw[p] || on_edge(i, j, Mw)) return;
-      double pm, pp, qm, qp, kk[4];
-      weno_derivs(v, Mw, i, j, h, &pm, &pp, &qm, &qp, kk);
-      const double c = s == 0 ? lt[p] - 4.0 * nw[p] * nw[p] : lt[p];
-      const double f = s == 0 ? 0.0 : rhs[p];
-      const double alx = 2.0 * fabs(ax[p]), alz = 2.0 * fabs(az[p]);
-      const double hlf = ax[p] * (pm + pp) + az[p] * (qm + qp) + c * v[p] - alx * 0.5 * (pp - pm) -
-                         alz * 0.5 * (qp - qm);
+      live = live && !__ldcg(fixw + p);
+      if (!QUAD && !live) return;
+      Derivs D;
+      derivs(v + p, Mw, D);
+      const double ap = fld(ax + p), bp = fld(az + p), lp = fld(lt + p), np = fld(nw + p), vp = fld(v + p);
+      const double c = s == 0 ? lp - 4.0 * np * np : lp;
+      const double f = s == 0 ? 0.0 : fld(rhs + p);
+      const double alx = 2.0 * fabs(ap), alz = 2.0 * fabs(bp);
+      const double hlf = ap * (D.m[0] + D.p[0]) + bp * (D.m[1] + D.p[1]) + c * vp - alx * 0.5 * (D.p[0] - D.m[0]) -
+                         alz * 0.5 * (D.p[1] - D.m[1]);
       // the first-order coefficient of v in hlf (c v not lagged), or its
       // value at the current WENO weights where that is larger
-      const double den = (alx + alz) / h + c;
-      if (!(den > 0.25 * (alx + alz) / h)) return;
-      const double kw = (ax[p] * (kk[0] - kk[1]) + az[p] * (kk[2] - kk[3]) + 0.5 * alx * (kk[0] + kk[1]) +
-                         0.5 * alz * (kk[2] + kk[3])) / h + c;
+      const double den = div_by(alx + alz, h, rh) + c;
+      if (!(den > div_by(0.25 * (alx + alz), h, rh))) return;
+      const double kw = div_by(ap * (D.km[0] - D.kp[0]) + bp * (D.km[1] - D.kp[1]) + 0.5 * alx * (D.km[0] + D.kp[0]) +
+                                   0.5 * alz * (D.km[1] + D.kp[1]), h, rh) + c;
       const double d = (f - hlf) / fmax(den, kw);
-      v[p] += d;
+      if (!live) return;
+      if (!QUAD || (lane & 3) == 0) v[p] = vp + d;
       if (fabs(d) > last && i >= a.w_r0 && i <= a.w_r1 && j >= a.w_r0 && j <= a.w_r1) last = fabs(d);
     };
     worst = 0.0;
     for (it = 0; it < a.max_iter; ++it) {
       last = 0.0;
       for (int o = 0; o < 4; ++o) {
-        sweep_once(o, Mw, tra);
-        extrapolate_edges(v, fixw, Mw);
+        sweep_once<QUAD>(tm, o, Mw, tra);
+        extrapolate_edges(tm, v, fixw, Mw);
       }
-      worst = block_max(last, &red);
+      worst = team_max(tm, last, &red);
       if (worst < a.tol) break;
     }
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && tm.rank == 0) {
       a.info[(size_t)k * 6 + 1 + s] = it;
       a.info[(size_t)k * 6 + 4 + s] = worst;
     }
   }
 
   // ---- the tables' column k at the nodes ----
-  for (int i = threadIdx.x; i < a.NI; i += blockDim.x) {
+  for (int i = tm.first(); i < a.NI; i += tm.stride()) {
     a.tau2[(size_t)i * a.ns + k] = cubic_at(M, a.lo, h, tau2, a.px[i], a.pz[i]);
     a.v0[(size_t)i * a.ns + k] = cubic_at(Mw, a.wlo, h, v0, a.px[i], a.pz[i]);
     a.v1[(size_t)i * a.ns + k] = cubic_at(Mw, a.wlo, h, v1, a.px[i], a.pz[i]);
@@ -580,7 +679,26 @@ void sweep_tables(int M, double lo, double h, int w0, int w1, int roi0, int roi1
   A.v0 = d_v0.p;
   A.v1 = d_v1.p;
   A.info = d_info.p;
-  sweep_kernel<<<(unsigned)ns, SW_THREADS>>>(A);
+  // CTAs per source: as many as two per SM hold, and no more than the longest
+  // anti-diagonal has warps; four lanes per point while the warps of one-lane
+  // points would leave FP64 units of sub-partitions idle
+  int dev = 0, nsm = 0;
+  HB_CUDA(cudaGetDevice(&dev));
+  HB_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  int nc = 1;
+  while (nc < 8 && 2LL * nc * ns <= 2LL * nsm && nc * 32 < M) nc *= 2;
+  const bool quad = (long long)ns * M <= 32LL * 4 * nsm * 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)ns * (unsigned)nc);
+  cfg.blockDim = dim3(SW_THREADS);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)nc;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  HB_CUDA(cudaLaunchKernelEx(&cfg, quad ? sweep_kernel<true> : sweep_kernel<false>, A, nc));
   HB_CHECK_LAUNCH();
   HB_CUDA(cudaDeviceSynchronize());
   d_t2.download(tau2, (size_t)NI * ns);
