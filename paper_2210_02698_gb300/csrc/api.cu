@@ -118,6 +118,8 @@ void free_all(hb_ctx* c) {
   hb::dev_free(c->d_xh);
   hb::dev_free(c->d_tasks[0]);
   hb::dev_free(c->d_tasks[1]);
+  hb::task_plan_free(c->task_plans[0]);
+  hb::task_plan_free(c->task_plans[1]);
   hb::flow_plan_free(c->flow_plan[0]);
   hb::flow_plan_free(c->flow_plan[1]);
   hb::tc_plan_free(c->tc_plan[0]);
@@ -150,6 +152,7 @@ void release_build(hb_ctx* c) {
     c->flow_plan[d] = nullptr;
     hb::tc_plan_free(c->tc_plan[d]);
     c->tc_plan[d] = nullptr;
+    hb::task_plan_free(c->task_plans[d]);
     c->step_begin[d].clear();
     c->tasks_h[d].clear();
     c->task_rows[d].clear();
@@ -288,6 +291,7 @@ hb_status hb_build(hb_handle h) {
       allocs.free_all();
       h->d_f64 = nullptr;
       h->d_tasks[0] = h->d_tasks[1] = nullptr;
+      h->task_plans[0] = h->task_plans[1] = hb::TaskPlan{};   // its arrays went with the others
       h->d_nat[0] = h->d_nat[1] = nullptr;
       h->d_tc[0] = h->d_tc[1] = nullptr;
       h->d_pperm = nullptr;

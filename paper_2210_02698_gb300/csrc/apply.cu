@@ -45,42 +45,46 @@ __global__ void scatter_kernel(const double2* __restrict__ y, const long long* _
 }
 
 // ------------------------------------------------------- step tasks ----
-// Y = op(F) X of one task on the FP16 tensor cores by integer digits
+// Y = op(F) X of the step tasks on the FP16 tensor cores by integer digits
 // (split_fixed.cuh), in the orientation of the mixed apply: the MMA's M is
 // right-hand sides, N outputs, K = 2 x 8 inputs with real and imaginary
 // parts interleaved; D_r takes A rows (Re X, -Im X), D_i (Im X, Re X).  Up to
 // eight right-hand sides (HALF) both go into one MMA, rows 0-7 and 8-15.
 //
-// A CTA of 8 warps takes up to 64 outputs (8 n-tiles; row_blocks CTAs per task) of
-// one task.  It scales X per right-hand side and F per task (tk.fe, found
-// when the plan is made), splits X into digit fragments in shared memory,
-// KC k-steps at a time, and every warp streams its n-tile's F straight from
-// global memory into registers, one k-step ahead, splitting it there (each
-// F value is used by one warp only).  With fewer than 8 n-tiles the k-steps
-// are dealt over 2, 4 or 8 warps and the integer sums added: the result does
-// not depend on the split.  The split is a function of the task alone, so a
-// shard's sums equal the whole apply's.
+// A unit is one n-tile (8 outputs) of one task.  A CTA takes an item: units of
+// tasks that read the same inputs (the two transfer blocks of a skeleton, the
+// V^0 of every HODBF level and the dense block of a leaf; the tasks of a step
+// are kept in input order).  It scales X per right-hand side, splits it into
+// digit fragments in shared memory once, TASK_KC k-steps at a time, and every
+// warp streams its unit's F from global memory into registers, one k-step
+// ahead, scaling it per task (tk.fe, found when the plan is made) and
+// splitting it there.  Long sums (ks k-steps) are dealt over kw(ks) warps and
+// the integer sums added.  A unit's sums depend on its task alone, so a
+// shard's equal the whole apply's.
 //
-// Bound by instruction issue: 42 (21) MMAs and about 150 integer instructions
-// a warp per 8 outputs x 8 inputs, as much again to split the task's X where
-// its rank is near 16, and the epilogue, against 1024 x 4 FP64 FMAs for 16
-// right-hand sides (2048 cycles of an SM's FP64 unit).  Measured (192^2, 16
-// right-hand sides): 3.67 -> 1.92 ms against one FP64 FMA loop per output;
-// 120 x 88 adjoint with 5: 601 -> 251 us.
-constexpr int TASK_THREADS = 256;
-constexpr int TASK_WARPS = TASK_THREADS / 32;
+// Bound by instruction issue: per 8 outputs x 8 inputs 42 (21) MMAs and
+// about 250 other instructions of a warp, as many as that to split X where a task's rank
+// is near 16, and the epilogue, against 1024 x 4 FP64 FMAs for 16
+// right-hand sides (2048 cycles of an SM's FP64 unit).  Measured: 192^2 x 16
+// 3.67 ms with one FP64 FMA loop per output, 1.92 with a CTA of 8 warps per
+// task, 1.30 with four warps and shared inputs; 120 x 88 adjoint x 5: 601,
+// 251, 205 us.
 constexpr int TASK_KC = 16;              // k-steps of X held at a time
 constexpr uint32_t SPLIT_IM_SIGN = 0x80000000u;
+constexpr int task_kw(int ks, int W) {   // warps sharing a unit's k-steps
+  const int k = ks <= 12 ? 1 : ks <= 32 ? 2 : 4;
+  return k < W ? k : W;
+}
 
-// Rows [row0, row1) of a task with plain FP64 FMAs: what a task does whose
-// inputs are not all finite (thread -> (row, right-hand side), rows fastest).
+// Rows [row0, row1) of a task with plain FP64 FMAs, one warp: what a task
+// does whose inputs are not all finite (lane -> (row, right-hand side), rows fastest).
 __device__ __noinline__ void task_plain(const Task* __restrict__ task, const double2* __restrict__ F, double2* x, double2* y,
                                         double2* xh, int R, int row0, int row1) {
   const Task& tk = *task;
   double2* bufs[3] = {x, y, xh};
   double2* out = bufs[tk.y_buf] + (size_t)tk.y_off * R;
   const int rows = row1 - row0, total = rows * R;
-  for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
+  for (int idx = threadIdx.x & 31; idx < total; idx += 32) {
     const int row = row0 + idx % rows, rr = idx / rows;
     double ar = 0, ai = 0;
     for (int t = 0; t < tk.nterm; ++t) {
@@ -114,184 +118,195 @@ __device__ __noinline__ void task_plain(const Task* __restrict__ task, const dou
   }
 }
 
-template <bool HALF>
-__global__ void __launch_bounds__(TASK_THREADS, HALF ? 3 : 2)
-    task_kernel(const Task* __restrict__ tasks, const double2* __restrict__ F, double2* x, double2* y, double2* xh,
-                int R, int row_blocks) {
+template <bool HALF, int W>
+__global__ void __launch_bounds__(32 * W, 16 / W)
+    task_kernel(const TaskItem* __restrict__ items, const TaskUnit* __restrict__ units, const Task* __restrict__ tasks,
+                const double2* __restrict__ F, double2* x, double2* y, double2* xh, int R) {
   constexpr int NR = HALF ? 8 : 16;        // right-hand sides of the MMA rows
   constexpr int NE = HALF ? 4 : 8;         // accumulator elements per lane and digit diagonal
   constexpr int XW = HALF ? 2 : 4;         // X fragment words per lane
+  constexpr int XK = 32 * W / NR;          // inputs the CTA's threads take at once
   extern __shared__ __align__(16) uint32_t xs[];   // [k-step][digit][lane][XW]
   __shared__ int s_ex[16];
   __shared__ int s_bad;
-  const Task* task = tasks + blockIdx.x / row_blocks;
-  const Task tk = *task;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
-  const int tile0 = 8 * (blockIdx.x % row_blocks);
-  const int ntile = min(8, (tk.r_out + 7) / 8 - tile0);
-  if (ntile <= 0) return;
-  const double2* xin = tk.x_buf == 0 ? x : tk.x_buf == 1 ? y : xh;
-  const int rin0 = tk.r_in[0], rin1 = tk.nterm > 1 ? tk.r_in[1] : 0;
+  const TaskItem item = items[blockIdx.x];
+  const int rin0 = item.r_in[0], rin1 = item.r_in[1];
+  const double2* xin = item.x_buf == 0 ? x : item.x_buf == 1 ? y : xh;
+  const double2* xin0 = xin + item.x_off[0] * R;
+  const double2* xin1 = xin + item.x_off[1] * R;
   const int ks0 = (rin0 + 7) / 8, ks = ks0 + (rin1 + 7) / 8;
+  const int kw = task_kw(ks, W), uw = W / kw;
+  const int wt = warp % uw, kp = warp / uw;
 
-  // the exponent of every right-hand side over the task's inputs
-  if (tid < 16) s_ex[tid] = 1;
-  if (tid == 0) s_bad = (tk.fe == SPLIT_NONFINITE) ? 1 : 0;
-  __syncthreads();
-  const int xr = tid & (NR - 1), xk = tid / NR;
-  constexpr int XK = TASK_THREADS / NR;
-  if (xr < R) {
-    int e = 1;
-    for (int k = xk; k < rin0; k += XK) e = max(e, block_exponent(xin[(tk.x_off[0] + k) * R + xr]));
-    for (int k = xk; k < rin1; k += XK) e = max(e, block_exponent(xin[(tk.x_off[1] + k) * R + xr]));
-    atomicMax(&s_ex[xr], e);
-    if (e == SPLIT_NONFINITE) s_bad = 1;
-  }
-  __syncthreads();
-  if (s_bad) {
-    task_plain(task, F, x, y, xh, R, 8 * tile0, min(tk.r_out, 8 * (tile0 + 8)));
-    return;
-  }
-
-  // warp -> n-tile and share of the k-steps
-  const int kw = ntile > 4 ? 1 : ntile > 2 ? 2 : ntile > 1 ? 4 : 8;
-  const int wt = warp % (TASK_WARPS / kw), kp = warp / (TASK_WARPS / kw);
-  const bool work = wt < ntile;
-  const int row = 8 * (tile0 + wt) + g;
-  const bool rok = work && row < tk.r_out;
-
-  // F values (row, k = 2t) and (row, 2t + 1) of k-step q
-  auto load_f = [&](int q, double2& f0, double2& f1) {
+  // the warp's unit, and F values (row, k = 2t) and (row, 2t + 1) of its k-step q
+  bool work = false, rok = false;
+  TaskUnit unit;
+  int fe = 0, row = 0;
+  double2 f0, f1;
+  auto load_f = [&](int q) {
     f0 = f1 = make_double2(0.0, 0.0);
     if (!rok || q >= ks) return;
-    const int term = q >= ks0, rin = term ? rin1 : rin0;
+    const bool term = q >= ks0;
+    const int rin = term ? rin1 : rin0;
     const int k = 8 * (term ? q - ks0 : q) + 2 * t;
-    const double2* f = F + (term ? tk.f_off[1] : tk.f_off[0]);
-    if (!tk.conj_t) {
-      if (k < rin) f0 = __ldcs(f + (size_t)k * tk.r_out + row);
-      if (k + 1 < rin) f1 = __ldcs(f + (size_t)(k + 1) * tk.r_out + row);
-    } else {
-      const double2* fr = f + (size_t)row * rin + k;
-      if (k < rin) f0 = __ldcs(fr);
-      if (k + 1 < rin) f1 = __ldcs(fr + 1);
-      f0.y = -f0.y;
-      f1.y = -f1.y;
-    }
+    const double2* f = F + (term ? unit.f_off[1] : unit.f_off[0]);
+    const double2* p0 = unit.conj_t ? f + (size_t)row * rin + k : f + (size_t)k * unit.r_out + row;
+    const double2* p1 = unit.conj_t ? p0 + 1 : p0 + unit.r_out;
+    if (k < rin) f0 = __ldcs(p0);
+    if (k + 1 < rin) f1 = __ldcs(p1);
+  };
+  auto take_unit = [&](int u0) {
+    work = u0 + wt < item.units;
+    unit = units[item.unit0 + (work ? u0 + wt : 0)];
+    row = 8 * unit.tile + g;
+    rok = work && row < unit.r_out;
+    fe = tasks[unit.task].fe;
+    load_f(kp);
+  };
+  take_unit(0);
+
+  // value `k` (of the padded, concatenated inputs) of right-hand side xr
+  const int xr = tid & (NR - 1), xk = tid / NR;
+  auto load_x = [&](int k) {
+    const bool term = k >= 8 * ks0;
+    const int kin = term ? k - 8 * ks0 : k;
+    double2 v = make_double2(0.0, 0.0);
+    if (xr < R && kin < (term ? rin1 : rin0)) v = (term ? xin1 : xin0)[(size_t)kin * R + xr];
+    return v;
   };
 
-  float acc[SPLIT_ACC][NE];
-  long long hi[NE], lo[NE];
+  // the exponent of every right-hand side over the inputs
+  if (tid < 16) s_ex[tid] = 0;
+  if (tid == 0) s_bad = 0;
+  int ex = 0;
+  for (int k = xk; k < 8 * ks; k += XK) ex = max(ex, block_exponent(load_x(k)));
+  __syncthreads();
+  if (ex) atomicMax(&s_ex[xr], ex);
+  __syncthreads();
+  const int myex = max(s_ex[xr], SPLIT_MIN_EXP);
+  if (xr < R && !split_exponent_ok(s_ex[xr])) s_bad = 1;   // read after the next barrier
+
+  // X of k-steps [c0, c1) into digit fragments: word j of lane (g, t) is
+  // (right-hand side g + 8 (j & 1), input 2t + (j >> 1)); HALF: (g, 2t + j)
+  auto split_x = [&](int k, int c0, double2 v) {
+    const int q = k >> 3, kk = k & 7;
+    uint32_t w[SPLIT_DIGITS];
+    split_pair(v, myex, 0u, w);
+    const int j = HALF ? (kk & 1) : 2 * (kk & 1) + (xr >> 3);
+    uint32_t* dst = xs + (((q - c0) * SPLIT_DIGITS) * 32 + (xr & 7) * 4 + (kk >> 1)) * XW + j;
 #pragma unroll
-  for (int e = 0; e < NE; ++e) {
-    hi[e] = lo[e] = 0;
+    for (int s = 0; s < SPLIT_DIGITS; ++s) dst[s * 32 * XW] = w[s];
+  };
+
+  for (int u0 = 0; u0 < item.units; u0 += uw) {   // several passes only when X is held whole
+    if (u0) take_unit(u0);
+    float acc[SPLIT_ACC][NE];
+    long long hi[NE], lo[NE];
 #pragma unroll
-    for (int d = 0; d < SPLIT_ACC; ++d) acc[d][e] = 0.f;
-  }
-  const int myex = s_ex[xr];
-  double2 f0, f1;
-  load_f(kp, f0, f1);
-  for (int c0 = 0; c0 < ks; c0 += TASK_KC) {
-    const int c1 = min(ks, c0 + TASK_KC);
-    if (c0) __syncthreads();
-    // X of k-steps [c0, c1) into digit fragments: word j of lane (g, t) is
-    // (right-hand side g + 8 (j & 1), input 2t + (j >> 1)); HALF: (g, 2t + j)
-    for (int k = 8 * c0 + xk; k < 8 * c1; k += XK) {
-      const int q = k >> 3, kk = k & 7;
-      const int term = q >= ks0, kin = term ? k - 8 * ks0 : k;
-      double2 v = make_double2(0.0, 0.0);
-      if (xr < R && kin < (term ? rin1 : rin0)) v = xin[((term ? tk.x_off[1] : tk.x_off[0]) + kin) * R + xr];
-      uint32_t w[SPLIT_DIGITS];
-      split_pair(v.x, v.y, myex, w);
-      const int j = HALF ? (kk & 1) : 2 * (kk & 1) + (xr >> 3);
-      uint32_t* dst = xs + (((q - c0) * SPLIT_DIGITS) * 32 + (xr & 7) * 4 + (kk >> 1)) * XW + j;
+    for (int e = 0; e < NE; ++e) {
+      hi[e] = lo[e] = 0;
 #pragma unroll
-      for (int s = 0; s < SPLIT_DIGITS; ++s) dst[s * 32 * XW] = w[s];
+      for (int d = 0; d < SPLIT_ACC; ++d) acc[d][e] = 0.f;
     }
-    __syncthreads();
-    if (work) {
-      int since = 0;
-      for (int q = c0 + (kp - c0 % kw + kw) % kw; q < c1; q += kw) {
-        const double2 a0 = f0, a1 = f1;
-        load_f(q + kw, f0, f1);
-        uint32_t b0[SPLIT_DIGITS], b1[SPLIT_DIGITS];
-        split_pair(a0.x, a0.y, tk.fe, b0);
-        split_pair(a1.x, a1.y, tk.fe, b1);
-        const uint32_t* xq = xs + ((q - c0) * SPLIT_DIGITS * 32 + lane) * XW;
+    for (int c0 = 0; c0 < ks; c0 += TASK_KC) {
+      const int c1 = min(ks, c0 + TASK_KC);
+      if (u0 == 0) {
+        if (c0) __syncthreads();
+        for (int k = 8 * c0 + xk; k < 8 * c1; k += XK) split_x(k, c0, load_x(k));
+        __syncthreads();
+      }
+      if (work && !s_bad && split_exponent_ok(fe)) {
+        int since = 0;
+        for (int q = c0 + kp; q < c1; q += kw) {   // TASK_KC is a multiple of kw
+          const double2 a0 = f0, a1 = f1;
+          load_f(q + kw);
+          uint32_t b0[SPLIT_DIGITS], b1[SPLIT_DIGITS];
+          const uint32_t cs = unit.conj_t ? 0x80000000u : 0u;
+          const int fx = max(fe, SPLIT_MIN_EXP);
+          split_pair(a0, fx, cs, b0);
+          split_pair(a1, fx, cs, b1);
+          const uint32_t* xq = xs + ((q - c0) * SPLIT_DIGITS * 32 + lane) * XW;
 #pragma unroll
-        for (int i = 0; i < SPLIT_DIGITS; ++i) {
-          if constexpr (HALF) {
-            const uint2 w = *reinterpret_cast<const uint2*>(xq + i * 32 * XW);
-            const uint32_t a[4] = {w.x ^ SPLIT_IM_SIGN, __byte_perm(w.x, 0, 0x1032), w.y ^ SPLIT_IM_SIGN,
-                                   __byte_perm(w.y, 0, 0x1032)};
+          for (int i = 0; i < SPLIT_DIGITS; ++i) {
+            if constexpr (HALF) {
+              const uint2 w = *reinterpret_cast<const uint2*>(xq + i * 32 * XW);
+              const uint32_t a[4] = {w.x ^ SPLIT_IM_SIGN, __byte_perm(w.x, 0, 0x1032), w.y ^ SPLIT_IM_SIGN,
+                                     __byte_perm(w.y, 0, 0x1032)};
 #pragma unroll
-            for (int j = 0; i + j < SPLIT_DIGITS; ++j)
-              mma_f16(acc[i == 2 && j == 0 ? 6 : i + j], a[0], a[1], a[2], a[3], b0[j], b1[j]);
-          } else {
-            const uint4 w = *reinterpret_cast<const uint4*>(xq + i * 32 * XW);
-            const uint32_t r[4] = {w.x ^ SPLIT_IM_SIGN, w.y ^ SPLIT_IM_SIGN, w.z ^ SPLIT_IM_SIGN, w.w ^ SPLIT_IM_SIGN};
-            const uint32_t m[4] = {__byte_perm(w.x, 0, 0x1032), __byte_perm(w.y, 0, 0x1032),
-                                   __byte_perm(w.z, 0, 0x1032), __byte_perm(w.w, 0, 0x1032)};
+              for (int j = 0; i + j < SPLIT_DIGITS; ++j)
+                mma_f16(acc[i == 2 && j == 0 ? 6 : i + j], a[0], a[1], a[2], a[3], b0[j], b1[j]);
+            } else {
+              const uint4 w = *reinterpret_cast<const uint4*>(xq + i * 32 * XW);
+              const uint32_t r[4] = {w.x ^ SPLIT_IM_SIGN, w.y ^ SPLIT_IM_SIGN, w.z ^ SPLIT_IM_SIGN, w.w ^ SPLIT_IM_SIGN};
+              const uint32_t m[4] = {__byte_perm(w.x, 0, 0x1032), __byte_perm(w.y, 0, 0x1032),
+                                     __byte_perm(w.z, 0, 0x1032), __byte_perm(w.w, 0, 0x1032)};
 #pragma unroll
-            for (int j = 0; i + j < SPLIT_DIGITS; ++j) {
-              const int d = i == 2 && j == 0 ? 6 : i + j;
-              mma_f16(acc[d], r[0], r[1], r[2], r[3], b0[j], b1[j]);
-              mma_f16(acc[d] + 4, m[0], m[1], m[2], m[3], b0[j], b1[j]);
+              for (int j = 0; i + j < SPLIT_DIGITS; ++j) {
+                const int d = i == 2 && j == 0 ? 6 : i + j;
+                mma_f16(acc[d], r[0], r[1], r[2], r[3], b0[j], b1[j]);
+                mma_f16(acc[d] + 4, m[0], m[1], m[2], m[3], b0[j], b1[j]);
+              }
             }
           }
-        }
-        if (++since == 2 || q + kw >= c1) {
-          since = 0;
+          if (++since == 2 || q + kw >= c1) {
+            since = 0;
 #pragma unroll
-          for (int e = 0; e < NE; ++e)
-            split_flush(acc[0][e], acc[1][e], acc[2][e], acc[3][e], acc[4][e], acc[5][e], acc[6][e], hi[e], lo[e]);
+            for (int e = 0; e < NE; ++e)
+              split_flush(acc[0][e], acc[1][e], acc[2][e], acc[3][e], acc[4][e], acc[5][e], acc[6][e], hi[e], lo[e]);
+          }
         }
       }
     }
-  }
-  // add the shares of the k-steps
-  if (kw > 1) {
-    longlong2* red = reinterpret_cast<longlong2*>(xs);   // [kp - 1][n-tile][element][lane]
-    __syncthreads();
-    if (work && kp > 0)
+    // add the shares of the k-steps (kw > 1: one pass)
+    if (kw > 1) {
+      longlong2* red = reinterpret_cast<longlong2*>(xs);   // [kp - 1][unit][element][lane]
+      __syncthreads();
+      if (work && kp > 0)
 #pragma unroll
-      for (int e = 0; e < NE; ++e) red[(((kp - 1) * ntile + wt) * NE + e) * 32 + lane] = make_longlong2(hi[e], lo[e]);
-    __syncthreads();
-    if (!work || kp > 0) return;
-    for (int p = 0; p < kw - 1; ++p)
+        for (int e = 0; e < NE; ++e) red[(((kp - 1) * uw + wt) * NE + e) * 32 + lane] = make_longlong2(hi[e], lo[e]);
+      __syncthreads();
+      if (kp == 0)
+        for (int p = 0; p < kw - 1; ++p)
 #pragma unroll
-      for (int e = 0; e < NE; ++e) {
-        const longlong2 v = red[((p * ntile + wt) * NE + e) * 32 + lane];
-        hi[e] += v.x;
-        lo[e] += v.y;
-      }
-  }
-  if (!work) return;
-  double2* out = (tk.y_buf == 0 ? x : tk.y_buf == 1 ? y : xh) + (size_t)tk.y_off * R;
-  // element e of D: right-hand side g + 8 (e >> 1), output 2t + (e & 1); HALF:
-  // elements 0, 1 are D_r and 2, 3 D_i of right-hand side g
-#pragma unroll
-  for (int e = 0; e < NE / 2; ++e) {
-    const int rr = HALF ? g : g + 8 * (e >> 1);
-    const int ro = 8 * (tile0 + wt) + 2 * t + (e & 1);
-    if (rr >= R || ro >= tk.r_out) continue;
-    const int ex = tk.fe + s_ex[rr] - 2 * SPLIT_EXP_BIAS;
-    const int ei = HALF ? e + 2 : e + 4;
-    double2 v = make_double2(fixed_to_double(hi[e], lo[e], ex), fixed_to_double(hi[ei], lo[ei], ex));
-    double2* o = out + (size_t)ro * R + rr;
-    if (tk.accumulate) {
-      const double2 prev = *o;
-      v.x += prev.x;
-      v.y += prev.y;
+          for (int e = 0; e < NE; ++e) {
+            const longlong2 v = red[((p * uw + wt) * NE + e) * 32 + lane];
+            hi[e] += v.x;
+            lo[e] += v.y;
+          }
     }
-    *o = v;
+    if (!work || kp > 0) continue;
+    if (s_bad || !split_exponent_ok(fe)) {
+      task_plain(tasks + unit.task, F, x, y, xh, R, 8 * unit.tile, min(unit.r_out, 8 * unit.tile + 8));
+      continue;
+    }
+    double2* out = (unit.y_buf == 0 ? x : unit.y_buf == 1 ? y : xh) + (size_t)unit.y_off * R;
+    // element e of D: right-hand side g + 8 (e >> 1), output 2t + (e & 1); HALF:
+    // elements 0, 1 are D_r and 2, 3 D_i of right-hand side g
+#pragma unroll
+    for (int e = 0; e < NE / 2; ++e) {
+      const int rr = HALF ? g : g + 8 * (e >> 1);
+      const int ro = 8 * unit.tile + 2 * t + (e & 1);
+      if (rr >= R || ro >= unit.r_out) continue;
+      const int sx = max(fe, SPLIT_MIN_EXP) + max(s_ex[rr], SPLIT_MIN_EXP) - 2 * SPLIT_EXP_BIAS;
+      const int ei = HALF ? e + 2 : e + 4;
+      double2 v = make_double2(fixed_to_double(hi[e], lo[e], sx), fixed_to_double(hi[ei], lo[ei], sx));
+      double2* o = out + (size_t)ro * R + rr;
+      if (unit.accumulate) {
+        const double2 prev = *o;
+        v.x += prev.x;
+        v.y += prev.y;
+      }
+      *o = v;
+    }
   }
 }
 
-// tasks[i].fe = the largest exponent of task i's factor blocks (1 before),
+// tasks[i].fe = the largest exponent of task i's factor blocks (0 before),
 // blockIdx.y of gridDim.y shares of them
 __global__ void __launch_bounds__(256) task_exponent_kernel(Task* __restrict__ tasks, const double2* __restrict__ F) {
   Task& tk = tasks[blockIdx.x];
-  int e = 1;
+  int e = 0;
   for (int t = 0; t < tk.nterm; ++t) {
     const long long cnt = (long long)tk.r_out * tk.r_in[t];
     const double2* f = F + tk.f_off[t];
@@ -309,33 +324,106 @@ void task_exponents(Task* d_tasks, int n, const double2* F, cudaStream_t st) {
   HB_CHECK_LAUNCH();
 }
 
-StepShape step_shape(const Task* tasks, int n) {
-  StepShape s{0, 0};
-  for (int i = 0; i < n; ++i) {
-    const Task& t = tasks[i];
-    s.max_out = std::max(s.max_out, t.r_out);
-    s.max_ks = std::max(s.max_ks, (t.r_in[0] + 7) / 8 + (t.nterm > 1 ? (t.r_in[1] + 7) / 8 : 0));
-  }
-  return s;
+bool task_reads_before(const Task& a, const Task& b) {
+  auto key = [](const Task& t) {
+    return std::make_tuple((int)t.x_buf, t.x_off[0], t.r_in[0], (int)t.nterm, t.nterm > 1 ? t.x_off[1] : -1LL,
+                           t.nterm > 1 ? t.r_in[1] : 0);
+  };
+  return key(a) < key(b);
 }
 
-// One launch of FP64 step tasks, R <= 16 right-hand sides.
-void run_tasks_fp64(const Task* d_tasks, int n, const StepShape& sh, const double2* F, double2* x, double2* y,
-                    double2* xh, int R, cudaStream_t st) {
-  if (n <= 0) return;
-  const int rb = std::max(1, (sh.max_out + 63) / 64);
-  const unsigned grid = (unsigned)n * (unsigned)rb;
-  const size_t frag = (size_t)std::min(TASK_KC, std::max(1, sh.max_ks)) * SPLIT_DIGITS * 32 * 4;
-  const size_t red = (size_t)7 * 32 * sizeof(longlong2);   // the k-step shares of one CTA: at most 7 n-tile shares
-  if (R <= 8) {
-    const size_t smem = std::max(frag * 2, red * 4);
-    task_kernel<true><<<grid, TASK_THREADS, smem, st>>>(d_tasks, F, x, y, xh, R, rb);
-  } else {
-    const size_t smem = std::max(frag * 4, red * 8);
-    HB_CUDA(cudaFuncSetAttribute(task_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 56 << 10));
-    task_kernel<false><<<grid, TASK_THREADS, smem, st>>>(d_tasks, F, x, y, xh, R, rb);
+TaskPlan task_plan(const std::vector<Task>& tasks, const std::vector<int>& begin, int W) {
+  TaskPlan P;
+  P.W = W;
+  std::vector<TaskUnit> units;
+  std::vector<TaskItem> items;
+  for (size_t s = 0; s + 1 < begin.size(); ++s) {
+    P.item_begin.push_back((int)items.size());
+    int max_ks = 1;
+    long long nu = 0;
+    for (int i = begin[s]; i < begin[s + 1]; ++i) nu += (tasks[(size_t)i].r_out + 7) / 8;
+    for (int i = begin[s]; i < begin[s + 1];) {
+      const Task& t = tasks[(size_t)i];
+      const int ks = (t.r_in[0] + 7) / 8 + (t.nterm > 1 ? (t.r_in[1] + 7) / 8 : 0);
+      max_ks = std::max(max_ks, ks);
+      const int first = (int)units.size();
+      int j = i;
+      for (; j < begin[s + 1] && !task_reads_before(t, tasks[(size_t)j]) && !task_reads_before(tasks[(size_t)j], t); ++j)
+        for (int q = 0; q < (tasks[(size_t)j].r_out + 7) / 8; ++q) {
+          const Task& tj = tasks[(size_t)j];
+          TaskUnit u{};
+          u.f_off[0] = tj.f_off[0];
+          u.f_off[1] = tj.f_off[1];
+          u.y_off = tj.y_off;
+          u.task = j;
+          u.tile = q;
+          u.r_out = tj.r_out;
+          u.conj_t = tj.conj_t;
+          u.y_buf = tj.y_buf;
+          u.accumulate = tj.accumulate;
+          units.push_back(u);
+        }
+      // units per CTA: one pass of its warps; up to three (X split once for
+      // all) while the step still has two CTAs for every SM's four
+      const int uw = W / task_kw(ks, W);
+      const int passes = ks > TASK_KC || task_kw(ks, W) > 1 ? 1 : (int)std::max<long long>(1, std::min<long long>(3, nu / uw / 1216));
+      const int per = uw * passes, all = (int)units.size() - first, cut = (all + per - 1) / per;
+      for (int c = 0; c < cut; ++c) {   // equal shares
+        const int a = (int)((long long)all * c / cut), b = (int)((long long)all * (c + 1) / cut);
+        TaskItem it{};
+        it.unit0 = first + a;
+        it.units = b - a;
+        it.x_buf = t.x_buf;
+        it.r_in[0] = t.r_in[0];
+        it.r_in[1] = t.nterm > 1 ? t.r_in[1] : 0;
+        it.x_off[0] = t.x_off[0];
+        it.x_off[1] = t.nterm > 1 ? t.x_off[1] : 0;
+        items.push_back(it);
+      }
+      i = j;
+    }
+    P.max_ks.push_back(max_ks);
   }
+  P.item_begin.push_back((int)items.size());
+  P.d_units = upload(units);
+  try {
+    P.d_items = upload(items);
+  } catch (...) {
+    dev_free(P.d_units);
+    throw;
+  }
+  HB_CUDA(cudaStreamSynchronize(0));   // the host arrays end here
+  return P;
+}
+
+void task_plan_free(TaskPlan& P) {
+  dev_free(P.d_units);
+  dev_free(P.d_items);
+  P = TaskPlan{};
+}
+
+template <bool HALF, int W>
+static void launch_tasks(const TaskPlan& P, int step, const Task* tasks, const double2* F, double2* x, double2* y, double2* xh,
+                         int R, cudaStream_t st) {
+  const int n = P.item_begin[(size_t)step + 1] - P.item_begin[(size_t)step];
+  if (n <= 0) return;
+  const size_t frag = (size_t)std::min(TASK_KC, P.max_ks[(size_t)step]) * SPLIT_DIGITS * 32 * (HALF ? 2 : 4) * 4;
+  const size_t red = (size_t)(W - 1) * 32 * (HALF ? 4 : 8) * sizeof(longlong2);
+  const size_t smem = P.max_ks[(size_t)step] > 12 ? std::max(frag, red) : frag;
+  HB_CUDA(cudaFuncSetAttribute(task_kernel<HALF, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, 56 << 10));
+  task_kernel<HALF, W><<<n, 32 * W, smem, st>>>(P.d_items + P.item_begin[(size_t)step], P.d_units, tasks, F, x, y, xh, R);
   HB_CHECK_LAUNCH();
+}
+
+void run_tasks_fp64(const TaskPlan& P, int step, const Task* d_tasks, const double2* F, double2* x, double2* y,
+                    double2* xh, int R, cudaStream_t st) {
+  if (P.W == 4) {
+    if (R <= 8) launch_tasks<true, 4>(P, step, d_tasks, F, x, y, xh, R, st);
+    else launch_tasks<false, 4>(P, step, d_tasks, F, x, y, xh, R, st);
+  } else {
+    if (R <= 8) launch_tasks<true, 8>(P, step, d_tasks, F, x, y, xh, R, st);
+    else launch_tasks<false, 8>(P, step, d_tasks, F, x, y, xh, R, st);
+  }
 }
 
 namespace {
@@ -485,14 +573,20 @@ DenseOp dense_op(const double2* A, long long m, long long k, cudaStream_t st) {
     tasks.push_back(t);
   }
   D.ntask = (int)tasks.size();
-  D.shape = step_shape(tasks.data(), D.ntask);
-  D.d_tasks = upload(tasks, st);
+  D.plan = task_plan(tasks, {0, D.ntask}, 8);
+  try {
+    D.d_tasks = upload(tasks, st);
+  } catch (...) {
+    task_plan_free(D.plan);
+    throw;
+  }
   task_exponents(D.d_tasks, D.ntask, A, st);
   HB_CUDA(cudaStreamSynchronize(st));
   return D;
 }
 
 void dense_op_free(DenseOp& D) {
+  task_plan_free(D.plan);
   dev_free(D.d_tasks);
   D = DenseOp{};
 }
@@ -517,7 +611,7 @@ void dense_product(const DenseOp& D, const double2* X, long long ldx, double2* Y
   const VecGrid in(D.k, R), out(D.m, R);
   pack_rows_kernel<<<in.grid, in.block, 0, st>>>(X, ldx, D.k, R, alpha, x);
   HB_CHECK_LAUNCH();
-  run_tasks_fp64(D.d_tasks, D.ntask, D.shape, D.A, x, y, nullptr, R, st);
+  run_tasks_fp64(D.plan, 0, D.d_tasks, D.A, x, y, nullptr, R, st);
   sum_rows_kernel<<<out.grid, out.block, 0, st>>>(y, D.m, D.ntask, R, Y, ldy, accumulate);
   HB_CHECK_LAUNCH();
 }
@@ -530,8 +624,8 @@ void run_steps(hb_ctx* c, const double2* F, int nrhs, int dir, cudaStream_t st, 
     const int n = sb[s + 1] - sb[s];
     if (n == 0) continue;
     ts.begin(dir ? "bf_step_adjoint" : "bf_step");
-    run_tasks_fp64(c->d_tasks[dir] + sb[s], n, c->step_shapes[dir][s], F, (double2*)c->d_x, (double2*)c->d_y,
-                   (double2*)c->d_xh, nrhs, st);
+    run_tasks_fp64(c->task_plans[dir], (int)s, c->d_tasks[dir], F, (double2*)c->d_x, (double2*)c->d_y, (double2*)c->d_xh,
+                   nrhs, st);
     ts.end();
   }
 }
@@ -598,7 +692,7 @@ void shard_rows(const hb_ctx* c, int nranks, int rank, long long* lo, long long*
 namespace {
 struct ShardSteps {
   std::vector<int> begin;
-  std::vector<StepShape> shapes;
+  TaskPlan plan;
   Task* d_tasks = nullptr;
 };
 }  // namespace
@@ -620,11 +714,11 @@ static ShardSteps& shard_steps(hb_ctx* c, int dir, long long lo, long long hi) {
     }
   }
   S->begin.push_back((int)keep.size());
-  for (size_t q = 0; q + 1 < S->begin.size(); ++q)
-    S->shapes.push_back(step_shape(keep.data() + S->begin[q], S->begin[q + 1] - S->begin[q]));
   try {
+    S->plan = task_plan(keep, S->begin, 4);
     S->d_tasks = upload(keep);
   } catch (...) {
+    task_plan_free(S->plan);
     delete S;
     throw;
   }
@@ -635,6 +729,7 @@ static ShardSteps& shard_steps(hb_ctx* c, int dir, long long lo, long long hi) {
 void shard_cache_free(hb_ctx* c) {
   for (auto& kv : c->shard_cache) {
     ShardSteps* S = static_cast<ShardSteps*>(kv.second);
+    task_plan_free(S->plan);
     dev_free(S->d_tasks);
     delete S;
   }
@@ -687,8 +782,7 @@ void apply_bf_shard(hb_ctx* c, const double2* s, double2* u, int nrhs, int adjoi
       for (size_t q = 0; q + 1 < S.begin.size(); ++q) {
         const int n = S.begin[q + 1] - S.begin[q];
         if (n == 0) continue;
-        run_tasks_fp64(S.d_tasks + S.begin[q], n, S.shapes[q], c->d_f64, (double2*)c->d_x, (double2*)c->d_y,
-                       (double2*)c->d_xh, R, st);
+        run_tasks_fp64(S.plan, (int)q, S.d_tasks, c->d_f64, (double2*)c->d_x, (double2*)c->d_y, (double2*)c->d_xh, R, st);
       }
       const VecGrid vs(shi - slo, R);
       scatter_kernel<<<vs.grid, vs.block, 0, st>>>((double2*)c->d_y, c->d_perm, uc, c->Nv, R, slo, shi);

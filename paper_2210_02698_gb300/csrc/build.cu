@@ -26,6 +26,7 @@
 #include <chrono>
 #include <map>
 #include <cmath>
+#include <numeric>
 #include <vector>
 
 #ifdef _OPENMP
@@ -544,14 +545,21 @@ static void make_plans(hb_ctx* c, std::vector<Butterfly>& bfs, const std::vector
     std::vector<int> begins;
     for (size_t q = 0; q < steps.size(); ++q) {
       begins.push_back((int)c->tasks_h[dir].size());
-      c->tasks_h[dir].insert(c->tasks_h[dir].end(), steps[q].begin(), steps[q].end());
-      c->task_rows[dir].insert(c->task_rows[dir].end(), srows[q].begin(), srows[q].end());
+      // tasks that read the same inputs side by side
+      std::vector<int> order(steps[q].size());
+      std::iota(order.begin(), order.end(), 0);
+      std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+        return task_reads_before(steps[q][(size_t)a], steps[q][(size_t)b]);
+      });
+      for (int i : order) {
+        c->tasks_h[dir].push_back(steps[q][(size_t)i]);
+        c->task_rows[dir].push_back(srows[q][(size_t)i]);
+      }
     }
     begins.push_back((int)c->tasks_h[dir].size());
     c->step_begin[dir] = begins;
-    c->step_shapes[dir].clear();
-    for (size_t q = 0; q + 1 < begins.size(); ++q)
-      c->step_shapes[dir].push_back(step_shape(c->tasks_h[dir].data() + begins[q], begins[q + 1] - begins[q]));
+    task_plan_free(c->task_plans[dir]);
+    c->task_plans[dir] = task_plan(c->tasks_h[dir], begins, 4);
     // the factor exponents are found on the device and kept on both sides (a
     // shard uploads a part of the host list)
     c->d_tasks[dir] = upload(c->tasks_h[dir]);

@@ -45,7 +45,7 @@ struct CurveBfly {
   int L = 0;
   long long nrows = 0, ncols = 0, xh_rows = 0, entries = 0;
   std::vector<int> step_begin;
-  std::vector<StepShape> shapes;   // per step
+  TaskPlan plan;
   std::vector<int> max_rank;    // per butterfly level
   Task* d_tasks = nullptr;
   double2* d_F = nullptr;
@@ -59,6 +59,7 @@ struct CurveBfly {
 
 void free_bfly(CurveBfly* B) {
   if (!B) return;
+  task_plan_free(B->plan);
   for (void* p : {(void*)B->d_tasks, (void*)B->d_F, (void*)B->d_rperm, (void*)B->d_cperm, (void*)B->d_x,
                   (void*)B->d_y, (void*)B->d_xh})
     dev_free(p);
@@ -390,7 +391,9 @@ CurveBfly* build_bfly(const hb_ctx* c, const BfSide& R, const BfSide& C, int L) 
     B->entries = fbase;
     B->xh_rows = xh;
     B->step_begin = sb;
-    for (size_t q = 0; q + 1 < sb.size(); ++q) B->shapes.push_back(step_shape(tasks.data() + sb[q], sb[q + 1] - sb[q]));
+    for (size_t q = 0; q + 1 < sb.size(); ++q)
+      std::stable_sort(tasks.begin() + sb[q], tasks.begin() + sb[q + 1], task_reads_before);
+    B->plan = task_plan(tasks, sb, 8);
     B->d_tasks = upload(tasks);
     task_exponents(B->d_tasks, (int)tasks.size(), B->d_F, 0);
     B->d_rperm = upload(R.perm);
@@ -487,8 +490,7 @@ void curve_bf_apply(hb_ctx* c, int which, const double2* x_nat, long long ldx, d
                                                                scale, B->d_x);
     HB_CHECK_LAUNCH();
     for (size_t s = 0; s + 1 < B->step_begin.size(); ++s)
-      run_tasks_fp64(B->d_tasks + B->step_begin[s], B->step_begin[s + 1] - B->step_begin[s], B->shapes[s], B->d_F,
-                     B->d_x, B->d_y, B->d_xh, R, st);
+      run_tasks_fp64(B->plan, (int)s, B->d_tasks, B->d_F, B->d_x, B->d_y, B->d_xh, R, st);
     scatter_tree_kernel<<<grid_for(B->nrows * R), 256, 0, st>>>(B->d_y, B->d_rperm, B->nrows, R,
                                                                y_nat + (size_t)r0 * ldy, ldy, accumulate);
     HB_CHECK_LAUNCH();

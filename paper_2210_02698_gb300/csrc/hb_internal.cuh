@@ -126,10 +126,25 @@ struct Task {
   unsigned char conj_t, kind;
   int fe;                   // largest biased exponent of its factor blocks (task_exponents)
 };
-// The largest task of a step: outputs, and k-steps of 8 inputs (each term's
-// inputs rounded up).
-struct StepShape {
-  int max_out, max_ks;
+// The step tasks of a plan cut into CTAs (apply.cu): units (task, n-tile of 8
+// outputs), items (first unit, units) of tasks with the same inputs.  The
+// tasks of a step are in the order of task_reads_before.
+// Both hold what a CTA needs of the tasks: one load each ahead of the data.
+struct TaskUnit {
+  long long f_off[2], y_off;
+  int task, tile, r_out;
+  unsigned char conj_t, y_buf, accumulate, pad;
+};
+struct TaskItem {
+  long long x_off[2];
+  int unit0, units, r_in[2], x_buf, pad;
+};
+struct TaskPlan {
+  int W = 4;                       // warps per CTA
+  TaskUnit* d_units = nullptr;
+  TaskItem* d_items = nullptr;
+  std::vector<int> item_begin;     // items of step s: [item_begin[s], item_begin[s + 1])
+  std::vector<int> max_ks;         // k-steps of 8 inputs of a step's longest task
 };
 // A stored dense operator (m x k, column-major) as step tasks over ranges of
 // its inputs (apply.cu).
@@ -137,7 +152,7 @@ struct DenseOp {
   const double2* A = nullptr;
   long long m = 0, k = 0;
   int ntask = 0;
-  StepShape shape{0, 0};
+  TaskPlan plan;
   Task* d_tasks = nullptr;
 };
 
@@ -294,7 +309,7 @@ struct hb_ctx {
   long long* d_pperm = nullptr;       // padded row -> natural index (-1: padding)
   // apply plans: steps[0] forward, steps[1] adjoint; each step = task range
   std::vector<int> step_begin[2];
-  std::vector<hb::StepShape> step_shapes[2];
+  hb::TaskPlan task_plans[2];
   std::vector<hb::Task> tasks_h[2];
   std::vector<std::pair<long long, long long>> task_rows[2];   // tree-position rows each task serves
   hb::Task* d_tasks[2] = {nullptr, nullptr};
@@ -436,18 +451,21 @@ void curve_bf_free(hb_ctx* c);
 void curve_bf_info(const hb_ctx* c, int which, int* levels, int* max_rank, long long* entries);
 void curve_bf_apply(hb_ctx* c, int which, const double2* x_nat, long long ldx, double scale, double2* y_nat,
                     long long ldy, int accumulate, int nrhs, cudaStream_t st);
-// FP64 step tasks (apply.cu): the factor exponents of n tasks, the largest
-// task of a step, and one step
+// FP64 step tasks (apply.cu): the factor exponents of n tasks, the order of a
+// step's tasks, their CTAs (begin: the steps' task ranges; W = 4 warps, or 8
+// for few tasks with long sums), and one step
 void task_exponents(Task* d_tasks, int n, const double2* F, cudaStream_t st);
-StepShape step_shape(const Task* tasks, int n);
+bool task_reads_before(const Task& a, const Task& b);
+TaskPlan task_plan(const std::vector<Task>& tasks, const std::vector<int>& begin, int W);
+void task_plan_free(TaskPlan& P);
+void run_tasks_fp64(const TaskPlan& P, int step, const Task* d_tasks, const double2* F, double2* x, double2* y,
+                    double2* xh, int R, cudaStream_t st);
 // a stored dense operator as step tasks; Y = alpha A X (or +=) for R <= 16
 // columns, x / y: row-major operands (k x R and ntask m x R)
 DenseOp dense_op(const double2* A, long long m, long long k, cudaStream_t st);
 void dense_op_free(DenseOp& D);
 void dense_product(const DenseOp& D, const double2* X, long long ldx, double2* Y, long long ldy, int R, double alpha,
                    int accumulate, double2* x, double2* y, cudaStream_t st);
-void run_tasks_fp64(const Task* d_tasks, int n, const StepShape& shape, const double2* F, double2* x, double2* y,
-                    double2* xh, int R, cudaStream_t st);
 void curve_free(hb_ctx* c);
 void curve_operators(hb_ctx* c, double2* k_s2s, double2* k_v2s, double2* k_s2v, cudaStream_t st);
 void apply_inclusion(hb_ctx* c, const double2* s, double2* u, int nrhs, int v2v_dense, cudaStream_t st);

@@ -6,12 +6,14 @@
 // and Rump, Numer. Algorithms 59 (2012), with the digits of a common fixed
 // point, as in the integer form of Ootomo, Ozaki and Yokota, 2024).
 //
-// A block's values share one exponent: v = T 2^(E - 1081), E the largest
-// biased exponent of the block, |T| < 2^59 an integer (the 53-bit mantissa
-// shifted up by 6 and down by the exponent difference: a value within 2^6 of
-// the largest keeps every bit, and none is off by more than 2^-59 of the
+// A block's values share one exponent: |v| = T 2^(E - 1080), E the largest
+// biased exponent of the block, T < 2^58 an integer (the 53-bit mantissa
+// shifted up by 5 and down by the exponent difference: a value within 2^5 of
+// the largest keeps every bit, and none is off by more than 2^-58 of the
 // largest; a product rounded in FP64 is off by 2^-53 of itself).  T is written in six
-// balanced base-1024 digits d_0 .. d_5, |d| <= 512, exact in FP16:
+// balanced base-1024 digits d_0 .. d_5, |d| <= 512, exact in FP16 (the sign
+// goes on every digit; blocks too small for their zeros to shift out, E < 65,
+// and those with values that are not finite are left to plain sums):
 // T = sum d_s 2^(10 (5 - s)).  The product of two values is
 //   sum_{i,j} d_i d'_j 2^(100 - 10 (i + j)),
 // of which the 21 digit products with i + j <= 5 are formed (the rest is
@@ -34,39 +36,48 @@ namespace hb {
 
 constexpr int SPLIT_DIGITS = 6;
 constexpr int SPLIT_ACC = 7;             // accumulators: diagonals 0 .. 5, and diagonal 2's third product
-constexpr int SPLIT_EXP_BIAS = 1081;     // v = T 2^(E - 1081)
-constexpr int SPLIT_NONFINITE = 0x7ff;
+constexpr int SPLIT_EXP_BIAS = 1080;     // |v| = T 2^(E - 1080)
+constexpr int SPLIT_MIN_EXP = 65;
 
-__device__ __forceinline__ int biased_exponent(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
-// the exponent a block scales by: that of a value, subnormals as 1
+// the exponent a block scales by: 0 when all is zero (subnormals count as 1);
+// integer operations only (a comparison with 0.0 is the FP64 unit's)
 __device__ __forceinline__ int block_exponent(double2 v) {
-  return max(1, max(biased_exponent(v.x), biased_exponent(v.y)));
+  const unsigned a = (unsigned)__double2hiint(v.x) & 0x7fffffffu, b = (unsigned)__double2hiint(v.y) & 0x7fffffffu;
+  const unsigned e = max(a, b) >> 20;
+  const unsigned any = a | b | (unsigned)__double2loint(v.x) | (unsigned)__double2loint(v.y);
+  return (int)max(e, min(any, 1u));
 }
+__device__ __forceinline__ bool split_exponent_ok(int e) { return e == 0 || (e >= SPLIT_MIN_EXP && e < 0x7ff); }
 
-// T + 512 (1 + 2^10 + .. + 2^50): the digits plus 512, each in its 10 bits
+// T + 512 (1 + 2^10 + .. + 2^50): the digits plus 512, each in its 10 bits (the
+// top one at most 256 + 1); E >= 65, so that zero (read as 2^-1022) shifts out
 __device__ __forceinline__ unsigned long long fixed_biased(double v, int E) {
-  const int hi = __double2hiint(v);
-  const int e = (hi >> 20) & 0x7ff;
-  const unsigned long long m =
-      ((unsigned long long)(unsigned)((hi & 0xfffff) | (e ? 0x100000 : 0)) << 32) | (unsigned)__double2loint(v);
-  const int sh = min(E - max(e, 1), 63);
-  const long long T = (long long)((m << 6) >> sh);
-  const long long s = (long long)(hi >> 31);
-  constexpr long long B = 512LL * (1LL + (1LL << 10) + (1LL << 20) + (1LL << 30) + (1LL << 40) + (1LL << 50));
-  return (unsigned long long)(((T ^ s) - s) + B);
+  const unsigned hi = (unsigned)__double2hiint(v);
+  const int sh = min(E - (int)((hi >> 20) & 0x7ff), 63);
+  const unsigned long long m = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(v);
+  constexpr unsigned long long B = 512ULL * (1ULL + (1ULL << 10) + (1ULL << 20) + (1ULL << 30) + (1ULL << 40) + (1ULL << 50));
+  return ((m << 5) >> sh) + B;
 }
 
-// Digit s of (re, im) as a pair of FP16 values (re in the low half).
-__device__ __forceinline__ void split_pair(double re, double im, int E, uint32_t (&w)[SPLIT_DIGITS]) {
-  const unsigned long long a = fixed_biased(re, E), b = fixed_biased(im, E);
+// Digit s of v as a pair of FP16 values (re in the low half); im_flip =
+// 0x80000000 negates the imaginary part.  Most of the work is integer logic,
+// which this part issues at half the rate of its multiply-adds: the digits are
+// cut with one shift a part, a byte permutation and one logic operation, and
+// bias and sign go on in one packed FP16 multiply-add.
+__device__ __forceinline__ void split_pair(double2 v, int E, uint32_t im_flip, uint32_t (&w)[SPLIT_DIGITS]) {
+  const unsigned long long a = fixed_biased(v.x, E), b = fixed_biased(v.y, E);
+  // packed +-1 and -+1536
+  const uint32_t sg = (((uint32_t)__double2hiint(v.x) >> 16) & 0x8000u) |
+                      (((uint32_t)__double2hiint(v.y) ^ im_flip) & 0x80000000u);
+  const uint32_t one = 0x3c003c00u ^ sg, off = 0xe600e600u ^ sg;
 #pragma unroll
   for (int s = 0; s < SPLIT_DIGITS; ++s) {
     const int p = 10 * (5 - s);
-    const uint32_t mask = s == 0 ? 0x7ffu : 0x3ffu;   // the top digit plus 512 may reach 1024
-    const uint32_t u = ((uint32_t)(a >> p) & mask) | (((uint32_t)(b >> p) & mask) << 16);
-    // 0x6400 + u is the FP16 value 1024 + u (u <= 1024); minus 1536 leaves the digit
-    const uint32_t h = u + 0x64006400u, c = 0x66006600u;
-    asm("sub.f16x2 %0, %1, %2;" : "=r"(w[s]) : "r"(h), "r"(c));
+    const uint32_t x = (uint32_t)(a >> p);
+    const uint32_t y = p < 16 ? (uint32_t)b << (16 - p) : (uint32_t)(b >> (p - 16));
+    // 0x6400 + u is the FP16 value 1024 + u; minus 1536 leaves the digit
+    const uint32_t h = (__byte_perm(x, y, 0x7610) & 0x03ff03ffu) | 0x64006400u;
+    asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(w[s]) : "r"(h), "r"(one), "r"(off));
   }
 }
 
