@@ -85,11 +85,6 @@ __device__ __forceinline__ void st_global_hint(uint4* p, const uint4& v, uint64_
 // cp.async (generic proxy, L2 only): 16 bytes global -> shared, grouped by
 // commit_group; wait_pending(n) waits until at most n groups of the thread
 // are still in flight (n > 3 waits as for 3)
-// 16 bytes, or zeros (the source is then not read)
-__device__ __forceinline__ void cp_async16_or_zero(void* dst, const void* src, bool ok) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(ok ? 16 : 0)
-               : "memory");
-}
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }

@@ -174,6 +174,7 @@ void setup_tables(hb_ctx* c) {
 // Hankel expansions of the dense apply.
 void compute_self(hb_ctx* c) {
   if (!c->d_self) c->d_self = dev_alloc<double2>(c->Nv);
+  if (!c->d_dense_ex) c->d_dense_ex = dev_alloc<int>(17);
   // the expansions of the Hankel pair up to the largest omega tau of the
   // tables (and a tenth of tau^2 more, for cells outside the node hull; past
   // the rows the kernels use the asymptotic series)
@@ -186,7 +187,7 @@ void compute_self(hb_ctx* c) {
   c->hank_top = 0.0f;
   if (nrow > 0) {
     c->d_hank = dev_alloc<double2>((size_t)nrow * HT_ROW);
-    hankel_table_kernel<<<(nrow + 127) / 128, 128>>>(c->d_hank, nrow);
+    hankel_table_kernel<<<(nrow + 31) / 32, 32>>>(c->d_hank, nrow);   // one warp an SM: a serial FP64 chain a row
     HB_CHECK_LAUNCH();
     c->hank_top = (float)top;
   }
@@ -226,6 +227,9 @@ EntryParams entry_params(const hb_ctx* c, int transposed) {
 }
 
 // ------------------------------------------------------- dense apply ----
+// The form in plain FP64 FMAs, for values that the digits of dense_split.cu do
+// not hold (not finite, or below 2^-960): it runs when that kernel's flag is up.
+//
 // One CTA owns the L <= 64 cells of one segment of a grid line (the outputs; a
 // line is cut into equal segments) and sweeps the source line segments of L
 // cells of its share of the source lines (blockIdx.y of gridDim.y contiguous
@@ -239,17 +243,17 @@ EntryParams entry_params(const hb_ctx* c, int transposed) {
 // observation contraction (the basis values in registers, the source's P
 // broadcast from shared memory), 27 for the Hankel pair (hankel_table.cuh)
 // and 4 RC.  sqrt(pi)/2 and the factors of f1 are folded into P.  Measured:
-// 64^2, one right-hand side 55 -> 3.3 ms, 144 x 100 with 16 (adjoint) 435 ->
-// 62 ms against the evaluation by recurrences with the basis in shared memory
-// (stride of 128 bytes: every lane on one bank).
+// 64^2, one right-hand side 3.3 ms, 144 x 100 with 16 (adjoint) 62 ms.
 constexpr int DT = 64;
 constexpr double HB_C0 = 0.88622692545275801365;   // sqrt(pi)/2
 
 template <int RC, bool ADJ, int KI>
 __global__ void __launch_bounds__(256, RC <= 4 ? 2 : 1) dense_kernel(EntryParams p, const double2* __restrict__ s,
                                                     double2* __restrict__ u, long long Nv, int L, int r0,
-                                                    double scale, double2* __restrict__ part) {
+                                                    double scale, double2* __restrict__ part,
+                                                    const int* __restrict__ flag) {
   extern __shared__ double smem[];
+  if (!*flag) return;   // the digit form (dense_split.cu) holds
   const int nI = p.nI;
   double* M = smem;                           // 3 x KI x KI
   double* P = M + 3 * KI * KI;                // 3 x DT x KI
@@ -266,7 +270,7 @@ __global__ void __launch_bounds__(256, RC <= 4 ? 2 : 1) dense_kernel(EntryParams
   const int grp = t / L;
   const bool active = grp < ngr && o < olen;
   const long long onat = (long long)bo * p.nx + ao0 + o;
-  const double w2 = p.omega * p.omega;
+  const double w2 = p.omega * p.omega, w2l = fma(p.omega, p.omega, -w2);
   const double c1 = 2.0 * HB_C0 / w2;
 
   double lxo[KI];
@@ -331,7 +335,7 @@ __global__ void __launch_bounds__(256, RC <= 4 ? 2 : 1) dense_kernel(EntryParams
             g = p.self[onat];
           } else {
             // g = i v0 H0 - i v1 x H1 (the constants are in P)
-            const HankelFG h = hankel_of_t2(p.hank, w2, f[0]);
+            const HankelFG h = hankel_of_t2(p.hank, w2, w2l, f[0]);
             g = make_double2(fma(-h.F.y, f[1], h.G.y * f[2]), fma(h.F.x, f[1], -h.G.x * f[2]));
           }
           if (ADJ) g.y = -g.y;
@@ -368,8 +372,10 @@ __global__ void __launch_bounds__(256, RC <= 4 ? 2 : 1) dense_kernel(EntryParams
 }
 
 // u[r0 + r][cell] = scale * (sum over the shares, in order, of part[share][r][cell])
+// (when the flag equals want: both forms of the apply write the shares)
 __global__ void dense_reduce_kernel(const double2* __restrict__ part, double2* __restrict__ u, long long Nv, int rc,
-                                    int nsplit, int r0, double scale) {
+                                    int nsplit, int r0, double scale, const int* __restrict__ flag, int want) {
+  if ((*flag != 0) != (want != 0)) return;
   const long long n = Nv * rc;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     double2 a = make_double2(0.0, 0.0);
@@ -385,35 +391,68 @@ __global__ void dense_reduce_kernel(const double2* __restrict__ part, double2* _
 
 template <int RC, bool ADJ, int KI>
 static void launch_dense(const EntryParams& p, const double2* s, double2* u, long long Nv, int L, int r0,
-                         double scale, int nsplit, double2* part, cudaStream_t st) {
+                         double scale, int nsplit, double2* part, const int* flag, cudaStream_t st) {
   size_t sm = sizeof(double) * (3 * KI * KI + 3 * DT * KI) + sizeof(double2) * (DT + 256) * RC;
   auto k = dense_kernel<RC, ADJ, KI>;
   HB_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   const int ntx = (p.nx + L - 1) / L;
-  k<<<dim3(ntx * p.ny, nsplit), 256, sm, st>>>(p, s, u, Nv, L, r0, scale, nsplit > 1 ? part : nullptr);
+  k<<<dim3(ntx * p.ny, nsplit), 256, sm, st>>>(p, s, u, Nv, L, r0, scale, nsplit > 1 ? part : nullptr, flag);
   HB_CHECK_LAUNCH();
   if (nsplit > 1) {
     const long long n = Nv * RC;
     dense_reduce_kernel<<<(unsigned)std::min<long long>((n + 255) / 256, 152LL * 8), 256, 0, st>>>(
-        part, u, Nv, RC, nsplit, r0, scale);
+        part, u, Nv, RC, nsplit, r0, scale, flag, 1);
     HB_CHECK_LAUNCH();
   }
+}
+
+// the FP64 form for rc right-hand sides from r0 on, in passes of 16, 8, 4, 2 and 1
+static void dense_plain(const EntryParams& p, const double2* s, double2* u, long long Nv, int L, int r0, int rc, int adjoint,
+                        double scale, int nsplit, double2* part, const int* flag, cudaStream_t st) {
+#define HB_DENSE_LAUNCH(R, A, K) launch_dense<R, A, K>(p, s, u, Nv, L, r0, scale, nsplit, part, flag, st)
+#define HB_DENSE_CASE(R)                        \
+  for (; rc >= R; rc -= R, r0 += R) {           \
+    if (p.nI <= 8) {                            \
+      if (adjoint) HB_DENSE_LAUNCH(R, true, 8); \
+      else HB_DENSE_LAUNCH(R, false, 8);        \
+    } else {                                    \
+      if (adjoint) HB_DENSE_LAUNCH(R, true, 16);\
+      else HB_DENSE_LAUNCH(R, false, 16);       \
+    }                                           \
+  }
+  HB_DENSE_CASE(16)
+  HB_DENSE_CASE(8)
+  HB_DENSE_CASE(4)
+  HB_DENSE_CASE(2)
+  HB_DENSE_CASE(1)
+#undef HB_DENSE_CASE
+#undef HB_DENSE_LAUNCH
 }
 
 void dense_apply(hb_ctx* c, const double2* s, double2* u, int nrhs, int adjoint, cudaStream_t st) {
   NvtxRange nr(adjoint ? "hb_apply_dense_adjoint" : "hb_apply_dense");
   EntryParams p = entry_params(c, adjoint);
   const double scale = c->h * c->h;
-  // small grids give few output CTAs: split the source lines into shares so
-  // that there are at least eight CTAs per SM (the entry evaluation is
-  // latency-bound FP64 work)
+  // small grids give few output CTAs: split the source lines into shares, up
+  // to eight CTAs per SM; of the counts that give, the one that leaves the
+  // least of the last wave (one CTA an SM) and of the longest share idle
   int dev = 0, nsm = 0;
   HB_CUDA(cudaGetDevice(&dev));
   HB_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
   // equal segments of at most DT cells: a ragged last segment would idle threads
   const int L = (p.nx + (p.nx + DT - 1) / DT - 1) / ((p.nx + DT - 1) / DT);
   const long long cta = (long long)((p.nx + L - 1) / L) * p.ny;
-  const int nsplit = (int)std::max<long long>(1, std::min<long long>(p.ny, (8LL * nsm + cta - 1) / cta));
+  const int most = (int)std::max<long long>(1, std::min<long long>(p.ny, (8LL * nsm + cta - 1) / cta));
+  int nsplit = 1;
+  double best = 0.0;
+  for (int k = 1; k <= most; ++k) {
+    const double waves = (double)((cta * k + nsm - 1) / nsm), share = (double)((p.ny + k - 1) / k);
+    const double eff = (double)(cta * p.ny) / (waves * nsm * (share + 0.1));   // a tenth of a line to set a CTA up
+    if (eff > best) {
+      best = eff;
+      nsplit = k;
+    }
+  }
   if (nsplit > 1) {
     const size_t need = (size_t)nsplit * 16 * (size_t)c->Nv;
     if (c->dense_part_cap < need) {
@@ -424,31 +463,20 @@ void dense_apply(hb_ctx* c, const double2* s, double2* u, int nrhs, int adjoint,
       c->dense_part_cap = need;
     }
   }
-  int r0 = 0;
-  while (r0 < nrhs) {
-    int left = nrhs - r0;
-    int rc = left >= 16 ? 16 : left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
-#define HB_DENSE_LAUNCH(R, A, K) launch_dense<R, A, K>(p, s, u, c->Nv, L, r0, scale, nsplit, c->d_dense_part, st)
-#define HB_DENSE_CASE(R)                                              \
-  case R:                                                             \
-    if (p.nI <= 8) {                                                  \
-      if (adjoint) HB_DENSE_LAUNCH(R, true, 8);                       \
-      else HB_DENSE_LAUNCH(R, false, 8);                              \
-    } else {                                                          \
-      if (adjoint) HB_DENSE_LAUNCH(R, true, 16);                      \
-      else HB_DENSE_LAUNCH(R, false, 16);                             \
-    }                                                                 \
-    break;
-    switch (rc) {
-      HB_DENSE_CASE(16)
-      HB_DENSE_CASE(8)
-      HB_DENSE_CASE(4)
-      HB_DENSE_CASE(2)
-      HB_DENSE_CASE(1)
+  // passes of up to 16 right-hand sides on the tensor cores; behind each the
+  // FP64 kernel, which runs where the digits did not hold the values
+  double2* part = nsplit > 1 ? c->d_dense_part : nullptr;
+  const int* flag = c->d_dense_ex + 16;
+  for (int r0 = 0; r0 < nrhs; r0 += 16) {
+    const int rc = std::min(nrhs - r0, 16);
+    dense_split(p, s, u, c->Nv, L, nsplit, r0, rc, adjoint, scale, part, c->d_dense_ex, st);
+    if (nsplit > 1) {
+      const long long n = c->Nv * rc;
+      dense_reduce_kernel<<<(unsigned)std::min<long long>((n + 255) / 256, 152LL * 8), 256, 0, st>>>(
+          part, u, c->Nv, rc, nsplit, r0, scale, flag, 0);
+      HB_CHECK_LAUNCH();
     }
-#undef HB_DENSE_CASE
-#undef HB_DENSE_LAUNCH
-    r0 += rc;
+    dense_plain(p, s, u, c->Nv, L, r0, rc, adjoint, scale, nsplit, part, flag, st);
   }
 }
 

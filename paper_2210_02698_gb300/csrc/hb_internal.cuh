@@ -336,6 +336,7 @@ struct hb_ctx {
   // dense apply: per-split partial sums when source lines are split over CTAs
   double2* d_dense_part = nullptr;
   size_t dense_part_cap = 0;
+  int* d_dense_ex = nullptr;   // dense apply: exponents of 16 right-hand sides, the flag of dense_split.cu
 
   // curve inclusion (inclusion.cu): segments and the dense surface operators
   long long ns = 0;                // segments; 0: no curve set
@@ -380,6 +381,8 @@ void sweep_tables(int M, double lo, double h, int w0, int w1, int roi0, int roi1
                   double tol, double* tau2, double* v0, double* v1, double* info);
 void sweep_taylor_one(const double* s2, double* out);
 void dense_apply(hb_ctx* c, const double2* s, double2* u, int nrhs, int adjoint, cudaStream_t st);
+void dense_split(const EntryParams& p, const double2* s, double2* u, long long Nv, int L, int nsplit, int r0, int rc,
+                 int adjoint, double scale, double2* part, int* exs, cudaStream_t st);   // dense_split.cu
 void eval_entries(hb_ctx* c, const long long* rows, int m, const long long* cols, int n,
                   double2* out, cudaStream_t st);
 void add_block(BlockBatchHost& B, const hb_ctx* c, const long long* rows, long long m,

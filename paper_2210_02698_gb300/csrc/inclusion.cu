@@ -117,8 +117,8 @@ __global__ void __launch_bounds__(128) seg_contract_kernel(PointTables P, const 
 // dense apply): i c (v0 H0 - (2 / w^2) v1 x H1)
 __device__ __forceinline__ double2 green_tab(const HankelTable& T, double omega, double t2, double v0, double v1) {
   const double c = 0.88622692545275801365;   // sqrt(pi)/2
-  const double w2 = omega * omega;
-  const HankelFG h = hankel_of_t2(T, w2, t2);
+  const double w2 = omega * omega, w2l = fma(omega, omega, -w2);
+  const HankelFG h = hankel_of_t2(T, w2, w2l, t2);
   const double a = c * v0, b = (2.0 * c / w2) * v1;
   return make_double2(fma(-h.F.y, a, h.G.y * b), fma(h.F.x, a, -h.G.x * b));
 }

@@ -47,3 +47,44 @@ def test_dense_apply_equals_the_entries(nx, ny, n_I, omega, nrhs):
     for got, want in ((u, h2 * (s @ K)), (a, h2 * (s @ K.mH))):
         assert float(torch.linalg.norm(got - want) / torch.linalg.norm(want)) < tol
     op.close()
+
+
+@pytest.mark.parametrize("nrhs", [3, 18])
+def test_right_hand_sides_outside_the_digits(nrhs):
+    """Columns that are all zero, tiny (1e-300), huge, or hold a value that is
+    not finite: the last fails the digits and the whole apply is summed in
+    FP64; every column equals the product with the entries."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2210_02698_gb300 import build
+    build.build()
+    op = _operator(20, 9, 6, 17.0)
+    nv = 180
+    K = torch.empty((nv, nv), dtype=torch.complex128, device="cuda")
+    op.entries(np.arange(nv), np.arange(nv), K)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    s = torch.randn((nrhs, nv), dtype=torch.complex128, device="cuda", generator=g)
+    s[0] = 0
+    s[-1] *= 1e250
+    for last in (1e-300, 1e-290, complex("nan"), complex("inf")):
+        s[1] = torch.randn(nv, dtype=torch.complex128, device="cuda", generator=g)
+        if np.isfinite(last):
+            s[1] *= last
+        else:
+            s[1, 77] = last
+        for fn, A in ((op.apply_dense, K), (op.apply_dense_adjoint, K.mH)):
+            u = torch.full_like(s, 7.0)
+            fn(s, u, nrhs)
+            torch.cuda.synchronize()
+            assert not u[0].any()
+            for k in range(1, nrhs):
+                if k == 1 and not np.isfinite(last):
+                    assert not torch.isfinite(torch.view_as_real(u[1])).all(-1).any()
+                    continue
+                w = abs(last) if k == 1 else 1e250 if k == nrhs - 1 else 1.0
+                want = op.h ** 2 * ((s[k] / w) @ A)
+                # the entries: as above; a column at 1e-300 is summed in subnormals' neighbourhood, 1e-308 / 1e-300 of it
+                tol = 1e-7 if w < 1e-280 else 1e-12
+                assert float(torch.linalg.norm(u[k] / w - want) / torch.linalg.norm(want)) < tol
+    op.close()
