@@ -21,7 +21,7 @@ def _built():
     build.build()
 
 
-@pytest.mark.parametrize("N,ns,nrhs", [(10, 1, 1), (19, 65, 3), (33, 200, 9), (40, 31, 16), (24, 130, 35)])
+@pytest.mark.parametrize("N,ns,nrhs", [(10, 1, 1), (19, 65, 3), (33, 200, 9), (40, 31, 16), (24, 130, 35), (12, 1300, 2)])
 def test_inclusion_equals_its_operators(N, ns, nrhs):
     import torch
     from paper_2210_02698_gb300 import binding
