@@ -27,10 +27,10 @@
 // and a lane's four entries g(o, c) are its four words of the A fragment of
 // the sum.  Running sums are 64-bit integer pairs at the largest exponent met.
 //
-// Bound by the FP64 unit still (63 % busy at 64^2, 8 warps an SM): the Hankel
+// Bound by the FP64 unit still (63 % busy at 64^2 with 8 warps an SM): the Hankel
 // pairs.  Measured, evaluation entry by entry through recurrences / plain FP64
 // with tabulated pairs (entries.cu) / this: 64^2, one right-hand side 53.4 /
-// 3.4 / 2.05 ms; 144 x 100, 16 right-hand sides (adjoint) 435 / 62 / 22.9 ms.
+// 3.4 / 1.97 ms; 144 x 100, 16 right-hand sides (adjoint) 435 / 62 / 22.9 ms.
 //
 // Values that are not finite, or too small for the digits (split_fixed.cuh),
 // raise *flag; the FP64 kernel of entries.cu, launched behind this one, then
@@ -434,8 +434,11 @@ void launch(const EntryParams& p, const double2* s, double2* u, long long Nv, in
             double2* part, const int* exs, int* flag, cudaStream_t st) {
   const int nmt = (L + 15) / 16;
   const int segs = (p.nx + 8 * DS_NT - 1) / (8 * DS_NT), LQ = (p.nx + segs - 1) / segs;
-  // three m-tiles need twelve warps to give every sub-partition of the SM as many
-  const int warps = nmt == 3 ? 12 : 8;
+  // twelve warps (all the registers hold) where the segment has three or four
+  // m-tiles: eight leave three m-tiles unevenly spread over the SM's
+  // sub-partitions, and 64^2 2.05 -> 1.97 ms, 120 x 100 16.6 -> 14.7, 100 x 80 x 5
+  // 9.25 -> 8.45; below that level (24^2), or slower (32^2 x 16: 384 -> 392 us)
+  const int warps = nmt >= 3 ? 12 : 8;
   const DsLayout Y(nmt, (LQ + 7) / 8, RT);
   const size_t red = (size_t)(warps / nmt) * nmt * RT * 4 * 32 * sizeof(double2);
   const size_t smem = std::max((size_t)Y.words * 4, red);
