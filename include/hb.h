@@ -81,9 +81,9 @@ typedef struct {
  * uniform proxy rows and nbr_radius_h: neighbour radius in units of h
  * (Eq. proxyv2v); precision: HB_FP64 or HB_MIXED_BF16X3 for hb_apply /
  * hb_apply_adjoint; workspace_mb: device workspace bound for the build
- * (0 = default); barrier_cycles: spin budget (SM clock cycles, counted from
- * the start of each kernel) of the bounded device waits of the mixed apply
- * (0 = default, 2^31).  A wait that runs out sets a mapped error word; the
+ * (0 = default); barrier_cycles: spin budget (SM clock cycles, counted in each
+ * launch from the moment it sees its predecessor complete) of the bounded
+ * device waits of the mixed apply (0 = default, 2^31).  A wait that runs out sets a mapped error word; the
  * kernel then lets its copies in flight land (waiting at least 2^31 cycles
  * for them) and stops; a later hb_apply / hb_apply_adjoint on the handle,
  * called once the device has run the apply that ran out, returns

@@ -196,7 +196,12 @@ __global__ void __launch_bounds__(TC_WARPS * 32, 1) bf_leaf_tc_kernel(TcArgs a) 
   volatile int* abf = &abort_flag;
   const long long i0 = a.ioff[blockIdx.x], i1 = a.ioff[blockIdx.x + 1];
   const long long c0 = a.coff[blockIdx.x], c1 = a.coff[blockIdx.x + 1];
-  const long long deadline = clock64() + a.budget;
+  // The launch may begin while earlier depths still run.  Warp 0 fetches its
+  // first factor runs meanwhile and waits for them below; the other warps have
+  // nothing to do before its input runs land.  The budget of the waits counts
+  // from there: what earlier depths take is not this launch's.
+  if (warp != 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  long long deadline = clock64() + a.budget;
 
   if (warp == 0) {
     // records: lane j holds record 32 w + j of the next window in registers;
@@ -232,6 +237,7 @@ __global__ void __launch_bounds__(TC_WARPS * 32, 1) bf_leaf_tc_kernel(TcArgs a) 
           asm volatile("griddepcontrol.wait;" ::: "memory");
           asm volatile("fence.proxy.async.global;" ::: "memory");
           waited = true;
+          deadline = clock64() + a.budget;
           for (int t = 0; t < nst; ++t)
             tma_load_1d(smem + (size_t)t * a.stage_bytes + (uint32_t)slot[t].nkg * TC_FKG, x_src(slot[t]),
                         (uint32_t)slot[t].nkg * XKG, &full[t], pol_v);
