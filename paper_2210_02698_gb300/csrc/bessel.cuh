@@ -86,12 +86,13 @@ static __constant__ BesselConsts g_bessel = bessel_consts();
 // the warp (constants, no conversions), divisions by small integers as
 // above and no FP64 comparisons.
 
-// Lanes start at their own M: before it their sums stay zero.
+// Lanes start at their own M <= 66 and skip the orders above it; the count is
+// every lane's (no exchange between lanes: the calls stand in branches), and
+// orders that no lane has reached cost a few integer instructions.
 __device__ __forceinline__ Bessel01 bessel01_miller_dev(double x) {
   const int M = 2 * (int)(0.8 * x + 13.0);
-  const int top = __reduce_max_sync(__activemask(), M);
   const double two_over_x = 2.0 / x;
-  double tp1 = 0.0, t = 0.0, norm = 0.0, sy0 = 0.0, sy1 = 0.0, t1 = 0.0;
+  double tp1 = 0.0, t = 1e-30, norm = 0.0, sy0 = 0.0, sy1 = 0.0, t1 = 0.0;
   const long long big = __double_as_longlong(1e250);
   auto step = [&](int n) {
     const double tm1 = __fma_rn(__dmul_rn(g_bessel.dk[n], two_over_x), t, -tp1);
@@ -102,9 +103,9 @@ __device__ __forceinline__ Bessel01 bessel01_miller_dev(double x) {
     }
   };
 #pragma unroll 1
-  for (int k = top >> 1; k >= 1; --k) {
+  for (int k = (BESSEL_K - 1) / 2; k >= 1; --k) {
+    if (2 * k > M) continue;
     // order 2k
-    if (2 * k == M) t = 1e-30;
     norm = __fma_rn(2.0, t, norm);
     const double q = div_by(t, g_bessel.dk[k], g_bessel.rk[k]);
     sy0 = __dadd_rn(sy0, (k & 1) ? -q : q);
