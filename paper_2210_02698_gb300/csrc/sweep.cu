@@ -147,11 +147,12 @@ __device__ __forceinline__ void weno_pair(const double* u, double h, double rh, 
   *dp = weno5(d[5], d[4], d[3], d[2], d[1], kp);
 }
 
-// The derivatives at one point along both axes, for every thread that takes
-// the point: p- = m[0], p+ = p[0] (x), q- = m[1], q+ = p[1] (z), and their
-// weights km, kp.  (Updated points are at least SW_EDGE = 3 off the edge: the
+// The value c at one point and the derivatives along both axes, for every thread
+// that takes the point: p- = m[0], p+ = p[0] (x), q- = m[1], q+ = p[1] (z), and
+// their weights km, kp.  (Updated points are at least SW_EDGE = 3 off the edge: the
 // stencils stay on the mesh.)
 struct Derivs {
+  double c;
   double m[2], p[2], km[2], kp[2];
 };
 
@@ -163,6 +164,7 @@ __device__ __forceinline__ void derivs_one(const double* c, int M, double h, dou
 #pragma unroll
     for (int k = 0; k < 7; ++k) u[k] = fld(c + (ptrdiff_t)(k - 3) * (ax ? M : 1));
     weno_pair(u, h, rh, &D.m[ax], &D.p[ax], &D.km[ax], &D.kp[ax]);
+    D.c = u[3];
   }
 }
 
@@ -170,12 +172,16 @@ __device__ __forceinline__ void derivs_one(const double* c, int M, double h, dou
 // axis).  A warp's FP64 instruction takes 64 cycles of its sub-partition's unit
 // whatever the other sub-partitions do, so a short anti-diagonal is
 // faster on four times the warps, each with a third of the instructions.
+// The point is read once, with the stencil, and every lane's reads come before
+// the barrier: the first lane then stores the updated value.
 __device__ __forceinline__ void derivs_quad(const double* c, int M, double h, double rh, int lane, Derivs& D) {
   const bool plus = lane & 1, z = lane & 2;
   const ptrdiff_t st = (z ? M : 1) * (plus ? -1 : 1);
   double w[6];
 #pragma unroll
   for (int k = 0; k < 6; ++k) w[k] = fld(c + (k - 3) * st);
+  D.c = w[3];
+  __syncwarp();
   double v[5];
 #pragma unroll
   for (int k = 0; k < 5; ++k) {
@@ -411,7 +417,7 @@ __global__ void __launch_bounds__(SW_THREADS, 2) sweep_kernel(SweepArgs a, int n
     if (!QUAD && !live) return;
     Derivs D;
     derivs(tb + p, M, D);
-    const double c = fld(tb + p), alpha = fld(tt + p), gxp = fld(gx + p), gzp = fld(gz + p);
+    const double c = D.c, alpha = fld(tt + p), gxp = fld(gx + p), gzp = fld(gz + p);
     const double A = alpha * 0.5 * (D.m[0] + D.p[0]) + c * gxp;
     const double B = alpha * 0.5 * (D.m[1] + D.p[1]) + c * gzp;
     const double H = sqrt(A * A + B * B);
@@ -487,7 +493,7 @@ __global__ void __launch_bounds__(SW_THREADS, 2) sweep_kernel(SweepArgs a, int n
       if (!QUAD && !live) return;
       Derivs D;
       derivs(v + p, Mw, D);
-      const double ap = fld(ax + p), bp = fld(az + p), lp = fld(lt + p), np = fld(nw + p), vp = fld(v + p);
+      const double ap = fld(ax + p), bp = fld(az + p), lp = fld(lt + p), np = fld(nw + p), vp = D.c;
       const double c = s == 0 ? lp - 4.0 * np * np : lp;
       const double f = s == 0 ? 0.0 : fld(rhs + p);
       const double alx = 2.0 * fabs(ap), alz = 2.0 * fabs(bp);
