@@ -177,8 +177,13 @@ hb_status hb_build(hb_handle h);
  * a previous hb_build (the handle is then unbuilt: call hb_build again
  * before hb_apply) and assembles a curve set with hb_curve_set again at the
  * new frequency (its compressed operators of hb_curve_compress are dropped).  The result equals a handle created at omega with the same
- * tables.  Synchronous.  Errors: HB_ERR_ARG (null handle, omega <= 0 or not
- * finite), HB_ERR_OOM, HB_ERR_CUDA. */
+ * tables.  When it returns HB_ERR_OOM before the curve is assembled, the
+ * handle keeps its old frequency, unbuilt and without a curve; when the curve
+ * does not fit, it has moved and has no curve.  Either way the call may be
+ * repeated.  Expansions of the Hankel pair (240 bytes for each 1/64 of omega
+ * tau, at most 31 MB, or 62 MB after frequencies have grown) stay with the
+ * handle until hb_destroy.  Synchronous.  Errors: HB_ERR_ARG (null handle,
+ * omega <= 0 or not finite), HB_ERR_OOM, HB_ERR_CUDA. */
 hb_status hb_set_omega(hb_handle h, double omega);
 
 /* hb_apply: u = K (h^2 s) with the compressed operator (Eq. butterfly_mat

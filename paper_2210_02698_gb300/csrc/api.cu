@@ -115,6 +115,7 @@ void free_all(hb_ctx* c) {
                   (void*)c->d_mxh, c->d_x, c->d_y, (void*)c->d_dense_part, (void*)c->d_flags, (void*)c->d_mx_tc,
                   (void*)c->d_tc[0], (void*)c->d_tc[1]})
     hb::dev_free(p);
+  for (double2* p : c->hank_old) hb::dev_free(p);
   hb::dev_free(c->d_xh);
   hb::dev_free(c->d_tasks[0]);
   hb::dev_free(c->d_tasks[1]);
@@ -329,8 +330,14 @@ hb_status hb_set_omega(hb_handle h, double omega) {
     }
     release_build(h);
     hb::curve_free(h);
+    const double was = h->omega;
     h->omega = omega;
-    hb::compute_self(h);
+    try {
+      hb::compute_self(h);
+    } catch (...) {   // the self terms are still those of the old frequency
+      h->omega = was;
+      throw;
+    }
     if (ns > 0) hb::curve_set(h, cen.data(), len.data(), nseg.data(), ns);
   });
 }

@@ -169,9 +169,31 @@ void setup_tables(hb_ctx* c) {
   compute_self(c);
 }
 
+// At least `need` rows of Hankel expansions.  A row depends on its place alone,
+// so an array serves every frequency that it is long enough for; a longer one
+// (at least twice, up to HT_CAP: no more than 62 MB in all) takes its place
+// and the outgrown one stays until the handle is destroyed, for graphs that
+// were captured with it.
+static void hankel_rows(hb_ctx* c, int need) {
+  if (need <= c->hank_rows) return;
+  const int most = (int)std::ceil((HT_CAP - HT_LO) * HT_PER) + 2;
+  const int rows = std::max(need, std::min(2 * c->hank_rows, most));
+  c->hank_old.reserve(c->hank_old.size() + 1);
+  double2* d = dev_alloc<double2>((size_t)rows * HT_ROW);
+  hankel_table_kernel<<<(rows + 31) / 32, 32>>>(d, rows);   // one warp an SM: a serial FP64 chain a row
+  if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
+    dev_free(d);
+    throw Error{HB_ERR_CUDA, "the Hankel expansions could not be computed"};
+  }
+  if (c->d_hank) c->hank_old.push_back(c->d_hank);
+  c->d_hank = d;
+  c->hank_rows = rows;
+}
+
 // The precomputed entry data that depends on omega (the tables do not): the
 // cell-integrated self terms into d_self (allocated on first use) and the
-// Hankel expansions of the dense apply.
+// Hankel expansions of the dense apply.  What can fail for lack of memory
+// comes before anything that the handle uses changes.
 void compute_self(hb_ctx* c) {
   if (!c->d_self) c->d_self = dev_alloc<double2>(c->Nv);
   if (!c->d_dense_ex) c->d_dense_ex = dev_alloc<int>(17);
@@ -181,16 +203,7 @@ void compute_self(hb_ctx* c) {
   double t2max = 0.0;
   for (double v : c->tab[0]) t2max = std::max(t2max, v);
   const double top = std::min(HT_CAP, c->omega * std::sqrt(1.1 * t2max) + 1.0);
-  const int nrow = top > HT_LO ? (int)std::ceil((top - HT_LO) * HT_PER) + 2 : 0;
-  dev_free(c->d_hank);
-  c->d_hank = nullptr;
-  c->hank_top = 0.0f;
-  if (nrow > 0) {
-    c->d_hank = dev_alloc<double2>((size_t)nrow * HT_ROW);
-    hankel_table_kernel<<<(nrow + 31) / 32, 32>>>(c->d_hank, nrow);   // one warp an SM: a serial FP64 chain a row
-    HB_CHECK_LAUNCH();
-    c->hank_top = (float)top;
-  }
+  hankel_rows(c, top > HT_LO ? (int)std::ceil((top - HT_LO) * HT_PER) + 2 : 0);
   std::vector<double> glx, glw;
   gauss_legendre(SELF_NGL, glx, glw);
   // the quadrature rule is scratch: freed on the way out, also when a step throws
@@ -209,6 +222,7 @@ void compute_self(hb_ctx* c) {
   }
   dev_free(d_gl);
   dev_free(d_gw);
+  c->hank_top = top > HT_LO ? (float)top : 0.0f;
 }
 
 EntryParams entry_params(const hb_ctx* c, int transposed) {

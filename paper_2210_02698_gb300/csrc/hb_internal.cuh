@@ -279,8 +279,10 @@ struct hb_ctx {
   double* d_H[2] = {nullptr, nullptr};
   double* d_ncell = nullptr;
   double2* d_self = nullptr;
-  double2* d_hank = nullptr;   // Hankel expansions (hankel_table.cuh) of x < hank_top
+  double2* d_hank = nullptr;   // Hankel expansions (hankel_table.cuh): hank_rows of them, x < hank_top in use
+  int hank_rows = 0;
   float hank_top = 0.0f;
+  std::vector<double2*> hank_old;   // arrays outgrown by hb_set_omega (captured graphs read them)
 
   // cluster tree
   int Lv = 0;
