@@ -310,7 +310,7 @@ hb_status hb_entries(hb_handle h, const long long* rows, int m, const long long*
  * hb_curve_set: evaluates the three operators densely on the device and
  * factors K^{s2s} (LU with partial pivoting) and keeps its inverse (N_s^2
  * more complex values); replaces an earlier curve.
- * Synchronous.  Device memory: (2 ns N_v + 2 ns^2) x 16 bytes, 48 n_I^2 + 256
+ * Synchronous.  Device memory: (2 ns N_v + 2 ns^2) x 16 bytes, 48 n_I^2 + 304
  * bytes a segment, the operands of the products (256 bytes a row of the
  * operators), and 2 ns x
  * nrhs x 16 bytes at the first hb_apply_inclusion, owned by the handle until the

@@ -57,8 +57,9 @@ __global__ void scatter_kernel(const double2* __restrict__ y, const long long* _
 // are kept in input order).  It scales X per right-hand side, splits it into
 // digit fragments in shared memory once, TASK_KC k-steps at a time, and every
 // warp streams its unit's F from global memory into registers, one k-step
-// ahead, scaling it per task (tk.fe, found when the plan is made) and
-// splitting it there.  Long sums (ks k-steps) are dealt over kw(ks) warps and
+// ahead, scaling it per output row (P.d_fe, found when the plan is made) and
+// splitting it there: a row far below the others of its task keeps its bits,
+// as in a plain FP64 sum.  Long sums (ks k-steps) are dealt over kw(ks) warps and
 // the integer sums added.  A unit's sums depend on its task alone, so a
 // shard's equal the whole apply's.
 //
@@ -67,8 +68,8 @@ __global__ void scatter_kernel(const double2* __restrict__ y, const long long* _
 // is near 16, and the epilogue, against 1024 x 4 FP64 FMAs for 16
 // right-hand sides (2048 cycles of an SM's FP64 unit).  Measured: 192^2 x 16
 // 3.67 ms with one FP64 FMA loop per output, 1.92 with a CTA of 8 warps per
-// task, 1.30 with four warps and shared inputs; 120 x 88 adjoint x 5: 601,
-// 251, 205 us.
+// task, 1.29 with four warps and shared inputs; 120 x 88 adjoint x 5: 601,
+// 251, 209 us (205 with one exponent a task, the same in every lane).
 constexpr int TASK_KC = 16;              // k-steps of X held at a time
 constexpr uint32_t SPLIT_IM_SIGN = 0x80000000u;
 constexpr int task_kw(int ks, int W) {   // warps sharing a unit's k-steps
@@ -120,8 +121,9 @@ __device__ __noinline__ void task_plain(const Task* __restrict__ task, const dou
 
 template <bool HALF, int W>
 __global__ void __launch_bounds__(32 * W, 16 / W)
-    task_kernel(const TaskItem* __restrict__ items, const TaskUnit* __restrict__ units, const Task* __restrict__ tasks,
-                const double2* __restrict__ F, double2* x, double2* y, double2* xh, int R) {
+    task_kernel(const TaskItem* __restrict__ items, const TaskUnit* __restrict__ units,
+                const unsigned short* __restrict__ fexp, const Task* __restrict__ tasks, const double2* __restrict__ F,
+                double2* x, double2* y, double2* xh, int R) {
   constexpr int NR = HALF ? 8 : 16;        // right-hand sides of the MMA rows
   constexpr int NE = HALF ? 4 : 8;         // accumulator elements per lane and digit diagonal
   constexpr int XW = HALF ? 2 : 4;         // X fragment words per lane
@@ -140,9 +142,9 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
   const int wt = warp % uw, kp = warp / uw;
 
   // the warp's unit, and F values (row, k = 2t) and (row, 2t + 1) of its k-step q
-  bool work = false, rok = false;
+  bool work = false, rok = false, fok = false;   // fok: the digits hold every row of the unit
   TaskUnit unit;
-  int fe = 0, row = 0;
+  int fe = 0, row = 0;   // of row 8 tile + g
   double2 f0, f1;
   auto load_f = [&](int q) {
     f0 = f1 = make_double2(0.0, 0.0);
@@ -158,10 +160,13 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
   };
   auto take_unit = [&](int u0) {
     work = u0 + wt < item.units;
-    unit = units[item.unit0 + (work ? u0 + wt : 0)];
+    const int at = item.unit0 + (work ? u0 + wt : 0);
+    unit = units[at];
+    fe = fexp[8 * (size_t)at + g];
     row = 8 * unit.tile + g;
     rok = work && row < unit.r_out;
-    fe = tasks[unit.task].fe;
+    fok = __all_sync(0xffffffffu, split_exponent_ok(fe));
+    fe = max(fe, SPLIT_MIN_EXP);
     load_f(kp);
   };
   take_unit(0);
@@ -216,16 +221,15 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
         for (int k = 8 * c0 + xk; k < 8 * c1; k += XK) split_x(k, c0, load_x(k));
         __syncthreads();
       }
-      if (work && !s_bad && split_exponent_ok(fe)) {
+      if (work && !s_bad && fok) {
         int since = 0;
         for (int q = c0 + kp; q < c1; q += kw) {   // TASK_KC is a multiple of kw
           const double2 a0 = f0, a1 = f1;
           load_f(q + kw);
           uint32_t b0[SPLIT_DIGITS], b1[SPLIT_DIGITS];
           const uint32_t cs = unit.conj_t ? 0x80000000u : 0u;
-          const int fx = max(fe, SPLIT_MIN_EXP);
-          split_pair(a0, fx, cs, b0);
-          split_pair(a1, fx, cs, b1);
+          split_pair(a0, fe, cs, b0);
+          split_pair(a1, fe, cs, b1);
           const uint32_t* xq = xs + ((q - c0) * SPLIT_DIGITS * 32 + lane) * XW;
 #pragma unroll
           for (int i = 0; i < SPLIT_DIGITS; ++i) {
@@ -276,11 +280,12 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
           }
     }
     if (!work || kp > 0) continue;
-    if (s_bad || !split_exponent_ok(fe)) {
+    if (s_bad || !fok) {
       task_plain(tasks + unit.task, F, x, y, xh, R, 8 * unit.tile, min(unit.r_out, 8 * unit.tile + 8));
       continue;
     }
     double2* out = (unit.y_buf == 0 ? x : unit.y_buf == 1 ? y : xh) + (size_t)unit.y_off * R;
+    const int fo[2] = {__shfl_sync(0xffffffffu, fe, 8 * t), __shfl_sync(0xffffffffu, fe, 8 * t + 4)};   // of rows 2t, 2t + 1
     // element e of D: right-hand side g + 8 (e >> 1), output 2t + (e & 1); HALF:
     // elements 0, 1 are D_r and 2, 3 D_i of right-hand side g
 #pragma unroll
@@ -288,7 +293,7 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
       const int rr = HALF ? g : g + 8 * (e >> 1);
       const int ro = 8 * unit.tile + 2 * t + (e & 1);
       if (rr >= R || ro >= unit.r_out) continue;
-      const int sx = max(fe, SPLIT_MIN_EXP) + max(s_ex[rr], SPLIT_MIN_EXP) - 2 * SPLIT_EXP_BIAS;
+      const int sx = fo[e & 1] + max(s_ex[rr], SPLIT_MIN_EXP) - 2 * SPLIT_EXP_BIAS;
       const int ei = HALF ? e + 2 : e + 4;
       double2 v = make_double2(fixed_to_double(hi[e], lo[e], sx), fixed_to_double(hi[ei], lo[ei], sx));
       double2* o = out + (size_t)ro * R + rr;
@@ -302,25 +307,33 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
   }
 }
 
-// tasks[i].fe = the largest exponent of task i's factor blocks (0 before),
-// blockIdx.y of gridDim.y shares of them
-__global__ void __launch_bounds__(256) task_exponent_kernel(Task* __restrict__ tasks, const double2* __restrict__ F) {
-  Task& tk = tasks[blockIdx.x];
+// fe[8 u + g] = the largest exponent of row g of unit u (0 past the task's rows), one warp a unit
+__global__ void __launch_bounds__(256) unit_exponent_kernel(const TaskUnit* __restrict__ units, const Task* __restrict__ tasks,
+                                                            const double2* __restrict__ F, int n,
+                                                            unsigned short* __restrict__ fe) {
+  const int u = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  if (u >= n) return;
+  const TaskUnit unit = units[u];
+  const Task& tk = tasks[unit.task];
+  const int row = 8 * unit.tile + g;
   int e = 0;
-  for (int t = 0; t < tk.nterm; ++t) {
-    const long long cnt = (long long)tk.r_out * tk.r_in[t];
-    const double2* f = F + tk.f_off[t];
+  if (row < unit.r_out)
+    for (int q = 0; q < tk.nterm; ++q) {
+      const int rin = tk.r_in[q];
+      const double2* f = F + unit.f_off[q] + (unit.conj_t ? (size_t)row * rin : (size_t)row);
+      const size_t step = unit.conj_t ? 1 : (size_t)unit.r_out;
 #pragma unroll 4
-    for (long long k = blockIdx.y * 256 + threadIdx.x; k < cnt; k += 256 * gridDim.y) e = max(e, block_exponent(f[k]));
-  }
-  e = __reduce_max_sync(0xffffffffu, e);
-  if ((threadIdx.x & 31) == 0) atomicMax(&tk.fe, e);
+      for (int k = t; k < rin; k += 4) e = max(e, block_exponent(f[k * step]));
+    }
+  e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
+  e = max(e, __shfl_xor_sync(0xffffffffu, e, 2));
+  if (t == 0) fe[8 * (size_t)u + g] = (unsigned short)e;
 }
 
-void task_exponents(Task* d_tasks, int n, const double2* F, cudaStream_t st) {
-  if (n <= 0) return;
-  const unsigned share = (unsigned)std::max(1, std::min(128, 608 / n));
-  task_exponent_kernel<<<dim3((unsigned)n, share), 256, 0, st>>>(d_tasks, F);
+void task_exponents(TaskPlan& P, const Task* d_tasks, const double2* F, cudaStream_t st) {
+  if (P.units == 0) return;
+  P.d_fe = dev_alloc<unsigned short>(8 * (size_t)P.units);
+  unit_exponent_kernel<<<(unsigned)((P.units + 7) / 8), 256, 0, st>>>(P.d_units, d_tasks, F, P.units, P.d_fe);
   HB_CHECK_LAUNCH();
 }
 
@@ -385,6 +398,7 @@ TaskPlan task_plan(const std::vector<Task>& tasks, const std::vector<int>& begin
     P.max_ks.push_back(max_ks);
   }
   P.item_begin.push_back((int)items.size());
+  P.units = (int)units.size();
   P.d_units = upload(units);
   try {
     P.d_items = upload(items);
@@ -399,6 +413,7 @@ TaskPlan task_plan(const std::vector<Task>& tasks, const std::vector<int>& begin
 void task_plan_free(TaskPlan& P) {
   dev_free(P.d_units);
   dev_free(P.d_items);
+  dev_free(P.d_fe);
   P = TaskPlan{};
 }
 
@@ -411,7 +426,8 @@ static void launch_tasks(const TaskPlan& P, int step, const Task* tasks, const d
   const size_t red = (size_t)(W - 1) * 32 * (HALF ? 4 : 8) * sizeof(longlong2);
   const size_t smem = P.max_ks[(size_t)step] > 12 ? std::max(frag, red) : frag;
   HB_CUDA(cudaFuncSetAttribute(task_kernel<HALF, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, 56 << 10));
-  task_kernel<HALF, W><<<n, 32 * W, smem, st>>>(P.d_items + P.item_begin[(size_t)step], P.d_units, tasks, F, x, y, xh, R);
+  task_kernel<HALF, W><<<n, 32 * W, smem, st>>>(P.d_items + P.item_begin[(size_t)step], P.d_units, P.d_fe, tasks, F, x, y, xh,
+                                                R);
   HB_CHECK_LAUNCH();
 }
 
@@ -576,12 +592,12 @@ DenseOp dense_op(const double2* A, long long m, long long k, cudaStream_t st) {
   D.plan = task_plan(tasks, {0, D.ntask}, 8);
   try {
     D.d_tasks = upload(tasks, st);
+    task_exponents(D.plan, D.d_tasks, A, st);
+    HB_CUDA(cudaStreamSynchronize(st));
   } catch (...) {
-    task_plan_free(D.plan);
+    dense_op_free(D);
     throw;
   }
-  task_exponents(D.d_tasks, D.ntask, A, st);
-  HB_CUDA(cudaStreamSynchronize(st));
   return D;
 }
 
@@ -717,8 +733,11 @@ static ShardSteps& shard_steps(hb_ctx* c, int dir, long long lo, long long hi) {
   try {
     S->plan = task_plan(keep, S->begin, 4);
     S->d_tasks = upload(keep);
+    task_exponents(S->plan, S->d_tasks, c->d_f64, 0);
+    HB_CUDA(cudaStreamSynchronize(0));   // the caller's stream may not wait for this one
   } catch (...) {
     task_plan_free(S->plan);
+    dev_free(S->d_tasks);
     delete S;
     throw;
   }

@@ -560,12 +560,8 @@ static void make_plans(hb_ctx* c, std::vector<Butterfly>& bfs, const std::vector
     c->step_begin[dir] = begins;
     task_plan_free(c->task_plans[dir]);
     c->task_plans[dir] = task_plan(c->tasks_h[dir], begins, 4);
-    // the factor exponents are found on the device and kept on both sides (a
-    // shard uploads a part of the host list)
     c->d_tasks[dir] = upload(c->tasks_h[dir]);
-    task_exponents(c->d_tasks[dir], (int)c->tasks_h[dir].size(), c->d_f64, 0);
-    HB_CUDA(cudaMemcpy(c->tasks_h[dir].data(), c->d_tasks[dir], sizeof(Task) * c->tasks_h[dir].size(),
-                       cudaMemcpyDeviceToHost));
+    task_exponents(c->task_plans[dir], c->d_tasks[dir], c->d_f64, 0);
   }
 
   // native arenas and plans of the mixed apply

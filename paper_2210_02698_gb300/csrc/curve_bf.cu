@@ -20,6 +20,9 @@
 // y(tau) = K^L_tau xh(L, tau).  K^{v2s}_ij = g(r^s_i, r_j) (rows: segments,
 // columns: cells), K^{s2v}_ij = g(r_i, r^s_j) w_j (rows: cells, columns:
 // segments), g = v0 f0 + v1 f1 interpolated at the points (inclusion.cu).
+// The IDs see the lengths; the stored factors of K^{s2v} have their powers of
+// two p (w = m p) taken out, as inclusion.cu does: V and W become
+// diag(p_skeleton) V diag(1 / p), K^L takes m, and the butterfly applies to p P.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -37,7 +40,8 @@ struct BfSide {
   std::vector<long long> perm;                  // tree position -> natural index
   std::vector<std::vector<long long>> bounds;   // [level] node boundaries (2^l + 1)
   std::vector<double> xz;                       // (x, z) of tree position p at 2p, 2p + 1
-  std::vector<double> w;                        // weight of tree position p (empty: 1)
+  std::vector<double> w;                        // weight of tree position p (empty: 1) and
+  std::vector<int> e;                           // its binary exponent
   long long size() const { return (long long)perm.size(); }
 };
 
@@ -130,10 +134,25 @@ unsigned grid_for(long long total) {
   return (unsigned)std::max<long long>(1, std::min<long long>((total + 255) / 256, 152LL * 8));
 }
 
+// V(k, j) *= 2^(er[k] - ec[j]) for the r x n block at off (column-major, one CTA a block)
+struct ScaleBlock {
+  long long off, ec, er;   // ec, er: where the block's exponents start
+  int r, n;
+};
+__global__ void scale_block_kernel(double2* __restrict__ V, const ScaleBlock* __restrict__ blocks, const int* __restrict__ ex) {
+  const ScaleBlock b = blocks[blockIdx.x];
+  for (long long i = threadIdx.x; i < (long long)b.r * b.n; i += blockDim.x) {
+    const int d = ex[b.er + i % b.r] - ex[b.ec + i / b.r];
+    double2 v = V[b.off + i];
+    if (d) V[b.off + i] = make_double2(scalbn(v.x, d), scalbn(v.y, d));
+  }
+}
+
 // The sampled blocks K(rows[b], cols[b]) (rows on side R, columns on side C,
-// column weights C.w) into d_out, block b column-major at off[b].
+// column weights C.w, or their significands) into d_out, block b column-major at off[b].
 void eval_blocks(const hb_ctx* c, const BfSide& R, const BfSide& C, const std::vector<std::vector<long long>>& rows,
-                 const std::vector<std::vector<long long>>& cols, const std::vector<long long>& off, double2* d_out) {
+                 const std::vector<std::vector<long long>>& cols, const std::vector<long long>& off, bool significands,
+                 double2* d_out) {
   std::vector<double2> obs;
   std::vector<GreenCol> jobs;
   for (size_t b = 0; b < rows.size(); ++b) {
@@ -145,7 +164,7 @@ void eval_blocks(const hb_ctx* c, const BfSide& R, const BfSide& C, const std::v
       J.obs0 = obs0;
       J.out_off = off[b] + (long long)t * m;
       J.src = make_double2(C.xz[2 * q], C.xz[2 * q + 1]);
-      J.w = C.w.empty() ? 1.0 : C.w[(size_t)q];
+      J.w = C.w.empty() ? 1.0 : significands ? std::scalbn(C.w[(size_t)q], -C.e[(size_t)q]) : C.w[(size_t)q];
       J.m = (int)m;
       jobs.push_back(J);
     }
@@ -268,7 +287,7 @@ CurveBfly* build_bfly(const hb_ctx* c, const BfSide& R, const BfSide& C, int L) 
       }
       DevBuf<double2> d_A, V;
       d_A.p = dev_alloc<double2>((size_t)aacc);
-      eval_blocks(c, R, C, rows, cols, aoff, d_A.p);
+      eval_blocks(c, R, C, rows, cols, aoff, false, d_A.p);
       std::vector<int> rank;
       std::vector<std::vector<int>> piv;
       std::vector<long long> voff;
@@ -308,6 +327,24 @@ CurveBfly* build_bfly(const hb_ctx* c, const BfSide& R, const BfSide& C, int L) 
         tasks.push_back(t);
         lsize += (long long)r * n[(size_t)b];
       }
+      if (!C.e.empty()) {
+        std::vector<ScaleBlock> sc;
+        std::vector<int> ex;
+        for (int b = 0; b < nb; ++b) {
+          ScaleBlock q{voff[(size_t)b], (long long)ex.size(), 0, rank[(size_t)b], n[(size_t)b]};
+          for (long long t : cols[(size_t)b]) ex.push_back(C.e[(size_t)t]);
+          q.er = (long long)ex.size();
+          for (long long t : skel[(size_t)k][(size_t)b]) ex.push_back(C.e[(size_t)t]);
+          sc.push_back(q);
+        }
+        DevBuf<ScaleBlock> d_sc;
+        DevBuf<int> d_ex;
+        to_dev(d_sc, sc);
+        to_dev(d_ex, ex);
+        scale_block_kernel<<<(unsigned)nb, 256>>>(V.p, d_sc.p, d_ex.p);
+        HB_CHECK_LAUNCH();
+        HB_CUDA(cudaDeviceSynchronize());
+      }
       sb.push_back((int)tasks.size());
       parts.push_back({V.take(), lsize});
       fbase += lsize;
@@ -336,7 +373,7 @@ CurveBfly* build_bfly(const hb_ctx* c, const BfSide& R, const BfSide& C, int L) 
     sb.push_back((int)tasks.size());
     DevBuf<double2> KL;
     KL.p = dev_alloc<double2>((size_t)std::max<long long>(kacc, 1));
-    eval_blocks(c, R, C, rows, cols, koff, KL.p);
+    eval_blocks(c, R, C, rows, cols, koff, true, KL.p);
     parts.push_back({KL.take(), kacc});
     fbase += kacc;
     // the factor arena, in task order
@@ -395,7 +432,7 @@ CurveBfly* build_bfly(const hb_ctx* c, const BfSide& R, const BfSide& C, int L) 
       std::stable_sort(tasks.begin() + sb[q], tasks.begin() + sb[q + 1], task_reads_before);
     B->plan = task_plan(tasks, sb, 8);
     B->d_tasks = upload(tasks);
-    task_exponents(B->d_tasks, (int)tasks.size(), B->d_F, 0);
+    task_exponents(B->plan, B->d_tasks, B->d_F, 0);
     B->d_rperm = upload(R.perm);
     B->d_cperm = upload(C.perm);
     HB_CUDA(cudaDeviceSynchronize());
@@ -445,6 +482,7 @@ void curve_compress(hb_ctx* c, int leaf_s) {
     segs.xz[(size_t)(2 * p)] = cx[(size_t)q];
     segs.xz[(size_t)(2 * p + 1)] = cz[(size_t)q];
     segs.w[(size_t)p] = len[(size_t)q];
+    segs.e.push_back(std::ilogb(len[(size_t)q]));
   }
   const int L = std::min((int)cells.bounds.size(), (int)segs.bounds.size()) - 1;
   curve_bf_free(c);

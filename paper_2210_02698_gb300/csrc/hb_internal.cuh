@@ -123,8 +123,7 @@ struct Task {
   int r_out;
   int r_in[2];
   unsigned char nterm, x_buf, y_buf, accumulate;
-  unsigned char conj_t, kind;
-  int fe;                   // largest biased exponent of its factor blocks (task_exponents)
+  unsigned char conj_t, kind, pad0, pad1;
 };
 // The step tasks of a plan cut into CTAs (apply.cu): units (task, n-tile of 8
 // outputs), items (first unit, units) of tasks with the same inputs.  The
@@ -143,6 +142,8 @@ struct TaskPlan {
   int W = 4;                       // warps per CTA
   TaskUnit* d_units = nullptr;
   TaskItem* d_items = nullptr;
+  unsigned short* d_fe = nullptr;  // largest biased exponent of each factor row, 8 per unit (task_exponents)
+  int units = 0;
   std::vector<int> item_begin;     // items of step s: [item_begin[s], item_begin[s + 1])
   std::vector<int> max_ks;         // k-steps of 8 inputs of a step's longest task
 };
@@ -344,13 +345,15 @@ struct hb_ctx {
   long long ns = 0;                // segments; 0: no curve set
   long long ns_set = 0;            // segments of the arrays below (set before ns, while they are assembled)
   double2* d_seg = nullptr;        // ns centres (x, z)
-  double* d_segw = nullptr;        // ns lengths
+  double* d_segw = nullptr;        // ns lengths w = m p, p a power of two, 1 <= m < 2
+  double* d_segm = nullptr;        // ns values m
+  double* d_segp = nullptr;        // ns values p
   double* d_segn = nullptr;        // ns values of n at the centres
   double2* d_lu = nullptr;         // K^{s2s} LU-factored in place (ns x ns, column-major)
   int* d_piv = nullptr;            // its row interchanges
-  double2* d_inv = nullptr;        // (K^{s2s})^{-1} from the LU factors, ns x ns column-major
+  double2* d_inv = nullptr;        // diag(p) (K^{s2s})^{-1} from the LU factors, ns x ns column-major
   double2* d_kv2s = nullptr;       // K^{v2s}, ns x N_v column-major
-  double2* d_ks2v = nullptr;       // K^{s2v}, N_v x ns column-major
+  double2* d_ks2v = nullptr;       // K^{s2v} diag(1 / p), N_v x ns column-major
   hb::DenseOp op_v2s, op_inv, op_s2v;   // the three as step tasks
   double* d_seglag = nullptr;      // Lagrange basis at the segment centres (inclusion.cu)
   double* d_segG = nullptr;        // table contractions at the segment centres (inclusion.cu)
@@ -456,10 +459,10 @@ void curve_bf_free(hb_ctx* c);
 void curve_bf_info(const hb_ctx* c, int which, int* levels, int* max_rank, long long* entries);
 void curve_bf_apply(hb_ctx* c, int which, const double2* x_nat, long long ldx, double scale, double2* y_nat,
                     long long ldy, int accumulate, int nrhs, cudaStream_t st);
-// FP64 step tasks (apply.cu): the factor exponents of n tasks, the order of a
-// step's tasks, their CTAs (begin: the steps' task ranges; W = 4 warps, or 8
-// for few tasks with long sums), and one step
-void task_exponents(Task* d_tasks, int n, const double2* F, cudaStream_t st);
+// FP64 step tasks (apply.cu): the order of a step's tasks, their CTAs (begin:
+// the steps' task ranges; W = 4 warps, or 8 for few tasks with long sums), the
+// exponents of the factor rows (once F is there), and one step
+void task_exponents(TaskPlan& P, const Task* d_tasks, const double2* F, cudaStream_t st);
 bool task_reads_before(const Task& a, const Task& b);
 TaskPlan task_plan(const std::vector<Task>& tasks, const std::vector<int>& begin, int W);
 void task_plan_free(TaskPlan& P);
