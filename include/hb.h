@@ -188,7 +188,11 @@ hb_status hb_set_omega(hb_handle h, double omega);
 
 /* hb_apply: u = K (h^2 s) with the compressed operator (Eq. butterfly_mat
  * summed over the HODBF, plus the dense leaf blocks), in the precision of
- * opts.precision (see hb_set_precision).  s, u: device, complex128,
+ * opts.precision (see hb_set_precision).  HB_FP64: each step's products are
+ * sums of integer digits on the tensor cores, rounded to FP64 once; a block
+ * counts every row of its factor and every right-hand side to 2^-57 of its
+ * largest value there.  A right-hand side that is not finite in a block, or
+ * all below 2^-958, takes plain FP64 sums there; the others are not affected.  s, u: device, complex128,
  * N_v x nrhs column-major, must not overlap.  1 <= nrhs <= 1024.
  * Errors: HB_ERR_STATE before hb_build, HB_ERR_ARG, HB_ERR_CUDA. */
 hb_status hb_apply(hb_handle h, const void* s, void* u, int nrhs, void* stream);
@@ -276,14 +280,21 @@ hb_status hb_set_wait_selftest(hb_handle h, int on);
 hb_status hb_device_alloc_cap(long long cap_bytes, long long* live_bytes);
 
 /* hb_apply_dense / hb_apply_dense_adjoint: the same sums (Eq. m_v2v) and
- * their adjoint, matrix free, every entry evaluated in FP64 on the fly
- * (Eq. chebinterpblock, Eq. babich, Appendix A).  Needs no hb_build.
+ * their adjoint, matrix free, every entry evaluated on the fly
+ * (Eq. chebinterpblock, Eq. babich, Appendix A).  The Hankel pair of an entry
+ * is FP64 arithmetic; the interpolation and the sums over sources are products
+ * of integer digits on the tensor cores, accumulated exactly and rounded to
+ * FP64: values count to 2^-57 of the largest one beside them (interpolation:
+ * of a row of operands; sums: of a 16 x 8 tile of entries and of the
+ * right-hand side).  A right-hand side with values that are not finite, or all
+ * below 2^-958, is summed in plain FP64 instead; the others of its call are not
+ * affected.  Needs no hb_build.
  * Same layout and limits as hb_apply.  On grids with fewer than eight
  * 64-cell output segments per SM the source lines are split over CTAs and
  * the first such call allocates the per-share partial sums (owned by the
  * handle, freed by hb_destroy): make that first call outside a CUDA graph
- * capture.  Results do not depend on the split being taken or not beyond
- * the order of the FP64 additions. */
+ * capture.  Results depend on the split only by the roundings of a few
+ * partial sums per output. */
 hb_status hb_apply_dense(hb_handle h, const void* s, void* u, int nrhs, void* stream);
 hb_status hb_apply_dense_adjoint(hb_handle h, const void* u, void* s, int nrhs, void* stream);
 
@@ -330,7 +341,8 @@ hb_status hb_curve_operators(hb_handle h, void* k_s2s, void* k_v2s, void* k_s2v,
  *   u = (K^{v2v} + K^{s2v} (K^{s2s})^{-1} K^{v2s}) (h^2 s),
  * s, u as for hb_apply.  K^{v2v} is applied matrix free in FP64 when
  * v2v_dense != 0 (no hb_build needed), else by the compressed operator in
- * the handle's precision (needs hb_build); the surface part runs in FP64.
+ * the handle's precision (needs hb_build); the surface part takes the FP64
+ * products of hb_apply, whatever the ratio of the segment lengths.
  * The first call with more right-hand sides than before allocates the
  * surface vectors: make it outside a CUDA graph capture.  Errors:
  * HB_ERR_STATE without a curve, or v2v_dense == 0 before hb_build. */

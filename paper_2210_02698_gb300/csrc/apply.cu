@@ -68,8 +68,8 @@ __global__ void scatter_kernel(const double2* __restrict__ y, const long long* _
 // is near 16, and the epilogue, against 1024 x 4 FP64 FMAs for 16
 // right-hand sides (2048 cycles of an SM's FP64 unit).  Measured: 192^2 x 16
 // 3.67 ms with one FP64 FMA loop per output, 1.92 with a CTA of 8 warps per
-// task, 1.29 with four warps and shared inputs; 120 x 88 adjoint x 5: 601,
-// 251, 209 us (205 with one exponent a task, the same in every lane).
+// task, 1.30 with four warps and shared inputs; 120 x 88 adjoint x 5: 601,
+// 251, 207 us (205 with one exponent a task, the same in every lane).
 constexpr int TASK_KC = 16;              // k-steps of X held at a time
 constexpr uint32_t SPLIT_IM_SIGN = 0x80000000u;
 constexpr int task_kw(int ks, int W) {   // warps sharing a unit's k-steps
@@ -77,16 +77,18 @@ constexpr int task_kw(int ks, int W) {   // warps sharing a unit's k-steps
   return k < W ? k : W;
 }
 
-// Rows [row0, row1) of a task with plain FP64 FMAs, one warp: what a task
-// does whose inputs are not all finite (lane -> (row, right-hand side), rows fastest).
+// Rows [row0, row1) of a task with plain FP64 FMAs, one warp, for the
+// right-hand sides in the mask: those whose inputs the digits do not hold, or
+// all when the factors are so (lane -> (row, right-hand side), rows fastest).
 __device__ __noinline__ void task_plain(const Task* __restrict__ task, const double2* __restrict__ F, double2* x, double2* y,
-                                        double2* xh, int R, int row0, int row1) {
+                                        double2* xh, int R, int row0, int row1, unsigned mask) {
   const Task& tk = *task;
   double2* bufs[3] = {x, y, xh};
   double2* out = bufs[tk.y_buf] + (size_t)tk.y_off * R;
   const int rows = row1 - row0, total = rows * R;
   for (int idx = threadIdx.x & 31; idx < total; idx += 32) {
     const int row = row0 + idx % rows, rr = idx / rows;
+    if (!(mask >> rr & 1)) continue;
     double ar = 0, ai = 0;
     for (int t = 0; t < tk.nterm; ++t) {
       const double2* f = F + tk.f_off[t];
@@ -130,7 +132,7 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
   constexpr int XK = 32 * W / NR;          // inputs the CTA's threads take at once
   extern __shared__ __align__(16) uint32_t xs[];   // [k-step][digit][lane][XW]
   __shared__ int s_ex[16];
-  __shared__ int s_bad;
+  __shared__ unsigned s_bad;   // right-hand sides that the digits do not hold
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
   const TaskItem item = items[blockIdx.x];
   const int rin0 = item.r_in[0], rin1 = item.r_in[1];
@@ -142,7 +144,7 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
   const int wt = warp % uw, kp = warp / uw;
 
   // the warp's unit, and F values (row, k = 2t) and (row, 2t + 1) of its k-step q
-  bool work = false, rok = false, fok = false;   // fok: the digits hold every row of the unit
+  bool work = false, rok = false;
   TaskUnit unit;
   int fe = 0, row = 0;   // of row 8 tile + g
   double2 f0, f1;
@@ -165,8 +167,6 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
     fe = fexp[8 * (size_t)at + g];
     row = 8 * unit.tile + g;
     rok = work && row < unit.r_out;
-    fok = __all_sync(0xffffffffu, split_exponent_ok(fe));
-    fe = max(fe, SPLIT_MIN_EXP);
     load_f(kp);
   };
   take_unit(0);
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
   if (ex) atomicMax(&s_ex[xr], ex);
   __syncthreads();
   const int myex = max(s_ex[xr], SPLIT_MIN_EXP);
-  if (xr < R && !split_exponent_ok(s_ex[xr])) s_bad = 1;   // read after the next barrier
+  if (tid < R && !split_exponent_ok(s_ex[tid])) atomicOr(&s_bad, 1u << tid);   // read after the next barrier
 
   // X of k-steps [c0, c1) into digit fragments: word j of lane (g, t) is
   // (right-hand side g + 8 (j & 1), input 2t + (j >> 1)); HALF: (g, 2t + j)
@@ -206,6 +206,8 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
 
   for (int u0 = 0; u0 < item.units; u0 += uw) {   // several passes only when X is held whole
     if (u0) take_unit(u0);
+    const bool fok = __all_sync(0xffffffffu, split_exponent_ok(fe));   // the digits hold every row of the unit
+    const int fx = max(fe, SPLIT_MIN_EXP);
     float acc[SPLIT_ACC][NE];
     long long hi[NE], lo[NE];
 #pragma unroll
@@ -221,15 +223,15 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
         for (int k = 8 * c0 + xk; k < 8 * c1; k += XK) split_x(k, c0, load_x(k));
         __syncthreads();
       }
-      if (work && !s_bad && fok) {
+      if (work && fok) {
         int since = 0;
         for (int q = c0 + kp; q < c1; q += kw) {   // TASK_KC is a multiple of kw
           const double2 a0 = f0, a1 = f1;
           load_f(q + kw);
           uint32_t b0[SPLIT_DIGITS], b1[SPLIT_DIGITS];
           const uint32_t cs = unit.conj_t ? 0x80000000u : 0u;
-          split_pair(a0, fe, cs, b0);
-          split_pair(a1, fe, cs, b1);
+          split_pair(a0, fx, cs, b0);
+          split_pair(a1, fx, cs, b1);
           const uint32_t* xq = xs + ((q - c0) * SPLIT_DIGITS * 32 + lane) * XW;
 #pragma unroll
           for (int i = 0; i < SPLIT_DIGITS; ++i) {
@@ -280,19 +282,16 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
           }
     }
     if (!work || kp > 0) continue;
-    if (s_bad || !fok) {
-      task_plain(tasks + unit.task, F, x, y, xh, R, 8 * unit.tile, min(unit.r_out, 8 * unit.tile + 8));
-      continue;
-    }
+    const unsigned plain = fok ? s_bad : 0xffffu;
     double2* out = (unit.y_buf == 0 ? x : unit.y_buf == 1 ? y : xh) + (size_t)unit.y_off * R;
-    const int fo[2] = {__shfl_sync(0xffffffffu, fe, 8 * t), __shfl_sync(0xffffffffu, fe, 8 * t + 4)};   // of rows 2t, 2t + 1
+    const int fo[2] = {__shfl_sync(0xffffffffu, fx, 8 * t), __shfl_sync(0xffffffffu, fx, 8 * t + 4)};   // of rows 2t, 2t + 1
     // element e of D: right-hand side g + 8 (e >> 1), output 2t + (e & 1); HALF:
     // elements 0, 1 are D_r and 2, 3 D_i of right-hand side g
 #pragma unroll
     for (int e = 0; e < NE / 2; ++e) {
       const int rr = HALF ? g : g + 8 * (e >> 1);
       const int ro = 8 * unit.tile + 2 * t + (e & 1);
-      if (rr >= R || ro >= unit.r_out) continue;
+      if (rr >= R || ro >= unit.r_out || (plain >> rr & 1)) continue;
       const int sx = fo[e & 1] + max(s_ex[rr], SPLIT_MIN_EXP) - 2 * SPLIT_EXP_BIAS;
       const int ei = HALF ? e + 2 : e + 4;
       double2 v = make_double2(fixed_to_double(hi[e], lo[e], sx), fixed_to_double(hi[ei], lo[ei], sx));
@@ -304,6 +303,7 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
       }
       *o = v;
     }
+    if (plain) task_plain(tasks + unit.task, F, x, y, xh, R, 8 * unit.tile, min(unit.r_out, 8 * unit.tile + 8), plain);
   }
 }
 

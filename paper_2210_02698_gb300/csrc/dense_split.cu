@@ -32,9 +32,10 @@
 // with tabulated pairs (entries.cu) / this: 64^2, one right-hand side 53.4 /
 // 3.4 / 1.97 ms; 144 x 100, 16 right-hand sides (adjoint) 435 / 62 / 22.9 ms.
 //
-// Values that are not finite, or too small for the digits (split_fixed.cuh),
-// raise *flag; the FP64 kernel of entries.cu, launched behind this one, then
-// computes the apply instead.
+// Right-hand sides that are not finite, or too small for the digits
+// (split_fixed.cuh), are marked in *flag (bit r), all of them where an operand
+// of the entries is so; the FP64 kernel of entries.cu, launched behind this one,
+// computes the marked ones instead, so no column depends on another's values.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -51,19 +52,14 @@ constexpr int DS_DIAGS = 7;      // diagonals of digit products in the contracti
 constexpr double DS_C0 = 0.88622692545275801365;   // sqrt(pi)/2
 constexpr uint32_t DS_IM = 0x80000000u;
 
-// ex[r] = largest exponent of right-hand side r; *flag raised where the digits do not hold it
-__global__ void __launch_bounds__(256) rhs_exponent_kernel(const double2* __restrict__ s, long long Nv, int* __restrict__ ex,
-                                                           int* __restrict__ flag) {
+// ex[r] = largest exponent of right-hand side r
+__global__ void __launch_bounds__(256) rhs_exponent_kernel(const double2* __restrict__ s, long long Nv, int* __restrict__ ex) {
   const double2* c = s + (size_t)blockIdx.y * Nv;
   int e = 0;
   for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < Nv; i += (long long)gridDim.x * 256)
     e = max(e, block_exponent(c[i]));
   e = __reduce_max_sync(0xffffffffu, e);
-  if ((threadIdx.x & 31) == 0) {
-    if (e) atomicMax(&ex[blockIdx.y], e);
-    // a share of tiny values alone does not condemn the column: the kernel checks the column's exponent
-    if (e >= 0x7ff) *flag = 1;
-  }
+  if ((threadIdx.x & 31) == 0 && e) atomicMax(&ex[blockIdx.y], e);
 }
 
 // the digit products of one 16 x 8 tile, k = 16: acc[i + j] += a_i b_j, i + j < DIAGS
@@ -146,16 +142,18 @@ __global__ void __launch_bounds__(384) dense_split_kernel(EntryParams p, const d
   const long long o0 = (long long)bo * p.nx + ao0;
   const double w2 = p.omega * p.omega, w2l = fma(p.omega, p.omega, -w2), c1 = 2.0 * DS_C0 / w2;
   bool bad = false;
-  __shared__ int s_flag;
-  if (tid == 0) s_flag = *reinterpret_cast<volatile int*>(flag);
-  __syncthreads();
-  if (s_flag) return;   // the FP64 kernel takes this apply
-  if (tid < 16) {
+  __shared__ unsigned s_left;   // right-hand sides left to the FP64 kernel
+  if (tid < 32) {
     const int e = tid < rc ? exs[tid] : 0;
-    s_exs[tid] = max(e, SPLIT_MIN_EXP);
-    if (!split_exponent_ok(e)) *flag = 1;
+    const unsigned left = __ballot_sync(0xffffffffu, !split_exponent_ok(e));
+    if (tid < 16) s_exs[tid] = max(e, SPLIT_MIN_EXP);
+    if (tid == 0) {
+      s_left = left;
+      if (left && blockIdx.x == 0 && blockIdx.y == 0) atomicOr(flag, (int)left);
+    }
   }
   __syncthreads();
+  if (s_left == (1u << rc) - 1) return;
 
   // rows of LX as an A fragment: cells base + g and base + 8 + g (below end), row exponents e0, e1
   auto basis_frag = [&](int base, int end, uint32_t (&a)[4][SPLIT_DIGITS], int& e0, int& e1) {
@@ -397,7 +395,7 @@ __global__ void __launch_bounds__(384) dense_split_kernel(EntryParams p, const d
     }
   }
   if (__syncthreads_or(bad)) {
-    if (tid == 0) *flag = 1;
+    if (tid == 0) atomicOr(flag, 0xffff);
     return;
   }
   // the parts' sums, added in order: part 0 keeps its own in registers
@@ -417,7 +415,7 @@ __global__ void __launch_bounds__(384) dense_split_kernel(EntryParams p, const d
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const int o = 16 * mt + g + 8 * (e >> 1), rr = 8 * r + 2 * t + (e & 1);
-      if (o >= olen || rr >= rc) continue;
+      if (o >= olen || rr >= rc || (s_left >> rr & 1)) continue;
       double2 a = make_double2(0.0, 0.0);
       for (int q = 0; q < nparts; ++q) {
         const double2 v = red[(((q * nmt + mt) * RT + r) * 4 + e) * 32 + lane];
@@ -451,13 +449,13 @@ void launch(const EntryParams& p, const double2* s, double2* u, long long Nv, in
 
 }  // namespace
 
-// rc <= 16 right-hand sides from r0 on; exs: 16 exponents and, behind them, the flag (all zeroed here)
+// rc <= 16 right-hand sides from r0 on; exs: 16 exponents and, behind them, the flags (all zeroed here)
 void dense_split(const EntryParams& p, const double2* s, double2* u, long long Nv, int L, int nsplit, int r0, int rc,
                  int adjoint, double scale, double2* part, int* exs, cudaStream_t st) {
   int* flag = exs + 16;
   HB_CUDA(cudaMemsetAsync(exs, 0, 17 * sizeof(int), st));
   rhs_exponent_kernel<<<dim3((unsigned)std::max<long long>(1, std::min<long long>((Nv + 1023) / 1024, 64)), (unsigned)rc), 256, 0,
-                        st>>>(s + (size_t)r0 * Nv, Nv, exs, flag);
+                        st>>>(s + (size_t)r0 * Nv, Nv, exs);
   HB_CHECK_LAUNCH();
   if (rc <= 8) {
     if (adjoint) launch<1, true>(p, s, u, Nv, L, nsplit, r0, rc, scale, part, exs, flag, st);

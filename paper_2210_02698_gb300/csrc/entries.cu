@@ -242,7 +242,8 @@ EntryParams entry_params(const hb_ctx* c, int transposed) {
 
 // ------------------------------------------------------- dense apply ----
 // The form in plain FP64 FMAs, for values that the digits of dense_split.cu do
-// not hold (not finite, or below 2^-960): it runs when that kernel's flag is up.
+// not hold (not finite, or below 2^-960): it runs where that kernel marked a
+// right-hand side of the pass (bit bit0 + r of *flag) and writes the marked ones.
 //
 // One CTA owns the L <= 64 cells of one segment of a grid line (the outputs; a
 // line is cut into equal segments) and sweeps the source line segments of L
@@ -265,9 +266,10 @@ template <int RC, bool ADJ, int KI>
 __global__ void __launch_bounds__(256, RC <= 4 ? 2 : 1) dense_kernel(EntryParams p, const double2* __restrict__ s,
                                                     double2* __restrict__ u, long long Nv, int L, int r0,
                                                     double scale, double2* __restrict__ part,
-                                                    const int* __restrict__ flag) {
+                                                    const int* __restrict__ flag, int bit0) {
   extern __shared__ double smem[];
-  if (!*flag) return;   // the digit form (dense_split.cu) holds
+  const int marked = *flag >> bit0 & ((1 << RC) - 1);
+  if (!marked) return;   // the digit form (dense_split.cu) holds
   const int nI = p.nI;
   double* M = smem;                           // 3 x KI x KI
   double* P = M + 3 * KI * KI;                // 3 x DT x KI
@@ -373,6 +375,7 @@ __global__ void __launch_bounds__(256, RC <= 4 ? 2 : 1) dense_kernel(EntryParams
   if (active && grp == 0) {
 #pragma unroll
     for (int r = 0; r < RC; ++r) {
+      if (!(marked >> r & 1)) continue;
       double2 a = acc[r];
       for (int qq = 0; qq < ngr - 1; ++qq) {
         double2 b = red[(qq * L + o) * RC + r];
@@ -386,36 +389,39 @@ __global__ void __launch_bounds__(256, RC <= 4 ? 2 : 1) dense_kernel(EntryParams
 }
 
 // u[r0 + r][cell] = scale * (sum over the shares, in order, of part[share][r][cell])
-// (when the flag equals want: both forms of the apply write the shares)
+// for the columns whose bit (bit0 + r of *flag) equals want: each form of the
+// apply has written the shares of its own
 __global__ void dense_reduce_kernel(const double2* __restrict__ part, double2* __restrict__ u, long long Nv, int rc,
-                                    int nsplit, int r0, double scale, const int* __restrict__ flag, int want) {
-  if ((*flag != 0) != (want != 0)) return;
+                                    int nsplit, int r0, double scale, const int* __restrict__ flag, int bit0, int want) {
+  const int cols = (want ? *flag : ~*flag) >> bit0 & ((1 << rc) - 1);
+  if (!cols) return;
   const long long n = Nv * rc;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const long long r = i / Nv, cell = i - r * Nv;
+    if (!(cols >> r & 1)) continue;
     double2 a = make_double2(0.0, 0.0);
     for (int k = 0; k < nsplit; ++k) {
       const double2 b = part[(size_t)k * n + i];
       a.x += b.x;
       a.y += b.y;
     }
-    const long long r = i / Nv, cell = i - r * Nv;
     u[(size_t)(r0 + r) * Nv + cell] = make_double2(a.x * scale, a.y * scale);
   }
 }
 
 template <int RC, bool ADJ, int KI>
 static void launch_dense(const EntryParams& p, const double2* s, double2* u, long long Nv, int L, int r0,
-                         double scale, int nsplit, double2* part, const int* flag, cudaStream_t st) {
+                         double scale, int nsplit, double2* part, const int* flag, int bit0, cudaStream_t st) {
   size_t sm = sizeof(double) * (3 * KI * KI + 3 * DT * KI) + sizeof(double2) * (DT + 256) * RC;
   auto k = dense_kernel<RC, ADJ, KI>;
   HB_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   const int ntx = (p.nx + L - 1) / L;
-  k<<<dim3(ntx * p.ny, nsplit), 256, sm, st>>>(p, s, u, Nv, L, r0, scale, nsplit > 1 ? part : nullptr, flag);
+  k<<<dim3(ntx * p.ny, nsplit), 256, sm, st>>>(p, s, u, Nv, L, r0, scale, nsplit > 1 ? part : nullptr, flag, bit0);
   HB_CHECK_LAUNCH();
   if (nsplit > 1) {
     const long long n = Nv * RC;
     dense_reduce_kernel<<<(unsigned)std::min<long long>((n + 255) / 256, 152LL * 8), 256, 0, st>>>(
-        part, u, Nv, RC, nsplit, r0, scale, flag, 1);
+        part, u, Nv, RC, nsplit, r0, scale, flag, bit0, 1);
     HB_CHECK_LAUNCH();
   }
 }
@@ -423,7 +429,8 @@ static void launch_dense(const EntryParams& p, const double2* s, double2* u, lon
 // the FP64 form for rc right-hand sides from r0 on, in passes of 16, 8, 4, 2 and 1
 static void dense_plain(const EntryParams& p, const double2* s, double2* u, long long Nv, int L, int r0, int rc, int adjoint,
                         double scale, int nsplit, double2* part, const int* flag, cudaStream_t st) {
-#define HB_DENSE_LAUNCH(R, A, K) launch_dense<R, A, K>(p, s, u, Nv, L, r0, scale, nsplit, part, flag, st)
+  const int first = r0;
+#define HB_DENSE_LAUNCH(R, A, K) launch_dense<R, A, K>(p, s, u, Nv, L, r0, scale, nsplit, part, flag, r0 - first, st)
 #define HB_DENSE_CASE(R)                        \
   for (; rc >= R; rc -= R, r0 += R) {           \
     if (p.nI <= 8) {                            \
@@ -478,7 +485,7 @@ void dense_apply(hb_ctx* c, const double2* s, double2* u, int nrhs, int adjoint,
     }
   }
   // passes of up to 16 right-hand sides on the tensor cores; behind each the
-  // FP64 kernel, which runs where the digits did not hold the values
+  // FP64 kernel, which takes the columns that the digits do not hold
   double2* part = nsplit > 1 ? c->d_dense_part : nullptr;
   const int* flag = c->d_dense_ex + 16;
   for (int r0 = 0; r0 < nrhs; r0 += 16) {
@@ -487,7 +494,7 @@ void dense_apply(hb_ctx* c, const double2* s, double2* u, int nrhs, int adjoint,
     if (nsplit > 1) {
       const long long n = c->Nv * rc;
       dense_reduce_kernel<<<(unsigned)std::min<long long>((n + 255) / 256, 152LL * 8), 256, 0, st>>>(
-          part, u, c->Nv, rc, nsplit, r0, scale, flag, 0);
+          part, u, c->Nv, rc, nsplit, r0, scale, flag, 0, 0);
       HB_CHECK_LAUNCH();
     }
     dense_plain(p, s, u, c->Nv, L, r0, rc, adjoint, scale, nsplit, part, flag, st);
