@@ -253,7 +253,10 @@ hb_status hb_apply_shard_adjoint(hb_handle h, const void* u, void* s, int nrhs, 
  * without a handle or a device. */
 hb_status hb_host_shard_rows(int nx, int ny, int leaf, int nranks, int rank, long long* lo, long long* hi);
 
-/* hb_set_precision: HB_FP64 or HB_MIXED_BF16X3 for later applies. */
+/* hb_set_precision: HB_FP64 or HB_MIXED_BF16X3 for later applies.  The FP64 step
+ * lists of a handle built for mixed applies are made by its first FP64 apply
+ * (HB_ERR_OOM from there when they do not fit; outside a CUDA graph capture,
+ * as for the apply scratch). */
 hb_status hb_set_precision(hb_handle h, int precision);
 
 /* hb_set_wait_selftest: failure-detection self-test of the mixed apply (no

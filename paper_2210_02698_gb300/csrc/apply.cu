@@ -417,6 +417,25 @@ void task_plan_free(TaskPlan& P) {
   P = TaskPlan{};
 }
 
+void ensure_task_plans(hb_ctx* c) {
+  for (int dir = 0; dir < 2; ++dir) {
+    if (c->d_tasks[dir]) continue;
+    TaskPlan P = task_plan(c->tasks_h[dir], c->step_begin[dir], 4);
+    Task* d = nullptr;
+    try {
+      d = upload(c->tasks_h[dir]);
+      task_exponents(P, d, c->d_f64, 0);
+      HB_CUDA(cudaStreamSynchronize(0));
+    } catch (...) {
+      task_plan_free(P);
+      dev_free(d);
+      throw;
+    }
+    c->task_plans[dir] = P;
+    c->d_tasks[dir] = d;
+  }
+}
+
 template <bool HALF, int W>
 static void launch_tasks(const TaskPlan& P, int step, const Task* tasks, const double2* F, double2* x, double2* y, double2* xh,
                          int R, cudaStream_t st) {
@@ -657,6 +676,7 @@ void apply_bf(hb_ctx* c, const double2* s, double2* u, int nrhs, int adjoint, in
   // right-hand sides per pass: the scratch vectors (skeleton rows x pass x 16
   // bytes for FP64) stay bounded for any nrhs
   const int chunk = std::min(nrhs, precision == HB_FP64 ? 16 : 32);
+  if (precision == HB_FP64) ensure_task_plans(c);
   ensure_scratch(c, chunk, precision == HB_FP64);
   TimerScope ts{c, st, {}};
   const double scale = c->h * c->h;

@@ -558,11 +558,8 @@ static void make_plans(hb_ctx* c, std::vector<Butterfly>& bfs, const std::vector
     }
     begins.push_back((int)c->tasks_h[dir].size());
     c->step_begin[dir] = begins;
-    task_plan_free(c->task_plans[dir]);
-    c->task_plans[dir] = task_plan(c->tasks_h[dir], begins, 4);
-    c->d_tasks[dir] = upload(c->tasks_h[dir]);
-    task_exponents(c->task_plans[dir], c->d_tasks[dir], c->d_f64, 0);
   }
+  if (c->opt.precision == HB_FP64) ensure_task_plans(c);   // else with the first FP64 apply
 
   // native arenas and plans of the mixed apply
   {

@@ -466,6 +466,7 @@ void task_exponents(TaskPlan& P, const Task* d_tasks, const double2* F, cudaStre
 bool task_reads_before(const Task& a, const Task& b);
 TaskPlan task_plan(const std::vector<Task>& tasks, const std::vector<int>& begin, int W);
 void task_plan_free(TaskPlan& P);
+void ensure_task_plans(hb_ctx* c);   // of the volume operator, both directions
 void run_tasks_fp64(const TaskPlan& P, int step, const Task* d_tasks, const double2* F, double2* x, double2* y,
                     double2* xh, int R, cudaStream_t st);
 // a stored dense operator as step tasks; Y = alpha A X (or +=) for R <= 16

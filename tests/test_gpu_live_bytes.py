@@ -1,0 +1,49 @@
+"""Device memory a handle holds: the FP64 step lists only where FP64 applies are
+made."""
+import gc
+
+import pytest
+
+from paper_2210_02698_gb300 import workloads as W
+from tests._common import gpu_op, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2210_02698_gb300 import build
+    build.build()
+
+
+def _live():
+    from paper_2210_02698_gb300 import binding
+    gc.collect()
+    return binding.device_alloc_cap(-1)
+
+
+def test_mixed_handles_hold_no_fp64_steps():
+    import torch
+    from paper_2210_02698_gb300 import binding
+    w = W.small_workload(W.LENS, 40, 5, 3)
+    s = to_dev(W.complex_normal_sources(w.grid.Nv, 3, 5))
+    live, held, out = _live(), {}, {}
+    for prec in (binding.HB_FP64, binding.HB_MIXED_BF16X3):
+        op = gpu_op(w, precision=prec)
+        op.build()
+        held[prec] = _live() - live
+        op.set_precision(binding.HB_FP64)   # the steps of a mixed handle are made by the first FP64 apply
+        u, a = torch.empty_like(s), torch.empty_like(s)
+        op.apply_adjoint(s, a, 3)
+        op.apply(s, u, 3)
+        torch.cuda.synchronize()
+        out[prec] = (u, a)
+        op.close()
+        assert _live() == live
+    assert held[binding.HB_MIXED_BF16X3] < held[binding.HB_FP64]
+    for x, y in zip(*out.values()):
+        assert torch.equal(x, y)
+
