@@ -325,9 +325,10 @@ hb_status hb_entries(hb_handle h, const long long* rows, int m, const long long*
  * factors K^{s2s} (LU with partial pivoting) and keeps its inverse (N_s^2
  * more complex values); replaces an earlier curve.
  * Synchronous.  Device memory: (2 ns N_v + 2 ns^2) x 16 bytes, 48 n_I^2 + 304
- * bytes a segment, the operands of the products (256 bytes a row of the
- * operators), and 2 ns x
- * nrhs x 16 bytes at the first hb_apply_inclusion, owned by the handle until the
+ * bytes a segment, the operands of the products (256 bytes x
+ * (inputs + outputs + at most 19456) of the largest operator, after
+ * hb_curve_compress of the inverse), and 2 ns x nrhs x 16 bytes at the first
+ * hb_apply_inclusion, owned by the handle until the
  * next hb_curve_set or hb_destroy.  Errors: HB_ERR_ARG for ns outside
  * [1, 16384], a non-finite centre, a length or n that is not positive, or a
  * singular K^{s2s} (the handle then has no curve); HB_ERR_OOM. */

@@ -490,15 +490,21 @@ void curve_compress(hb_ctx* c, int leaf_s) {
   // cells, columns segments weighted by their lengths
   CurveBfly* v2s = build_bfly(c, segs, cells, L);
   CurveBfly* s2v = nullptr;
+  double2* pack = nullptr;
   try {
     s2v = build_bfly(c, cells, segs, L);
+    pack = dev_alloc<double2>(dense_op_rows(c->op_inv) * 16);
   } catch (...) {
+    free_bfly(s2v);
     free_bfly(v2s);
     throw;
   }
   c->curve_bf[0] = v2s;
   c->curve_bf[1] = s2v;
-  // the dense forms are not needed any more
+  // the dense forms are not needed any more, and of the products' operands
+  // only the inverse's
+  dev_free(c->d_pack);
+  c->d_pack = pack;
   dense_op_free(c->op_v2s);
   dense_op_free(c->op_s2v);
   dev_free(c->d_kv2s);

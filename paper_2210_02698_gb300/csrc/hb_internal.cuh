@@ -473,6 +473,7 @@ void run_tasks_fp64(const TaskPlan& P, int step, const Task* d_tasks, const doub
 // columns, x / y: row-major operands (k x R and ntask m x R)
 DenseOp dense_op(const double2* A, long long m, long long k, cudaStream_t st);
 void dense_op_free(DenseOp& D);
+inline size_t dense_op_rows(const DenseOp& D) { return (size_t)D.k + (size_t)D.ntask * (size_t)D.m; }   // of x and y together
 void dense_product(const DenseOp& D, const double2* X, long long ldx, double2* Y, long long ldy, int R, double alpha,
                    int accumulate, double2* x, double2* y, cudaStream_t st);
 void curve_free(hb_ctx* c);

@@ -673,7 +673,7 @@ void curve_set(hb_ctx* c, const double* centers, const double* lengths, const do
       c->op_s2v = dense_op(c->d_ks2v, c->Nv, ns, 0);
       size_t rows = 0;
       for (const DenseOp* D : {&c->op_v2s, &c->op_inv, &c->op_s2v})
-        rows = std::max<size_t>(rows, (size_t)D->k + (size_t)D->ntask * (size_t)D->m);
+        rows = std::max(rows, dense_op_rows(*D));
       c->d_pack = dev_alloc<double2>(rows * 16);
     } catch (...) {
       cudaDeviceSynchronize();
