@@ -330,9 +330,8 @@ __global__ void __launch_bounds__(256) unit_exponent_kernel(const TaskUnit* __re
   if (t == 0) fe[8 * (size_t)u + g] = (unsigned short)e;
 }
 
-void task_exponents(TaskPlan& P, const Task* d_tasks, const double2* F, cudaStream_t st) {
+void task_exponents(const TaskPlan& P, const Task* d_tasks, const double2* F, cudaStream_t st) {
   if (P.units == 0) return;
-  P.d_fe = dev_alloc<unsigned short>(8 * (size_t)P.units);
   unit_exponent_kernel<<<(unsigned)((P.units + 7) / 8), 256, 0, st>>>(P.d_units, d_tasks, F, P.units, P.d_fe);
   HB_CHECK_LAUNCH();
 }
@@ -399,21 +398,24 @@ TaskPlan task_plan(const std::vector<Task>& tasks, const std::vector<int>& begin
   }
   P.item_begin.push_back((int)items.size());
   P.units = (int)units.size();
-  P.d_units = upload(units);
+  // the units and, behind them, the exponents of their rows (an allocation
+  // costs a new curve some 10 us)
+  P.d_units = reinterpret_cast<TaskUnit*>(dev_alloc<unsigned char>(units.size() * (sizeof(TaskUnit) + 8 * sizeof(unsigned short))));
+  P.d_fe = reinterpret_cast<unsigned short*>(P.d_units + units.size());
   try {
+    HB_CUDA(cudaMemcpyAsync(P.d_units, units.data(), units.size() * sizeof(TaskUnit), cudaMemcpyHostToDevice, 0));
     P.d_items = upload(items);
+    HB_CUDA(cudaStreamSynchronize(0));   // the host arrays end here
   } catch (...) {
-    dev_free(P.d_units);
+    task_plan_free(P);
     throw;
   }
-  HB_CUDA(cudaStreamSynchronize(0));   // the host arrays end here
   return P;
 }
 
 void task_plan_free(TaskPlan& P) {
   dev_free(P.d_units);
   dev_free(P.d_items);
-  dev_free(P.d_fe);
   P = TaskPlan{};
 }
 

@@ -142,7 +142,7 @@ struct TaskPlan {
   int W = 4;                       // warps per CTA
   TaskUnit* d_units = nullptr;
   TaskItem* d_items = nullptr;
-  unsigned short* d_fe = nullptr;  // largest biased exponent of each factor row, 8 per unit (task_exponents)
+  unsigned short* d_fe = nullptr;  // behind d_units: largest biased exponent of each factor row, 8 per unit
   int units = 0;
   std::vector<int> item_begin;     // items of step s: [item_begin[s], item_begin[s + 1])
   std::vector<int> max_ks;         // k-steps of 8 inputs of a step's longest task
@@ -347,7 +347,7 @@ struct hb_ctx {
   double2* d_seg = nullptr;        // ns centres (x, z)
   double* d_segw = nullptr;        // ns lengths w = m p, p a power of two, 1 <= m < 2
   double* d_segm = nullptr;        // ns values m
-  double* d_segp = nullptr;        // ns values p
+  double* d_segp = nullptr;        // ns values p, behind d_segm
   double* d_segn = nullptr;        // ns values of n at the centres
   double2* d_lu = nullptr;         // K^{s2s} LU-factored in place (ns x ns, column-major)
   int* d_piv = nullptr;            // its row interchanges
@@ -462,7 +462,7 @@ void curve_bf_apply(hb_ctx* c, int which, const double2* x_nat, long long ldx, d
 // FP64 step tasks (apply.cu): the order of a step's tasks, their CTAs (begin:
 // the steps' task ranges; W = 4 warps, or 8 for few tasks with long sums), the
 // exponents of the factor rows (once F is there), and one step
-void task_exponents(TaskPlan& P, const Task* d_tasks, const double2* F, cudaStream_t st);
+void task_exponents(const TaskPlan& P, const Task* d_tasks, const double2* F, cudaStream_t st);
 bool task_reads_before(const Task& a, const Task& b);
 TaskPlan task_plan(const std::vector<Task>& tasks, const std::vector<int>& begin, int W);
 void task_plan_free(TaskPlan& P);

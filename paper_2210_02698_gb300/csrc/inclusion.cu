@@ -582,7 +582,7 @@ void green_jobs(const hb_ctx* c, const double2* d_obs, const GreenCol* d_jobs, l
 void curve_free(hb_ctx* c) {
   for (void* p : {(void*)c->d_seg, (void*)c->d_segw, (void*)c->d_segn, (void*)c->d_lu, (void*)c->d_piv,
                   (void*)c->d_kv2s, (void*)c->d_ks2v, (void*)c->d_cy, (void*)c->d_inv, (void*)c->d_seglag,
-                  (void*)c->d_segG, (void*)c->d_pack, (void*)c->d_segm, (void*)c->d_segp})
+                  (void*)c->d_segG, (void*)c->d_pack, (void*)c->d_segm})
     dev_free(p);
   dense_op_free(c->op_v2s);
   dense_op_free(c->op_inv);
@@ -616,13 +616,13 @@ void curve_set(hb_ctx* c, const double* centers, const double* lengths, const do
     c->d_seg = upload(cen);
     c->d_segw = upload(std::vector<double>(lengths, lengths + ns));
     c->d_segn = upload(std::vector<double>(n_seg, n_seg + ns));
-    std::vector<double> m((size_t)ns), p((size_t)ns);
+    std::vector<double> mp(2 * (size_t)ns);
     for (long long i = 0; i < ns; ++i) {
-      p[(size_t)i] = std::ldexp(1.0, std::ilogb(lengths[i]));
-      m[(size_t)i] = lengths[i] / p[(size_t)i];
+      mp[(size_t)(ns + i)] = std::ldexp(1.0, std::ilogb(lengths[i]));
+      mp[(size_t)i] = lengths[i] / mp[(size_t)(ns + i)];
     }
-    c->d_segm = upload(m);
-    c->d_segp = upload(p);
+    c->d_segm = upload(mp);
+    c->d_segp = c->d_segm + ns;
     c->ns_set = ns;
     c->d_seglag = dev_alloc<double>((size_t)ns * 32);
     c->d_segG = dev_alloc<double>((size_t)6 * c->NI * ns);
