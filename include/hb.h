@@ -397,7 +397,7 @@ hb_status hb_curve_info(hb_handle h, int which, int* levels, int* max_rank, long
  * src[k] (at a source's own node tau2 is 0, v0 = B_0 and v1 = C_0 by
  * Eq. expansionT..V1: set those entries, which the interpolation only
  * approximates); info: HOST ns x 6, the iterations and the last largest
- * update of the three solves.  One CTA per source; each anti-diagonal of a
+ * update of the three solves.  One CTA or a cluster per source; each anti-diagonal of a
  * sweep is updated in parallel, which gives the row-by-row Gauss-Seidel
  * iterates bit for bit.  Device memory: ns x (5 M^2 + 7 (w1 - w0 + 1)^2) x
  * 8 bytes.  Synchronous.  Errors: HB_ERR_ARG (null array, bad mesh - M < 8,

@@ -6,9 +6,11 @@
 //   u  = y scattered back to natural order
 //
 // FP64 path: complex128 factors and vectors, the step tasks' products on the
-// FP16 tensor cores by integer digits, as accurate as FP64 FMAs.  Mixed path (HB_MIXED_BF16X3): split-BF16 factors and
-// vectors in the MMA-fragment layout of bf_mma.cu, up to 32 right-hand
-// sides per pass.
+// FP16 tensor cores by integer digits, as accurate as FP64 FMAs as long as a
+// factor row and a right-hand side of a task do not hide one another's small
+// values (split_fixed.cuh; inclusion.cu keeps the segment lengths out of them
+// for that).  Mixed path (HB_MIXED_BF16X3): split-BF16 factors and vectors in
+// the MMA-fragment layout of bf_mma.cu, up to 32 right-hand sides per pass.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -200,8 +200,7 @@ __global__ void __launch_bounds__(384) dense_split_kernel(EntryParams p, const d
     }
   }
 
-  const int mt = warp % nmt, part_of = warp / nmt, nparts = nwarp / nmt;
-  const bool sums = part_of < nparts;   // warps past a whole number of groups only help to stage
+  const int mt = warp % nmt, part_of = warp / nmt, nparts = nwarp / nmt;   // nmt divides the warps (launch)
   // running sums: element e of tile (rt, re / im): output 16 mt + g + 8 (e >> 1), right-hand side 8 rt + 2t + (e & 1)
   long long hi[RT][2][4], lo[RT][2][4];
 #pragma unroll
@@ -312,7 +311,6 @@ __global__ void __launch_bounds__(384) dense_split_kernel(EntryParams p, const d
           *reinterpret_cast<uint2*>(sm + Y.sfrag + ((w * SPLIT_DIGITS + d) * 32 + lane) * 2) = make_uint2(b0[d], b1[d]);
       }
       __syncthreads();
-      if (!sums) continue;
       const uint32_t* af = sm + Y.lxo + (mt * SPLIT_DIGITS * 32 + lane) * 4;
       for (int tile = part_of; tile < ntile; tile += nparts) {
         // the entries (o, c): o = 16 mt + g + 8 (e >> 1), c = 8 tile + 2t + (e & 1)
@@ -406,10 +404,10 @@ __global__ void __launch_bounds__(384) dense_split_kernel(EntryParams p, const d
     for (int e = 0; e < 4; ++e) {
       const int ex = erun + s_exs[8 * r + 2 * t + (e & 1)] - 2 * SPLIT_EXP_BIAS;
       const double2 v = make_double2(fixed_to_double(hi[r][0][e], lo[r][0][e], ex), fixed_to_double(hi[r][1][e], lo[r][1][e], ex));
-      if (sums) red[(((part_of * nmt + mt) * RT + r) * 4 + e) * 32 + lane] = v;
+      red[(((part_of * nmt + mt) * RT + r) * 4 + e) * 32 + lane] = v;
     }
   __syncthreads();
-  if (!sums || part_of) return;
+  if (part_of) return;
 #pragma unroll
   for (int r = 0; r < RT; ++r)
 #pragma unroll
@@ -435,7 +433,8 @@ void launch(const EntryParams& p, const double2* s, double2* u, long long Nv, in
   // twelve warps (all the registers hold) where the segment has three or four
   // m-tiles: eight leave three m-tiles unevenly spread over the SM's
   // sub-partitions, and 64^2 2.05 -> 1.97 ms, 120 x 100 16.6 -> 14.7, 100 x 80 x 5
-  // 9.25 -> 8.45; below that level (24^2), or slower (32^2 x 16: 384 -> 392 us)
+  // 9.25 -> 8.45; below that level (24^2), or slower (32^2 x 16: 384 -> 392 us).
+  // 1, 2, 3 and 4 divide their count.
   const int warps = nmt >= 3 ? 12 : 8;
   const DsLayout Y(nmt, (LQ + 7) / 8, RT);
   const size_t red = (size_t)(warps / nmt) * nmt * RT * 4 * 32 * sizeof(double2);

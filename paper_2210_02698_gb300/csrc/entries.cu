@@ -256,7 +256,7 @@ EntryParams entry_params(const hb_ctx* c, int transposed) {
 //
 // Bound by the FP64 unit (2 FMAs a cycle and SM).  Per entry: 3 KI for the
 // observation contraction (the basis values in registers, the source's P
-// broadcast from shared memory), 27 for the Hankel pair (hankel_table.cuh)
+// broadcast from shared memory), 28 for the Hankel pair (hankel_table.cuh)
 // and 4 RC.  sqrt(pi)/2 and the factors of f1 are folded into P.  Measured:
 // 64^2, one right-hand side 3.3 ms, 144 x 100 with 16 (adjoint) 62 ms.
 constexpr int DT = 64;

@@ -74,7 +74,7 @@ __device__ __forceinline__ void basis_at(const double* nodes, const double* bw, 
 // ---- the dense curve operators ----
 // Every entry is g(seg, cell), g(cell, seg) or g(seg, seg'), so the tables are
 // contracted with a segment's basis once, and the cells' tensor structure
-// does the rest line by line: 48 FMAs and a tabulated Hankel pair (27) an
+// does the rest line by line: 48 FMAs and a tabulated Hankel pair (28) an
 // entry.  (Contracting per source cell and evaluating the full basis and the
 // recurrences per entry took 28.8 ms of FP64 at 96^2 with 300 segments.)
 
@@ -134,7 +134,8 @@ __device__ __forceinline__ double2 green_tab(const HankelTable& T, double omega,
 
 // Segment p (one thread) against the cells [a0, a1) of grid line line0 + blockIdx.y.
 // V2S: out[cell ns + p] = g(seg_p, cell) (G: the transposed contractions); else
-// out[p Nv + cell] = w_p g(cell, seg_p), two cells at a time (one 32-byte sector).
+// out[p Nv + cell] = w_p g(cell, seg_p) (16 bytes a lane at stride Nv: the L2 joins the halves of a
+// sector before they leave it).
 template <bool V2S>
 __global__ void __launch_bounds__(64) seg_line_kernel(EntryParams E, const double* __restrict__ G, long long ns,
                                                       const double* __restrict__ w, int line0, double2* __restrict__ out) {
@@ -217,8 +218,8 @@ __global__ void __launch_bounds__(128) seg_seg_kernel(EntryParams E, const doubl
 
 // Batched columns of curve-operator blocks: job q (one CTA) writes
 // out[J.out_off + a] = J.w g(obs[J.obs0 + a], J.src) for a < J.m - the
-// same evaluation as green_columns_kernel, for sampled blocks whose rows
-// are gathered into obs.
+// evaluation of one entry at a time, by the recurrences, for sampled blocks
+// whose rows are gathered into obs.
 __global__ void __launch_bounds__(256) green_jobs_kernel(PointTables P, const double2* __restrict__ obs,
                                                          const GreenCol* __restrict__ jobs,
                                                          double2* __restrict__ out) {

@@ -6,23 +6,29 @@
 // and Rump, Numer. Algorithms 59 (2012), with the digits of a common fixed
 // point, as in the integer form of Ootomo, Ozaki and Yokota, 2024).
 //
-// A block's values share one exponent: |v| = T 2^(E - 1080), E the largest
-// biased exponent of the block, T < 2^58 an integer (the 53-bit mantissa
-// shifted up by 5 and down by the exponent difference: a value within 2^5 of
-// the largest keeps every bit, and none is off by more than 2^-58 of the
+// The values of a row of an operand share one exponent: |v| = T 2^(E - 1080), E
+// the largest biased exponent of the row, T < 2^58 an integer (the 53-bit
+// mantissa shifted up by 5 and down by the exponent difference: a value within
+// 2^5 of the largest keeps every bit, and none is off by more than 2^-57 of the
 // largest; a product rounded in FP64 is off by 2^-53 of itself).  T is written in six
 // balanced base-1024 digits d_0 .. d_5, |d| <= 512, exact in FP16 (the sign
 // goes on every digit; blocks too small for their zeros to shift out, E < 65,
 // and those with values that are not finite are left to plain sums):
 // T = sum d_s 2^(10 (5 - s)).  The product of two values is
 //   sum_{i,j} d_i d'_j 2^(100 - 10 (i + j)),
-// of which the 21 digit products with i + j <= 5 are formed (the rest is
-// below 2^-57 of the largest product).  Those of one diagonal i + j share an
+// of which the 21 digit products with i + j <= 5 are formed.  The rest can
+// reach 2^-53.7 of the largest product (every digit at +-512: five products of
+// 2^18 on diagonal 6); for digits of random signs its root mean square is about
+// 2^-57.  Those of one diagonal i + j share an
 // FP32 accumulator; each digit product is at most 2^18.  Over two k-steps of
 // 16 (32 real products) the sums of diagonals 0, 1 and 2 (the latter held in
 // two accumulators, of two products and of one) stay within 2^24, so they
-// are exact integers whatever the data; for diagonals 3 to 5 a rounding of
-// the FP32 sum is below 2^-54 of the sum's terms.  After two k-steps the
+// are exact integers whatever the data.  Diagonal 3 can reach 1.5 x 2^24 where
+// all 32 products have digits near 512 of one sign pattern, i.e. for nearly
+// equal values all of one such pattern in both operands; it then rounds, by up
+// to 2^-46 of the sum of the terms' magnitudes (32 plain additions: 2^-48).
+// Digits of random signs stay 16 standard deviations below 2^24.  Diagonals 4
+// and 5 round at 2^-55 of that sum or less.  After two k-steps the
 // accumulators are added to 64-bit integers: `hi` in units of diagonal 2,
 // `lo` in units of diagonal 5; the result is hi 2^30 + lo, converted to FP64
 // with one rounding by integer instructions (four FP64 ones would cost more
