@@ -20,7 +20,7 @@
 // on average.
 //
 // A CTA owns the L <= 64 cells of one segment of a grid line and sweeps segments
-// of up to 144 source cells of its share of the source lines.  Warp w works for
+// of up to 200 source cells of its share of the source lines.  Warp w works for
 // the 16 outputs of m-tile w mod nmt and every (warps / nmt)-th n-tile of 8
 // sources.  The accumulator layout of one stage is the operand layout of the
 // next: P's (cells, i1) tile is the B fragment of the f stage (its pairs of i1),
@@ -46,7 +46,12 @@
 namespace hb {
 namespace {
 
-constexpr int DS_NT = 18;        // n-tiles (8 sources) of a source segment at most
+// n-tiles (8 sources) of a source segment at most: what 227 KB hold beside four
+// m-tiles and two tiles of right-hand sides (222.5 KB).  Longer segments share
+// their staging and barriers among more entries; 12 / 18 / 25 tiles: 200 x 60 x 4
+// 18.2 / 17.7 / 16.7 ms, 144 x 100 x 16 26.6 / 22.8 / 22.8, 120 x 100 17.2 / 14.7 /
+// 14.7, 64^2 1.98 each.
+constexpr int DS_NT = 25;
 constexpr int DS_K = 16;         // interpolation nodes per axis (padded with zeros)
 constexpr int DS_DIAGS = 7;      // diagonals of digit products in the contractions (sums: 6)
 constexpr double DS_C0 = 0.88622692545275801365;   // sqrt(pi)/2
