@@ -74,7 +74,13 @@ __global__ void scatter_kernel(const double2* __restrict__ y, const long long* _
 // 251, 207 us (205 with one exponent a task, the same in every lane).
 constexpr int TASK_KC = 16;              // k-steps of X held at a time
 constexpr uint32_t SPLIT_IM_SIGN = 0x80000000u;
-constexpr int task_kw(int ks, int W) {   // warps sharing a unit's k-steps
+// Warps sharing a unit's k-steps: one where a warp's own sums are short beside
+// the exchange, more where a step has few long ones.  Measured (us; 192^2 x 16 /
+// 120 x 88 adjoint x 5 / 64^2 x 5 / inclusion at 128^2 with 512 segments x 8):
+// always one 1270 / 217 / 109 / 366; two and four from 25 and 65 k-steps on
+// 1307 / 216 / 109 / 351, from 13 and 33 1315 / 218 / 107 / 294, from 7 and 17
+// 1337 / 223 / 104 / 275.
+constexpr int task_kw(int ks, int W) {
   const int k = ks <= 12 ? 1 : ks <= 32 ? 2 : 4;
   return k < W ? k : W;
 }
@@ -612,7 +618,7 @@ DenseOp dense_op(const double2* A, long long m, long long k, cudaStream_t st) {
     tasks.push_back(t);
   }
   D.ntask = (int)tasks.size();
-  D.plan = task_plan(tasks, {0, D.ntask}, 8);
+  D.plan = task_plan(tasks, {0, D.ntask}, 8);   // 4 warps: apply with 300 segments at 96^2 338 us, 8: 334
   try {
     D.d_tasks = upload(tasks, st);
     task_exponents(D.plan, D.d_tasks, A, st);
