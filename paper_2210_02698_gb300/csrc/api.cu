@@ -568,16 +568,14 @@ hb_status hb_id_batch(int count, const int* m, const int* n, const long long* a_
     if (count == 0) return;
     std::vector<long long> soff(count), voff(count);
     long long sacc = 0, vacc = 0;
-    int max_n = 0;
-    long long max_mn = 0;
+    hb::IdSizes sizes;
     for (int b = 0; b < count; ++b) {
       if (m[b] < 1 || n[b] < 1) throw hb::arg_error("matrix %d has an empty dimension", b);
       soff[b] = sacc;
       voff[b] = vacc;
       sacc += n[b];
       vacc += (long long)n[b] * n[b];
-      max_n = std::max(max_n, n[b]);
-      max_mn = std::max(max_mn, (long long)m[b] * n[b]);
+      sizes.add(m[b], n[b]);
     }
     int* d_m = hb::upload(std::vector<int>(m, m + count));
     int* d_n = hb::upload(std::vector<int>(n, n + count));
@@ -585,7 +583,7 @@ hb_status hb_id_batch(int count, const int* m, const int* n, const long long* a_
     long long* d_s = hb::upload(soff);
     long long* d_v = hb::upload(voff);
     int* d_perm = hb::dev_alloc<int>(sacc);
-    hb::id_batch(count, d_m, d_n, d_a, (double2*)A, eps, rank, d_perm, d_s, max_n, max_mn, 0);
+    hb::id_batch(count, d_m, d_n, d_a, (double2*)A, eps, rank, d_perm, d_s, sizes, 0);
     hb::emit_v(count, d_m, d_n, d_a, (const double2*)A, rank, d_perm, d_s, d_v, 0, (double2*)V, nullptr, 0);
     HB_CUDA(cudaMemcpy(skel, d_perm, sizeof(int) * sacc, cudaMemcpyDeviceToDevice));
     HB_CUDA(cudaDeviceSynchronize());

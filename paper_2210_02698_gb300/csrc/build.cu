@@ -204,8 +204,7 @@ void build(hb_ctx* c) {
         std::vector<int> hm(cnt), hn(cnt);
         std::vector<long long> haoff(cnt), hsoff(cnt);
         long long aoff = 0, soff = 0;
-        int max_n = 1;
-        long long max_mn = 0;
+        IdSizes sizes;
         std::vector<std::pair<int, size_t>> rec_here;   // (t, index in c->id_recs)
         for (int t = 0; t < cnt; ++t) {
           Job& jb = desc[q0 + t];
@@ -227,8 +226,7 @@ void build(hb_ctx* c) {
           hsoff[t] = soff;
           aoff += (long long)hm[t] * hn[t];
           soff += hn[t];
-          max_n = std::max(max_n, hn[t]);
-          max_mn = std::max(max_mn, (long long)hm[t] * hn[t]);
+          sizes.add(hm[t], hn[t]);
         }
         sampled += aoff;
         id_blocks += cnt;
@@ -245,7 +243,7 @@ void build(hb_ctx* c) {
         long long* d_soff = upload(hsoff);
         int* d_rank = dev_alloc<int>(cnt);
         int* d_perm = dev_alloc<int>((size_t)soff);
-        id_batch(cnt, d_m, d_n, d_aoff, d_A, c->opt.eps, d_rank, d_perm, d_soff, max_n, max_mn, st);
+        id_batch(cnt, d_m, d_n, d_aoff, d_A, c->opt.eps, d_rank, d_perm, d_soff, sizes, st);
         std::vector<int> hrank(cnt), hperm((size_t)soff);
         HB_CUDA(cudaMemcpyAsync(hrank.data(), d_rank, sizeof(int) * cnt, cudaMemcpyDeviceToHost, st));
         HB_CUDA(cudaMemcpyAsync(hperm.data(), d_perm, sizeof(int) * soff, cudaMemcpyDeviceToHost, st));

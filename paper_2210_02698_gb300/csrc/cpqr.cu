@@ -76,7 +76,7 @@ __device__ __forceinline__ double warp_sum2(double a, double b, int lane) {
 // alone): one CTA has one SM's FP64 unit, and the blocks of the first levels
 // (1300 x 64 at 64^2) then outlast the rest of their launch several times
 // over.  Clusters of 8, or of 4 where the launch has matrices enough to fill
-// the chip.  Decompositions of a 64^2 build, ms: one CTA each 39, the shared
+// the chip (id_cluster).  Decompositions of a 64^2 build, ms: one CTA each 39, the shared
 // reductions 36, clusters of 8 from 12288 / 3072 / 1024 entries on 24 / 18 / 16; a whole build at
 // 256^2: clusters of 8 2.12 s, of 4 2.06 s.
 constexpr long long ID_BIG = 1024;
@@ -292,16 +292,43 @@ __global__ void emit_v_kernel(const int* __restrict__ M, const int* __restrict__
   }
 }
 
+// CTAs a matrix.  Unequal matrices (a build's levels: a few outlast the rest):
+// 8, or 4 past 512 matrices.  Nearly equal ones: one CTA keeps its SM's FP64
+// unit busy, so what counts is how evenly the CTAs fill the chip, and what a
+// cluster of 2, 4 or 8 loses to its barriers (5, 25, 35 %).  Measured, 400 x 64
+// of rank 20, us with 1 / 2 / 4 / 8: 40 matrices 1992 / 1183 / 1079 / 892, 110
+// 1997 / 1936 / 1552 / 1829, 228 3671 / 2885 / 3438 / 3495, 304 3681 / 3816 / 4390
+// / 4503, 700 9047 / 9271 / 9204 / 9977.
+static int id_cluster(int count, const IdSizes& sizes) {
+  if (sizes.work < 0.8 * count * sizes.max_work) return count <= 512 ? 8 : 4;
+  int dev = 0, nsm = 0;
+  HB_CUDA(cudaGetDevice(&dev));
+  HB_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  const double loss[4] = {1.0, 1.05, 1.25, 1.35};
+  int best = 1;
+  double cost = 0.0;
+  for (int k = 0; k < 4; ++k) {
+    const long long per = 1 << k, waves = (count * per + nsm - 1) / nsm;
+    const double c = (double)waves / (double)per * loss[k];
+    if (k == 0 || c < cost) {
+      cost = c;
+      best = (int)per;
+    }
+  }
+  return best;
+}
+
 void id_batch(int count, const int* d_m, const int* d_n, const long long* d_aoff, double2* d_A, double eps,
-              int* d_rank, int* d_perm, const long long* d_soff, int max_n, long long max_mn, cudaStream_t st) {
+              int* d_rank, int* d_perm, const long long* d_soff, const IdSizes& sizes, cudaStream_t st) {
   if (count == 0) return;
   // clusters only where a matrix takes one and their second norm buffer fits
   const size_t col = sizeof(double) + sizeof(double2) + sizeof(int);
-  const bool cl = max_mn >= ID_BIG && (col + sizeof(double)) * (size_t)max_n <= (200u << 10);
-  const size_t sm = std::max<size_t>((size_t)max_n * (col + (cl ? sizeof(double) : 0)), 1);
+  const int cs = sizes.max_mn >= ID_BIG && (col + sizeof(double)) * (size_t)sizes.max_n <= (200u << 10)
+                     ? id_cluster(count, sizes) : 1;
+  const bool cl = cs > 1;
+  const size_t sm = std::max<size_t>((size_t)sizes.max_n * (col + (cl ? sizeof(double) : 0)), 1);
   if (cl) HB_CUDA(cudaFuncSetAttribute(id_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   else HB_CUDA(cudaFuncSetAttribute(id_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  const int cs = !cl ? 1 : count <= 512 ? 8 : 4;
   const int most = (1 << 30) / cs;
   for (int b0 = 0; b0 < count; b0 += most) {
     const int cnt = std::min(count - b0, most);
@@ -441,12 +468,10 @@ void id_batch_noalloc(int count, const int* m, const int* n, const long long* a_
   if (count > ID_NOALLOC_MAX)
     throw arg_error("hb_id_batch_noalloc: count=%d exceeds the static scratch limit of %d matrices", count,
                     ID_NOALLOC_MAX);
-  int max_n = 1;
-  long long max_mn = 0;
+  IdSizes sizes;
   for (int b = 0; b < count; ++b) {
     if (m[b] < 1 || n[b] < 1) throw arg_error("matrix %d has an empty dimension", b);
-    max_n = std::max(max_n, n[b]);
-    max_mn = std::max(max_mn, (long long)m[b] * n[b]);
+    sizes.add(m[b], n[b]);
   }
   if (count == 0) return;
   std::lock_guard<std::mutex> lk(g_noalloc_mu);
@@ -470,7 +495,7 @@ void id_batch_noalloc(int count, const int* m, const int* n, const long long* a_
   HB_CUDA(cudaMemcpyAsync(d_a, h_a, sizeof(long long) * count, cudaMemcpyHostToDevice, st));
   noalloc_offsets_kernel<<<1, 1024, 0, st>>>(d_n, count, d_s, d_v);
   HB_CHECK_LAUNCH();
-  id_batch(count, d_m, d_n, d_a, A, eps, rank, skel, d_s, max_n, max_mn, st);
+  id_batch(count, d_m, d_n, d_a, A, eps, rank, skel, d_s, sizes, st);
   emit_v(count, d_m, d_n, d_a, A, rank, skel, d_s, d_v, 0, V, nullptr, st);
 }
 

@@ -187,16 +187,14 @@ void id_level(const hb_ctx* c, double2* d_A, const std::vector<int>& m, const st
   const int cnt = (int)m.size();
   std::vector<long long> soff((size_t)cnt);
   long long sacc = 0;
-  int max_n = 0;
-  long long max_mn = 0;
+  IdSizes sizes;
   for (int b = 0; b < cnt; ++b) {
-    max_mn = std::max(max_mn, (long long)m[(size_t)b] * n[(size_t)b]);
+    sizes.add(m[(size_t)b], n[(size_t)b]);
     soff[(size_t)b] = sacc;
     sacc += n[(size_t)b];
-    max_n = std::max(max_n, n[(size_t)b]);
   }
   // the ID kernel keeps 28 bytes per column of a block in shared memory
-  if (max_n > 8000)
+  if (sizes.max_n > 8000)
     throw Error{HB_ERR_UNSUPPORTED,
                 "a curve butterfly block with more than 8000 columns (too few tree levels: more segments or a "
                 "smaller leaf_s)"};
@@ -208,7 +206,7 @@ void id_level(const hb_ctx* c, double2* d_A, const std::vector<int>& m, const st
   to_dev(d_s, soff);
   d_rank.p = dev_alloc<int>((size_t)cnt);
   d_perm.p = dev_alloc<int>((size_t)sacc);
-  id_batch(cnt, d_m.p, d_n.p, d_a.p, d_A, c->opt.eps, d_rank.p, d_perm.p, d_s.p, max_n, max_mn, 0);
+  id_batch(cnt, d_m.p, d_n.p, d_a.p, d_A, c->opt.eps, d_rank.p, d_perm.p, d_s.p, sizes, 0);
   HB_CUDA(cudaDeviceSynchronize());
   rank.assign((size_t)cnt, 0);
   std::vector<int> perm((size_t)sacc);

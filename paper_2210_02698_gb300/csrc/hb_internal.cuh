@@ -393,9 +393,21 @@ void eval_entries(hb_ctx* c, const long long* rows, int m, const long long* cols
 void add_block(BlockBatchHost& B, const hb_ctx* c, const long long* rows, long long m,
                const long long* cols, long long n, long long out_off);
 void run_blocks(hb_ctx* c, BlockBatchHost& B, double2* d_out, cudaStream_t st);
+// of the matrices of an id_batch: the largest n and m n, the sum and the largest of m n min(m, n)
+struct IdSizes {
+  int max_n = 1;
+  long long max_mn = 0;
+  double work = 0.0, max_work = 0.0;
+  void add(int m, int n) {
+    const double w = (double)m * n * std::min(m, n);
+    max_n = std::max(max_n, n);
+    max_mn = std::max(max_mn, (long long)m * n);
+    work += w;
+    max_work = std::max(max_work, w);
+  }
+};
 void id_batch(int count, const int* d_m, const int* d_n, const long long* d_aoff, double2* d_A,
-              double eps, int* d_rank, int* d_perm, const long long* d_soff, int max_n, long long max_mn,
-              cudaStream_t st);   // max_n, max_mn: the largest n and m n of the matrices
+              double eps, int* d_rank, int* d_perm, const long long* d_soff, const IdSizes& sizes, cudaStream_t st);
 void emit_v(int count, const int* d_m, const int* d_n, const long long* d_aoff, const double2* d_A,
             const int* d_rank, const int* d_perm, const long long* d_soff, const long long* d_voff,
             int ld_is_rank, double2* V64, float2* V32, cudaStream_t st);
