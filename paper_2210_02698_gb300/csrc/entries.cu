@@ -181,7 +181,7 @@ static void hankel_rows(hb_ctx* c, int need) {
   c->hank_old.reserve(c->hank_old.size() + 1);
   double2* d = dev_alloc<double2>((size_t)rows * HT_ROW);
   hankel_table_kernel<<<(rows + 31) / 32, 32>>>(d, rows);   // one warp an SM: a serial FP64 chain a row
-  if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
+  if (cudaGetLastError() != cudaSuccess) {
     dev_free(d);
     throw Error{HB_ERR_CUDA, "the Hankel expansions could not be computed"};
   }
