@@ -59,7 +59,7 @@ __global__ void scatter_kernel(const double2* __restrict__ y, const long long* _
 // are kept in input order).  It scales X per right-hand side, splits it into
 // digit fragments in shared memory once, TASK_KC k-steps at a time, and every
 // warp streams its unit's F from global memory into registers, one k-step
-// ahead, scaling it per output row (P.d_fe, found when the plan is made) and
+// ahead, scaling it per output row (unit.fe, found when the plan is made) and
 // splitting it there: a row far below the others of its task keeps its bits,
 // as in a plain FP64 sum.  Long sums (ks k-steps) are dealt over kw(ks) warps and
 // the integer sums added.  A unit's sums depend on its task alone, so a
@@ -70,7 +70,7 @@ __global__ void scatter_kernel(const double2* __restrict__ y, const long long* _
 // is near 16, and the epilogue, against 1024 x 4 FP64 FMAs for 16
 // right-hand sides (2048 cycles of an SM's FP64 unit).  Measured: 192^2 x 16
 // 3.67 ms with one FP64 FMA loop per output, 1.92 with a CTA of 8 warps per
-// task, 1.30 with four warps and shared inputs; 120 x 88 adjoint x 5: 601,
+// task, 1.28 with four warps and shared inputs; 120 x 88 adjoint x 5: 601,
 // 251, 207 us (205 with one exponent a task, the same in every lane).
 constexpr int TASK_KC = 16;              // k-steps of X held at a time
 constexpr uint32_t SPLIT_IM_SIGN = 0x80000000u;
@@ -132,8 +132,7 @@ __device__ __noinline__ void task_plain(const Task* __restrict__ task, const dou
 template <bool HALF, int W>
 __global__ void __launch_bounds__(32 * W, 16 / W)
     task_kernel(const TaskItem* __restrict__ items, const TaskUnit* __restrict__ units,
-                const unsigned short* __restrict__ fexp, const Task* __restrict__ tasks, const double2* __restrict__ F,
-                double2* x, double2* y, double2* xh, int R) {
+                const Task* __restrict__ tasks, const double2* __restrict__ F, double2* x, double2* y, double2* xh, int R) {
   constexpr int NR = HALF ? 8 : 16;        // right-hand sides of the MMA rows
   constexpr int NE = HALF ? 4 : 8;         // accumulator elements per lane and digit diagonal
   constexpr int XW = HALF ? 2 : 4;         // X fragment words per lane
@@ -172,7 +171,7 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
     work = u0 + wt < item.units;
     const int at = item.unit0 + (work ? u0 + wt : 0);
     unit = units[at];
-    fe = fexp[8 * (size_t)at + g];
+    fe = units[at].fe[g];
     row = 8 * unit.tile + g;
     rok = work && row < unit.r_out;
     load_f(kp);
@@ -315,10 +314,9 @@ __global__ void __launch_bounds__(32 * W, 16 / W)
   }
 }
 
-// fe[8 u + g] = the largest exponent of row g of unit u (0 past the task's rows), one warp a unit
-__global__ void __launch_bounds__(256) unit_exponent_kernel(const TaskUnit* __restrict__ units, const Task* __restrict__ tasks,
-                                                            const double2* __restrict__ F, int n,
-                                                            unsigned short* __restrict__ fe) {
+// units[u].fe[g] = the largest exponent of row g of unit u (0 past the task's rows), one warp a unit
+__global__ void __launch_bounds__(256) unit_exponent_kernel(TaskUnit* __restrict__ units, const Task* __restrict__ tasks,
+                                                            const double2* __restrict__ F, int n) {
   const int u = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   if (u >= n) return;
   const TaskUnit unit = units[u];
@@ -335,12 +333,12 @@ __global__ void __launch_bounds__(256) unit_exponent_kernel(const TaskUnit* __re
     }
   e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
   e = max(e, __shfl_xor_sync(0xffffffffu, e, 2));
-  if (t == 0) fe[8 * (size_t)u + g] = (unsigned short)e;
+  if (t == 0) units[u].fe[g] = (unsigned short)e;
 }
 
 void task_exponents(const TaskPlan& P, const Task* d_tasks, const double2* F, cudaStream_t st) {
   if (P.units == 0) return;
-  unit_exponent_kernel<<<(unsigned)((P.units + 7) / 8), 256, 0, st>>>(P.d_units, d_tasks, F, P.units, P.d_fe);
+  unit_exponent_kernel<<<(unsigned)((P.units + 7) / 8), 256, 0, st>>>(P.d_units, d_tasks, F, P.units);
   HB_CHECK_LAUNCH();
 }
 
@@ -406,12 +404,8 @@ TaskPlan task_plan(const std::vector<Task>& tasks, const std::vector<int>& begin
   }
   P.item_begin.push_back((int)items.size());
   P.units = (int)units.size();
-  // the units and, behind them, the exponents of their rows (an allocation
-  // costs a new curve some 10 us)
-  P.d_units = reinterpret_cast<TaskUnit*>(dev_alloc<unsigned char>(units.size() * (sizeof(TaskUnit) + 8 * sizeof(unsigned short))));
-  P.d_fe = reinterpret_cast<unsigned short*>(P.d_units + units.size());
+  P.d_units = upload(units);
   try {
-    HB_CUDA(cudaMemcpyAsync(P.d_units, units.data(), units.size() * sizeof(TaskUnit), cudaMemcpyHostToDevice, 0));
     P.d_items = upload(items);
     HB_CUDA(cudaStreamSynchronize(0));   // the host arrays end here
   } catch (...) {
@@ -455,8 +449,7 @@ static void launch_tasks(const TaskPlan& P, int step, const Task* tasks, const d
   const size_t red = (size_t)(W - 1) * 32 * (HALF ? 4 : 8) * sizeof(longlong2);
   const size_t smem = P.max_ks[(size_t)step] > 12 ? std::max(frag, red) : frag;
   HB_CUDA(cudaFuncSetAttribute(task_kernel<HALF, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, 56 << 10));
-  task_kernel<HALF, W><<<n, 32 * W, smem, st>>>(P.d_items + P.item_begin[(size_t)step], P.d_units, P.d_fe, tasks, F, x, y, xh,
-                                                R);
+  task_kernel<HALF, W><<<n, 32 * W, smem, st>>>(P.d_items + P.item_begin[(size_t)step], P.d_units, tasks, F, x, y, xh, R);
   HB_CHECK_LAUNCH();
 }
 

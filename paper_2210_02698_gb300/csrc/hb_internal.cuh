@@ -133,6 +133,7 @@ struct TaskUnit {
   long long f_off[2], y_off;
   int task, tile, r_out;
   unsigned char conj_t, y_buf, accumulate, pad;
+  unsigned short fe[8];     // largest biased exponent of each factor row (task_exponents)
 };
 struct TaskItem {
   long long x_off[2];
@@ -142,7 +143,6 @@ struct TaskPlan {
   int W = 4;                       // warps per CTA
   TaskUnit* d_units = nullptr;
   TaskItem* d_items = nullptr;
-  unsigned short* d_fe = nullptr;  // behind d_units: largest biased exponent of each factor row, 8 per unit
   int units = 0;
   std::vector<int> item_begin;     // items of step s: [item_begin[s], item_begin[s + 1])
   std::vector<int> max_ks;         // k-steps of 8 inputs of a step's longest task
